@@ -60,7 +60,7 @@ typedef struct CUstream_st* hist_cuda_stream; /* the same type as cudaStream_t *
 #define HIST_BUDGET_MAX 8192  /* ... up to 32 per bin (a 32 KiB table) */
 #define HIST_THETA_MILLI_DEFAULT 450 /* Sec. III.C: critical degeneracy 40-50 % */
 
-#define HIST_FLAG_PLAIN 0u    /* the per-warp kernel (NVHist) */
+#define HIST_FLAG_PLAIN 0u    /* the plain kernel (NVHist) */
 #define HIST_FLAG_ADAPTIVE 1u /* the sub-binned kernel (AHist) */
 
 const char* hist_strerror(int code);
@@ -75,8 +75,8 @@ int hist_device_sms(void);
  * off[b] .. off[b]+k_b-1, and a pixel of value b read by warp lane l is
  * counted in slot off[b] + (l mod k_b) (sub-bins allotted to the lanes of a
  * warp cyclically, Sec. III.A).  The histogram is the per-bin sum of its
- * slots, so any valid pattern gives the exact histogram; the pattern only
- * changes speed.  Valid: log2k[b] <= 5, off[b] a multiple of k_b, the ranges
+ * slots, so any valid pattern gives the exact histogram (see hist_adaptive
+ * for how the slots are held).  Valid: log2k[b] <= 5, off[b] a multiple of k_b, the ranges
  * disjoint, used = sum k_b <= budget <= HIST_BUDGET_MAX.  776 bytes. */
 typedef struct hist_pattern {
   uint16_t off[HIST_BINS];
@@ -130,16 +130,23 @@ int degeneracy_u64(const uint64_t* d_hist, uint32_t theta_milli, hist_degeneracy
                    hist_cuda_stream s);
 
 /* --------------------------------------------------------- one-shot kernels -- */
-/* Plain per-warp kernel (NVHist, Sec. I and Table 2: one sub-histogram of 256
- * bins per warp in shared memory, merged per bin).  d_out: uint32_t[256],
- * overwritten.  n >= 2^32 -> HIST_EINVAL.  d_in may be null only if n == 0. */
+/* Plain kernel (NVHist's place, Sec. I and Table 2): privatised sub-histograms
+ * in shared memory, no pattern, merged per bin.  The sub-histograms are one
+ * per lane (32 of 256 bins, shared by the CTA's warps) rather than one per
+ * warp: the same 32 KiB, and a warp's increments fall in 32 banks whatever
+ * the pixels are (64 MiB of uniform pixels: 2.2 -> 4.6 TB/s).  The per-warp
+ * layout itself is measured by hist_ablation without a pattern.  d_out:
+ * uint32_t[256], overwritten.  n >= 2^32 -> HIST_EINVAL.  d_in may be null
+ * only if n == 0. */
 int hist_plain(const uint8_t* d_in, size_t n, uint32_t* d_out, hist_cuda_stream s);
 
-/* Adaptive kernel (AHist, Sec. III.A) with the device-resident pattern d_pat.
- * Same contract as hist_plain.  The pattern must be valid (as written by
- * binning_pattern / default_pattern, or checked with hist_pattern_check);
- * the kernel never addresses memory outside its own table whatever d_pat
- * holds, but an invalid pattern gives an unspecified histogram. */
+/* Adaptive kernel (AHist, Sec. III.A) for the device-resident pattern d_pat.
+ * Same contract as hist_plain.  The counts are those of the pattern's slots
+ * summed per bin, which every valid pattern gives; they are held in the
+ * lane-private table, which splits each slot by lane (the words of bin b
+ * that lanes l = j mod k_b count in are slot off[b] + j), so the pattern
+ * needs no lookup per pixel.  hist_ablation counts in the pattern's own
+ * slots. */
 int hist_adaptive(const uint8_t* d_in, size_t n, const hist_pattern* d_pat, uint32_t* d_out,
                   hist_cuda_stream s);
 
@@ -515,8 +522,9 @@ int hist_stream_change(hist_stream* st, uint32_t tau_milli, hist_change_result* 
  *   2  + clear the shared sub-histogram;
  *   3  + read the binning pattern and compute every pixel's sub-bin address;
  *   4  + the shared-memory increments;
- *   5  + sum the sub-bins per bin and write the histogram (= hist_adaptive,
- *        or hist_plain without a pattern);
+ *   5  + sum the sub-bins per bin and write the histogram: the paper's
+ *        complete kernels, AHist in the pattern's own slots, or NVHist (one
+ *        table per warp) without a pattern;
  *   6  stage 5 with warp-aggregated increments (the lanes holding one value
  *        elect a leader, which adds the group's size);
  *   7  stage 5 with the input staged through shared memory by 1-D bulk

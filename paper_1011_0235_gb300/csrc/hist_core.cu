@@ -14,45 +14,112 @@ namespace {
 
 thread_local int g_last_cuda_error = 0;
 
-// One-shot histogram of [in, in+n) into out (zeroed beforehand by the caller).
-// pat == nullptr selects the per-warp (PLAIN) layout.  One CTA of 1024
-// threads per SM with four loads in flight per thread: as many bytes in
-// flight as two CTAs with two loads each, without two CTAs on one SM
-// finishing their ranges apart (1 GiB, full table: 6.05 -> 6.25 TB/s
-// uniform, 6.14 -> 6.41 TB/s N(128, 8); per-warp tables unchanged).
-__global__ void __launch_bounds__(kThreads, 1)
-    oneshot_kernel(const uint8_t* __restrict__ in, size_t n, const hist_pattern* __restrict__ pat,
-                   uint32_t* __restrict__ out) {
-  extern __shared__ __align__(16) uint32_t smem[];
-  uint32_t* table = smem;
-  uint32_t* lut = smem + kTableWords;
-  __shared__ CtaShared cs;
+// ------------------------------------------------------ one-shot kernels --
+//
+// hist_plain and hist_adaptive count in the lane-private table
+// (hist_device.cuh), which refines every pattern: one code path, bound by the
+// HBM read on a long input and by launch and latency on a short one.
 
-  zero_table(table);
-  if (pat) {
-    const uint32_t* src = reinterpret_cast<const uint32_t*>(pat);
-    uint32_t* dst = reinterpret_cast<uint32_t*>(&cs.pat);
-    for (int i = threadIdx.x; i < (int)(sizeof(hist_pattern) / 4); i += kThreads) dst[i] = src[i];
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ uint32_t cluster_size() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %cluster_nctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// The word at shared address `a` of CTA `rank` of the cluster.
+__device__ __forceinline__ uint32_t cluster_ld(uint32_t a, uint32_t rank) {
+  uint32_t r, v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+  asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(r) : "memory");
+  return v;
+}
+
+// A short input: one cluster of 1, 2, 4, 8 or 16 CTAs counts it, each CTA an
+// equal part, and the CTAs sum each other's tables through distributed
+// shared memory: no cleared output, no global atomics, one launch.  Bound by
+// latency (launch, one round of loads, two barriers of the cluster): 1 MiB of
+// uniform pixels 10.3 -> 8.2 us a call in a row (a clearing memset and 16
+// CTAs of per-warp tables before), 5.9 us of it on the GPU; 4 KiB 8.0 -> 3.6
+// us on the GPU.
+__global__ void __launch_bounds__(kThreads, 1)
+    oneshot_cluster_kernel(const uint8_t* __restrict__ in, size_t n, uint32_t* __restrict__ out) {
+  extern __shared__ __align__(16) uint32_t smem[];
+  __shared__ uint32_t res[HIST_BINS];
+  const int t = threadIdx.x;
+  const uint32_t C = cluster_size(), rank = cluster_rank();
+  const Split sp = split_bytes(in, n);
+  const uint4* body = reinterpret_cast<const uint4*>(in + sp.head);
+  const size_t begin = part_begin(sp.nvec, C, rank), end = part_begin(sp.nvec, C, rank + 1);
+  uint4 v[4];
+  lane_load<4>(v, body, begin + t, end, kThreads);
+  zero_table(smem);
+  __syncthreads();
+  lane_count<4>(v, body, begin + t, end, kThreads, smem_addr(smem) + ((t & 31) << 2));
+  __syncthreads();
+  lane_reduce<kThreads, false>(smem, res, t);
+  __syncthreads();
+  if (rank == 0) count_edges_into(in, sp, res);
+  if (C == 1) {
     __syncthreads();
-    classify_pattern(cs.pat, lut, cs);
-  } else {
-    if (threadIdx.x == 0) {
-      cs.path = PATH_PLAIN;
-      cs.lk = 0;
-    }
-    __syncthreads();
+    if (t < HIST_BINS) out[t] = res[t];
+    return;
   }
+  cluster_sync();
+  // CTA r sums bins r 256 / C ..., C neighbouring lanes to a bin, one per CTA
+  if (t < HIST_BINS) {
+    const uint32_t bin = rank * (HIST_BINS / C) + t / C;
+    uint32_t sum = cluster_ld(smem_addr(res + bin), t & (C - 1));
+    for (uint32_t o = 1; o < C; o <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if ((t & (C - 1)) == 0) out[bin] = sum;
+  }
+  cluster_sync();  // no CTA leaves while another reads its sums
+}
+
+// A longer input: out is cleared by a launch of its own, which lets the
+// counting launch start at once; that one waits for it only before it adds.
+// The clearing launch itself starts when the work before it has completed,
+// so the pixels are there before either starts.
+__global__ void __launch_bounds__(HIST_BINS) oneshot_clear_kernel(uint32_t* __restrict__ out) {
+  pdl_launch_dependents();
+  out[threadIdx.x] = 0;
+}
+
+// One CTA of 1024 threads per SM with four loads in flight per thread: as
+// many bytes in flight as two CTAs with two loads each, without two CTAs on
+// one SM finishing their ranges apart.  Bound by the HBM read.  On the GPU,
+// clearing launch included: 64 MiB of uniform pixels 30.7 -> 14.7 us, 256 MiB
+// 98.4 -> 43.1 us (6.2 TB/s; per-warp tables before).
+__global__ void __launch_bounds__(kThreads, 1)
+    oneshot_kernel(const uint8_t* __restrict__ in, size_t n, uint32_t* __restrict__ out) {
+  extern __shared__ __align__(16) uint32_t smem[];
+  __shared__ uint32_t res[HIST_BINS];
+  const int t = threadIdx.x;
+  pdl_launch_dependents();
   const Split sp = split_bytes(in, n);
   const uint4* body = reinterpret_cast<const uint4*>(in + sp.head);
   const size_t begin = part_begin(sp.nvec, gridDim.x, blockIdx.x);
   const size_t end = part_begin(sp.nvec, gridDim.x, blockIdx.x + 1);
-  count_range_dispatch<4>(cs.path, cs.lk, body, begin, end, table, lut, threadIdx.x, kThreads);
-  flush_table(cs.path, cs.lk, table, cs.pat, lut, cs);
+  uint4 v[4];
+  lane_load<4>(v, body, begin + t, end, kThreads);
+  zero_table(smem);
+  __syncthreads();
+  lane_count<4>(v, body, begin + t, end, kThreads, smem_addr(smem) + ((t & 31) << 2));
+  __syncthreads();
+  lane_reduce<kThreads, false>(smem, res, t);
+  __syncthreads();
   if (blockIdx.x == 0) {
-    count_edges(in, sp, cs);
+    count_edges_into(in, sp, res);
     __syncthreads();
   }
-  if (threadIdx.x < HIST_BINS && cs.res[threadIdx.x]) atomicAdd(out + threadIdx.x, cs.res[threadIdx.x]);
+  pdl_wait();
+  if (t < HIST_BINS && res[t]) atomicAdd(out + t, res[t]);
 }
 
 // Change detection between two uint64 histograms (256 threads).
@@ -122,20 +189,65 @@ int ensure_smem_attr_bytes(const void* fn, int* done, size_t bytes) {
   return HIST_OK;
 }
 
-int oneshot(const uint8_t* d_in, size_t n, const hist_pattern* d_pat, uint32_t* d_out, cudaStream_t s) {
-  if (!d_out || (!d_in && n) || n >= ((size_t)1 << 32)) return HIST_EINVAL;
-  cudaError_t e = cudaMemsetAsync(d_out, 0, HIST_BINS * sizeof(uint32_t), s);
+int ensure_wide_cluster(const void* fn, int* done) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return cuda_fail(e);
-  if (n == 0) return HIST_OK;
-  static int attr_done[kMaxDevices];
-  int rc = ensure_smem_attr((const void*)oneshot_kernel, attr_done);
-  if (rc) return rc;
-  const Split sp = split_bytes(d_in, n);
-  const size_t want = (sp.nvec + 4 * kThreads - 1) / (4 * kThreads);
-  const size_t cap = 1 * (size_t)sm_count();
-  const int grid = (int)(want < 1 ? 1 : (want > cap ? cap : want));
-  oneshot_kernel<<<grid, kThreads, kSmemBytes, s>>>(d_in, n, d_pat, d_out);
+  if (dev >= 0 && dev < kMaxDevices && done[dev]) return HIST_OK;
+  e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e != cudaSuccess) return cuda_fail(e);
+  if (dev >= 0 && dev < kMaxDevices) done[dev] = 1;
+  return HIST_OK;
+}
+
+// Bytes of one load per thread of a CTA: a cluster has a CTA for each, up to
+// 16.
+constexpr size_t kClusterStep = (size_t)kThreads * 16;
+// Longest input of the cluster path: one round of four loads per thread of 16
+// CTAs.  Calls in a row on 1 MiB (the second launch costs the host 2.5 us):
+// 8.2 us against 9.7 with the clearing and the counting launch; replayed from
+// a graph 5.9 against 5.65, and 7.7 against 5.8 at 2 MiB, where 16 SMs are
+// too few.
+constexpr size_t kClusterMax = 16 * 4 * kClusterStep;
+constexpr size_t kOneshotSmem = (size_t)kTableWords * 4;
+
+int oneshot(const uint8_t* d_in, size_t n, uint32_t* d_out, cudaStream_t s) {
+  if (!d_out || (!d_in && n) || n >= ((size_t)1 << 32)) return HIST_EINVAL;
+  cudaError_t e;
+  if (n == 0) {
+    e = cudaMemsetAsync(d_out, 0, HIST_BINS * sizeof(uint32_t), s);
+    return e == cudaSuccess ? HIST_OK : cuda_fail(e);
+  }
+  cudaLaunchConfig_t lc = {};
+  cudaLaunchAttribute at[1];
+  lc.blockDim = dim3(kThreads);
+  lc.dynamicSmemBytes = kOneshotSmem;
+  lc.stream = s;
+  lc.attrs = at;
+  if (n <= kClusterMax) {
+    unsigned c = 1;
+    while (c < 16 && c * kClusterStep < n) c <<= 1;
+    static int wide_done[kMaxDevices];
+    if (c > 8) {
+      const int rc = ensure_wide_cluster((const void*)oneshot_cluster_kernel, wide_done);
+      if (rc) return rc;
+    }
+    lc.gridDim = dim3(c);
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = c;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    lc.numAttrs = c > 1 ? 1 : 0;
+    e = cudaLaunchKernelEx(&lc, oneshot_cluster_kernel, d_in, n, d_out);
+    return e == cudaSuccess ? HIST_OK : cuda_fail(e);
+  }
+  oneshot_clear_kernel<<<1, HIST_BINS, 0, s>>>(d_out);
   e = cudaGetLastError();
+  if (e != cudaSuccess) return cuda_fail(e);
+  lc.gridDim = dim3((unsigned)sm_count());
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  lc.numAttrs = 1;
+  e = cudaLaunchKernelEx(&lc, oneshot_kernel, d_in, n, d_out);
   return e == cudaSuccess ? HIST_OK : cuda_fail(e);
 }
 
@@ -184,13 +296,13 @@ int hist_pattern_check(const hist_pattern* p) {
 }
 
 int hist_plain(const uint8_t* d_in, size_t n, uint32_t* d_out, hist_cuda_stream s) {
-  return oneshot(d_in, n, nullptr, d_out, (cudaStream_t)s);
+  return oneshot(d_in, n, d_out, (cudaStream_t)s);
 }
 
 int hist_adaptive(const uint8_t* d_in, size_t n, const hist_pattern* d_pat, uint32_t* d_out,
                   hist_cuda_stream s) {
   if (!d_pat) return HIST_EINVAL;
-  return oneshot(d_in, n, d_pat, d_out, (cudaStream_t)s);
+  return oneshot(d_in, n, d_out, (cudaStream_t)s);
 }
 
 int binning_pattern(const uint32_t* d_prev_hist, uint32_t budget, hist_pattern* d_pat, hist_cuda_stream s) {

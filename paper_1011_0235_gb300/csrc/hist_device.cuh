@@ -229,6 +229,64 @@ static __device__ __noinline__ void count_call4(int path, int lk, const uint4* p
   count_range_dispatch<4>(path, lk, p, begin, end, table, lut, threadIdx.x, kThreads);
 }
 
+// ------------------------------------------------- the lane-private table --
+//
+// The table of k = 32 sub-bins per bin: bin v of lane l at word 32 v + l, so
+// a warp's 32 increments fall in 32 banks whatever the pixels are (one
+// shared-memory wavefront per 32 pixels; one table per warp takes 3.5 on
+// uniform pixels, a 960-slot pattern about 3.6 and a lookup besides).  It
+// refines every valid pattern: the lanes that a pattern lets share a slot
+// have words of their own, summed when the table is reduced, so the counts
+// are those of the pattern's slots.
+
+// Load this thread's next U vectors of [i, end): i, i + nthr, ...
+template <int U>
+__device__ __forceinline__ void lane_load(uint4 (&v)[U], const uint4* __restrict__ p, size_t i, size_t end,
+                                          int nthr) {
+#pragma unroll
+  for (int u = 0; u < U; ++u)
+    if (i + (size_t)u * nthr < end) v[u] = ldg_stream(p + i + (size_t)u * nthr);
+}
+
+// Count this thread's vectors of [i, end) -- i, i + nthr, ... -- whose first U
+// are loaded in v (lane_load), keeping the next U in flight while it counts.
+template <int U>
+__device__ __forceinline__ void lane_count(uint4 (&v)[U], const uint4* __restrict__ p, size_t i, size_t end, int nthr,
+                                           uint32_t base) {
+  const LaneOrder o = {0, 0};  // the natural order: every lane has its own bank
+  while (i < end) {
+    const size_t next = i + (size_t)U * nthr;
+    uint4 w[U];
+    lane_load<U>(w, p, next, end, nthr);
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (i + (size_t)u * nthr < end) count_vec<PATH_SHIFT, 5>(v[u], base, 0, 0, o);
+#pragma unroll
+    for (int u = 0; u < U; ++u) v[u] = w[u];
+    i = next;
+  }
+}
+
+// The per-bin sums of a lane-private table into res[0..255], by NTHR threads
+// (t: 0 .. NTHR - 1), and with CLEAR the table set to zero.  Four threads
+// take a row, each 8 words of it as two 16-byte reads; the rows of odd index
+// take them the other way round, so that the 8 lanes of a 128-byte wavefront
+// (two rows) read 32 banks.  The caller's barriers stand before and after.
+template <int NTHR, bool CLEAR>
+__device__ __forceinline__ void lane_reduce(uint32_t* table, uint32_t* res, int t) {
+#pragma unroll
+  for (int r0 = 0; r0 < HIST_BINS; r0 += NTHR / 4) {
+    const int row = r0 + (t >> 2), q = t & 3, s = row & 1;
+    uint4* a = reinterpret_cast<uint4*>(table + row * 32 + q * 8);
+    const uint4 x = a[s], y = a[s ^ 1];
+    if (CLEAR) a[s] = a[s ^ 1] = make_uint4(0, 0, 0, 0);
+    uint32_t sum = x.x + x.y + x.z + x.w + y.x + y.y + y.z + y.w;
+    sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+    sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+    if (q == 0) res[row] = sum;
+  }
+}
+
 __device__ __forceinline__ void zero_table(uint32_t* table) {
   uint4* t4 = reinterpret_cast<uint4*>(table);
   for (int i = threadIdx.x; i < kTableWords / 4; i += kThreads) t4[i] = make_uint4(0, 0, 0, 0);

@@ -17,7 +17,10 @@ int sm_count();
 // Opt a kernel into the library's dynamic shared-memory size on this device.
 int ensure_smem_attr(const void* fn, int* done);
 int ensure_smem_attr_bytes(const void* fn, int* done, size_t bytes);
+// Allow a kernel clusters of more than 8 CTAs on this device (once per kernel
+// and device; `done` as above).
+int ensure_wide_cluster(const void* fn, int* done);
 // The one-shot histogram (hist_plain / hist_adaptive).
-int oneshot(const uint8_t* d_in, size_t n, const hist_pattern* d_pat, uint32_t* d_out, cudaStream_t s);
+int oneshot(const uint8_t* d_in, size_t n, uint32_t* d_out, cudaStream_t s);
 
 }  // namespace histlib
