@@ -159,19 +159,14 @@ int hist_adaptive(const uint8_t* d_in, size_t n, const hist_pattern* d_pat, uint
  * runs the plain kernel with default_pattern(budget).
  *
  * The chunks of a push are counted back to back by one launch (one per
- * 1024 chunks), and each
- * chunk's exact switch and pattern are computed from its histogram in its
- * epilogue.  A chunk's counts do not depend on the kernel or the layout that
- * count it.  Where those depend on the previous chunk's histogram -- the
- * switch in AUTO mode, the pattern of the adaptive kernel below
- * HIST_BUDGET_MAX -- a launch before the count predicts them from a
- * 4096-pixel sample of the previous chunk; in AUTO mode a chunk whose
- * predicted kernel is not the one the switch chose is counted again with
- * that kernel (hist_stream_state.recounted), while a predicted layout that
- * differs from the exact pattern only costs speed.  At HIST_BUDGET_MAX the
- * layouts are known in advance (the rule gives the full table after every
- * non-empty chunk and the default pattern after an empty one) and are
- * checked against the exact patterns (status bit 8 otherwise). */
+ * 1024 chunks), and each chunk's exact switch and pattern are computed from
+ * its histogram in its epilogue.  A chunk's counts do not depend on the
+ * kernel or the pattern that count it: both kernels count in the lane-private
+ * table (see hist_adaptive).  In AUTO mode the launch also takes a
+ * 4096-pixel sample of every chunk but the push's last (of every chunk with a
+ * moving window) and counts the chunks whose sample gives another switch
+ * than the whole chunk (hist_stream_state.recounted): how often a switch
+ * predicted from a sample would have been wrong. */
 #define HIST_MODE_AUTO 0u     /* kernel chosen by the degeneracy switch */
 #define HIST_MODE_PLAIN 1u    /* always the plain kernel (pattern still refreshed) */
 #define HIST_MODE_ADAPTIVE 2u /* always the adaptive kernel */
@@ -192,22 +187,17 @@ int hist_adaptive(const uint8_t* d_in, size_t n, const hist_pattern* d_pat, uint
  * push's counting launch may then begin reading its chunks while the work
  * before it on `s` (normally the stream's previous push) is still running,
  * so consecutive pushes overlap on the device.  Without the flag (default)
- * the counting launch still starts early and clears its tables, but reads
- * no chunk byte before the work before it on `s` has completed, so a chunk
- * written by the kernel just before the push -- even one that lets its
- * dependents start early -- is read whole.  The one-launch paths (PLAIN,
- * or ADAPTIVE at HIST_BUDGET_MAX, with a window of one chunk) overlap the
- * counting itself; an AUTO push (prediction, count, recount, chained the
- * same way) overlaps only its prediction's sampling with the work before
- * it, since the count needs the prediction; the other paths run after the
- * work before them. */
+ * the counting launch still starts early, clears its tables and reads its
+ * range, but reads no chunk byte before the work before it on `s` has
+ * completed, so a chunk written by the kernel just before the push -- even
+ * one that lets its dependents start early -- is read whole. */
 #define HIST_OVERLAP_PUSHES 1u
 
 typedef struct hist_config {
   uint32_t budget;      /* sub-bin table slots, HIST_BUDGET_MIN..MAX (default MAX) */
   uint32_t theta_milli; /* critical degeneracy per mille, 0..1000 (default 450) */
   uint32_t mode;        /* HIST_MODE_* (default AUTO) */
-  uint32_t grid;        /* CTAs of a push's counting launch; 0 = every CTA that can be resident */
+  uint32_t grid;        /* most CTAs of a push's counting launch; 0 = every CTA that can be resident */
   uint32_t window;      /* chunks in the moving window, 1..HIST_WINDOW_MAX (default 1) */
   uint32_t flags;       /* HIST_OVERLAP_PUSHES or 0 (default 0) */
   uint32_t reserved[2]; /* zero */
@@ -309,12 +299,12 @@ typedef struct hist_stream_state {
   uint64_t chunks;              /* chunks completed */
   uint32_t flag;                /* switch from the last chunk (next kernel in AUTO) */
   uint32_t last_kernel;         /* kernel the last chunk ran */
-  uint32_t status;              /* 0, or device-side error bits: 4 = a bounded wait
-                                   ran out, 8 = a chunk's layout differed from the
-                                   pattern rule (never expected) */
-  uint32_t recounted;           /* AUTO streams: chunks counted a second time
-                                   because their kernel was predicted from a
-                                   sample that misjudged the chunk before */
+  uint32_t status;            /* 0, or device-side error bits: 4 = a bounded wait
+                                   ran out */
+  uint32_t recounted;         /* AUTO streams: chunks whose kernel a sample of the
+                                   chunk before would have chosen wrongly (counted a
+                                   second time while the kernels had tables of their
+                                   own) */
   uint32_t reserved[6];
 } hist_stream_state;
 

@@ -56,12 +56,13 @@ __global__ void __launch_bounds__(kThreads, 1)
   const uint32_t C = cluster_size(), rank = cluster_rank();
   const Split sp = split_bytes(in, n);
   const uint4* body = reinterpret_cast<const uint4*>(in + sp.head);
-  const size_t begin = part_begin(sp.nvec, C, rank), end = part_begin(sp.nvec, C, rank + 1);
-  uint4 v[4];
-  lane_load<4>(v, body, begin + t, end, kThreads);
+  const uint32_t begin = (uint32_t)part_begin(sp.nvec, C, rank), end = (uint32_t)part_begin(sp.nvec, C, rank + 1);
+  uint4 v[kLaneLoads];
+  const LaneRange r = lane_range(body, begin, end, t);
+  lane_load<kLaneLoads, kThreads>(v, r);
   zero_table(smem);
   __syncthreads();
-  lane_count<4>(v, body, begin + t, end, kThreads, smem_addr(smem) + ((t & 31) << 2));
+  lane_count<kLaneLoads, kThreads>(v, r, smem_addr(smem) + ((t & 31) << 2));
   __syncthreads();
   lane_reduce<kThreads, false>(smem, res, t);
   __syncthreads();
@@ -104,13 +105,14 @@ __global__ void __launch_bounds__(kThreads, 1)
   pdl_launch_dependents();
   const Split sp = split_bytes(in, n);
   const uint4* body = reinterpret_cast<const uint4*>(in + sp.head);
-  const size_t begin = part_begin(sp.nvec, gridDim.x, blockIdx.x);
-  const size_t end = part_begin(sp.nvec, gridDim.x, blockIdx.x + 1);
-  uint4 v[4];
-  lane_load<4>(v, body, begin + t, end, kThreads);
+  const uint32_t begin = (uint32_t)part_begin(sp.nvec, gridDim.x, blockIdx.x);
+  const uint32_t end = (uint32_t)part_begin(sp.nvec, gridDim.x, blockIdx.x + 1);
+  uint4 v[kLaneLoads];
+  const LaneRange r = lane_range(body, begin, end, t);
+  lane_load<kLaneLoads, kThreads>(v, r);
   zero_table(smem);
   __syncthreads();
-  lane_count<4>(v, body, begin + t, end, kThreads, smem_addr(smem) + ((t & 31) << 2));
+  lane_count<kLaneLoads, kThreads>(v, r, smem_addr(smem) + ((t & 31) << 2));
   __syncthreads();
   lane_reduce<kThreads, false>(smem, res, t);
   __syncthreads();

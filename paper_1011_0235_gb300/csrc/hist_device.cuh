@@ -239,40 +239,73 @@ static __device__ __noinline__ void count_call4(int path, int lk, const uint4* p
 // have words of their own, summed when the table is reduced, so the counts
 // are those of the pattern's slots.
 
-// Load this thread's next U vectors of [i, end): i, i + nthr, ...
-template <int U>
-__device__ __forceinline__ void lane_load(uint4 (&v)[U], const uint4* __restrict__ p, size_t i, size_t end,
-                                          int nthr) {
-#pragma unroll
-  for (int u = 0; u < U; ++u)
-    if (i + (size_t)u * nthr < end) v[u] = ldg_stream(p + i + (size_t)u * nthr);
+constexpr int kLaneLoads = 4;  // vectors in flight per thread
+
+// A thread's vectors of a range counted by NTHR threads: q, q + NTHR, ... as
+// long as fewer than `left` vectors lie before it (left = the range's end -
+// q, 0 if q lies past it).  (An input is below 2^32 bytes, so its vectors are
+// numbered in 32 bits.)
+struct LaneRange {
+  const uint4* q;
+  uint32_t left;
+};
+// Thread t's vectors of [begin, end) of p.
+__device__ __forceinline__ LaneRange lane_range(const uint4* p, uint32_t begin, uint32_t end, int t) {
+  const uint32_t i = begin + (uint32_t)t;
+  return LaneRange{p + i, i < end ? end - i : 0u};
 }
 
-// Count this thread's vectors of [i, end) -- i, i + nthr, ... -- whose first U
-// are loaded in v (lane_load), keeping the next U in flight while it counts.
-template <int U>
-__device__ __forceinline__ void lane_count(uint4 (&v)[U], const uint4* __restrict__ p, size_t i, size_t end, int nthr,
-                                           uint32_t base) {
-  const LaneOrder o = {0, 0};  // the natural order: every lane has its own bank
-  while (i < end) {
-    const size_t next = i + (size_t)U * nthr;
-    uint4 w[U];
-    lane_load<U>(w, p, next, end, nthr);
+// Load this thread's next U vectors.
+template <int U, int NTHR>
+__device__ __forceinline__ void lane_load(uint4 (&v)[U], const LaneRange& r) {
 #pragma unroll
-    for (int u = 0; u < U; ++u)
-      if (i + (size_t)u * nthr < end) count_vec<PATH_SHIFT, 5>(v[u], base, 0, 0, o);
+  for (int u = 0; u < U; ++u)
+    if ((uint32_t)(u * NTHR) < r.left) v[u] = ldg_stream(r.q + u * NTHR);
+}
+
+// Count this thread's vectors of r, whose first U are loaded in v
+// (lane_load), keeping U loads in flight while it counts: the next ones of
+// its own, and at its end the first U of r2, the range that comes next (left
+// = 0: none), which v holds on return.  (Refilling each vector's registers as
+// soon as it is counted, with 4 to 8 vectors, put every load behind 16
+// increments in the memory queue: 64 chunks of 16 MiB 161 -> 168-172 us,
+// 1024 of 64 KiB 24 -> 32 us.)
+template <int U, int NTHR>
+__device__ __forceinline__ void lane_count(uint4 (&v)[U], LaneRange r, uint32_t base,
+                                           const LaneRange& r2 = LaneRange{nullptr, 0}) {
+  const LaneOrder o = {0, 0};  // the natural order: every lane has its own bank
+  uint4 w[U];
+  while (r.left > (uint32_t)((2 * U - 1) * NTHR)) {  // this round and the next are whole
+#pragma unroll
+    for (int u = 0; u < U; ++u) w[u] = ldg_stream(r.q + (U + u) * NTHR);
+#pragma unroll
+    for (int u = 0; u < U; ++u) count_vec<PATH_SHIFT, 5>(v[u], base, 0, 0, o);
 #pragma unroll
     for (int u = 0; u < U; ++u) v[u] = w[u];
-    i = next;
+    r.q += U * NTHR;
+    r.left -= (uint32_t)(U * NTHR);
+  }
+  for (;;) {
+    const bool more = r.left > (uint32_t)(U * NTHR);
+    const LaneRange next = {more ? r.q + U * NTHR : r2.q, more ? r.left - (uint32_t)(U * NTHR) : r2.left};
+    lane_load<U, NTHR>(w, next);
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if ((uint32_t)(u * NTHR) < r.left) count_vec<PATH_SHIFT, 5>(v[u], base, 0, 0, o);
+#pragma unroll
+    for (int u = 0; u < U; ++u) v[u] = w[u];
+    if (!more) return;
+    r = next;
   }
 }
 
-// The per-bin sums of a lane-private table into res[0..255], by NTHR threads
-// (t: 0 .. NTHR - 1), and with CLEAR the table set to zero.  Four threads
-// take a row, each 8 words of it as two 16-byte reads; the rows of odd index
-// take them the other way round, so that the 8 lanes of a 128-byte wavefront
-// (two rows) read 32 banks.  The caller's barriers stand before and after.
-template <int NTHR, bool CLEAR>
+// The per-bin sums of a lane-private table into res[0..255] (with ADD: added
+// to it), by NTHR threads (t: 0 .. NTHR - 1), and with CLEAR the table set to
+// zero.  Four threads take a row, each 8 words of it as two 16-byte reads;
+// the rows of odd index take them the other way round, so that the 8 lanes
+// of a 128-byte wavefront (two rows) read 32 banks.  The caller's barriers
+// stand before and after.
+template <int NTHR, bool CLEAR, bool ADD = false>
 __device__ __forceinline__ void lane_reduce(uint32_t* table, uint32_t* res, int t) {
 #pragma unroll
   for (int r0 = 0; r0 < HIST_BINS; r0 += NTHR / 4) {
@@ -283,8 +316,24 @@ __device__ __forceinline__ void lane_reduce(uint32_t* table, uint32_t* res, int 
     uint32_t sum = x.x + x.y + x.z + x.w + y.x + y.y + y.z + y.w;
     sum += __shfl_xor_sync(0xffffffffu, sum, 1);
     sum += __shfl_xor_sync(0xffffffffu, sum, 2);
-    if (q == 0) res[row] = sum;
+    if (q == 0) res[row] = ADD ? res[row] + sum : sum;
   }
+}
+
+// The sum of row t of a lane-private table, which is cleared: one thread per
+// row, its 16-byte words from word t mod 8 on, so that the 8 lanes of a
+// 128-byte wavefront read 32 banks.
+__device__ __forceinline__ uint32_t lane_row(uint32_t* table, int t) {
+  uint4* row = reinterpret_cast<uint4*>(table + t * 32);
+  uint32_t sum = 0;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    uint4* a = row + ((k + t) & 7);
+    const uint4 x = *a;
+    *a = make_uint4(0, 0, 0, 0);
+    sum += x.x + x.y + x.z + x.w;
+  }
+  return sum;
 }
 
 __device__ __forceinline__ void zero_table(uint32_t* table) {
@@ -483,126 +532,18 @@ __device__ __forceinline__ void count_edges(const uint8_t* a, const Split& sp, C
 
 namespace histdev {
 
-// ------------------------------------------------- single-warp epilogue --
+// -------------------------------------------------------------- epilogue --
 
-// floor(a / b) for 0 < b < 2^32 and a / b < 2^20, exactly: an FP32 estimate
-// (relative error below 2^-22, so within 1/4 of a quotient below 2^20)
-// corrected by one integer step each way.  Other operands take the integer
-// division.
-__device__ __forceinline__ unsigned long long div_floor(unsigned long long a, unsigned long long b, float rb) {
-  if (b < (1ull << 32) && a < (b << 20)) {
-    unsigned long long q = (unsigned long long)(uint32_t)((float)a * rb);
-    if (q * b > a) q -= 1;
-    else if ((q + 1) * b <= a) q += 1;
-    return q;
-  }
-  return a / b;
+// log2 of k0 = min(32, largest power of two <= want), want = 1 + floor(spare h
+// / total), without the division: want >= 2^l iff spare h >= (2^l - 1) total.
+// (spare < 2^13, h < 2^32, total < 2^40: the products are below 2^46.)
+__device__ __forceinline__ uint32_t pattern_k0(uint32_t spare, uint32_t h, unsigned long long total) {
+  const unsigned long long x = (unsigned long long)spare * h;
+  uint32_t lk = 0;
+#pragma unroll
+  for (int l = 1; l <= 5; ++l) lk += x >= total * ((1u << l) - 1u);
+  return lk;
 }
-
-// One warp computes the degeneracy (Sec. III.C) and the binning pattern (the
-// rule stated in hist.h) of the 256-bin histogram `hist`.  Lane l holds bins
-// l + 32 i, i = 0..7.  Writes P (off, log2k, budget, used) and returns the
-// degeneracy to every lane.
-template <class T>
-__device__ hist_degeneracy_result warp_epilogue(const T* hist, uint32_t budget, uint32_t theta_milli,
-                                                hist_pattern& P) {
-  const int lane = threadIdx.x & 31;
-  unsigned long long h[8];
-  unsigned long long tot = 0, mx = 0;
-  int arg = 0;
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    h[i] = (unsigned long long)hist[lane + 32 * i];
-    tot += h[i];
-    if (h[i] > mx) {  // bins of one lane rise with i: the first maximum is the lowest
-      mx = h[i];
-      arg = lane + 32 * i;
-    }
-  }
-  tot = warp_sum(tot);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const unsigned long long m2 = __shfl_xor_sync(0xffffffffu, mx, o);
-    const int a2 = __shfl_xor_sync(0xffffffffu, arg, o);
-    if (m2 > mx || (m2 == mx && a2 < arg)) {
-      mx = m2;
-      arg = a2;
-    }
-  }
-  hist_degeneracy_result r;
-  r.max = mx;
-  r.total = tot;
-  r.maxbin = mx == 0 ? 0u : (uint32_t)arg;
-  r.flag = reaches_theta(mx, tot, theta_milli) ? HIST_FLAG_ADAPTIVE : HIST_FLAG_PLAIN;
-
-  uint32_t lk[8];
-  if (tot == 0) {
-#pragma unroll
-    for (int i = 0; i < 8; ++i) lk[i] = default_lk(lane + 32 * i, budget);
-  } else {
-    const unsigned long long spare = budget - HIST_BINS;
-    const float rt = 1.0f / (float)tot;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      // spare < 2^13 and h <= tot, so the quotient is below 2^13
-      const unsigned long long want = 1ull + div_floor(spare * h[i], tot, rt);
-      const uint32_t l0 = ilog2_u64(want);
-      lk[i] = l0 > 5 ? 5 : l0;
-    }
-    uint32_t lf = 0;
-    for (uint32_t f = 1; f <= 5; ++f) {
-      unsigned long long s = 0;
-#pragma unroll
-      for (int i = 0; i < 8; ++i) s += 1ull << (lk[i] > f ? lk[i] : f);
-      s = warp_sum(s);
-      if (s <= budget) lf = f;
-    }
-#pragma unroll
-    for (int i = 0; i < 8; ++i) lk[i] = lk[i] > lf ? lk[i] : lf;
-  }
-  // layout: classes of decreasing k, bins of one class in increasing index
-  // (index lane + 32 i orders by i, then lane)
-  uint32_t cnt[6];
-#pragma unroll
-  for (int c = 0; c < 6; ++c) cnt[c] = 0;
-#pragma unroll
-  for (int i = 0; i < 8; ++i)
-#pragma unroll
-    for (int c = 0; c < 6; ++c) cnt[c] += __popc(__ballot_sync(0xffffffffu, lk[i] == (uint32_t)c));
-  uint32_t base[6];
-  uint32_t acc = 0;
-#pragma unroll
-  for (int c = 5; c >= 0; --c) {
-    base[c] = acc;
-    acc += cnt[c] << c;
-  }
-  const unsigned lt = (1u << lane) - 1u;
-  uint32_t run[6];
-#pragma unroll
-  for (int c = 0; c < 6; ++c) run[c] = 0;
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-#pragma unroll
-    for (int c = 0; c < 6; ++c) {
-      const unsigned m = __ballot_sync(0xffffffffu, lk[i] == (uint32_t)c);
-      if (lk[i] == (uint32_t)c) {
-        P.off[lane + 32 * i] = (uint16_t)(base[c] + ((run[c] + __popc(m & lt)) << c));
-        P.log2k[lane + 32 * i] = (uint8_t)c;
-      }
-      run[c] += __popc(m);
-    }
-  }
-  if (lane == 0) {
-    P.used = acc;
-    P.budget = budget;
-  }
-  __syncwarp();
-  return r;
-}
-
-}  // namespace histdev
-
-namespace histdev {
 
 // Shared scratch of block_epilogue.
 struct EpiShared {
@@ -612,28 +553,35 @@ struct EpiShared {
   uint32_t cls[8][6];   // per-warp bins of each sub-bin class
 };
 
-// Degeneracy (Sec. III.C) and binning pattern (rule in hist.h) of the 256-bin
-// histogram `hist` whose total is known to be `total`, by threads 0..255 (one
-// bin each, warp reductions in hardware); all threads of the CTA call (two
-// barriers).  Writes P; returns the degeneracy to threads 0..255.
-static __device__ __noinline__ hist_degeneracy_result block_epilogue(const uint32_t* hist, unsigned long long total,
-                                                        uint32_t budget, uint32_t theta_milli, hist_pattern& P,
-                                                        EpiShared& es) {
-  const int t = threadIdx.x, w = t >> 5, lane = t & 31;
+// The barrier of the threads that run an epilogue: the whole CTA, or a group
+// of NTHR threads on named barrier `id`.
+struct CtaBar {
+  __device__ __forceinline__ void sync() const { __syncthreads(); }
+};
+template <int NTHR>
+struct GroupBar {
+  int id;
+  __device__ __forceinline__ void sync() const { asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(NTHR) : "memory"); }
+};
+
+// Degeneracy (Sec. III.C) and binning pattern (rule in hist.h) of a 256-bin
+// histogram whose total is known to be `total`, by threads t = 0..255, which
+// hold a bin each in h (warp reductions in hardware), of those that share
+// `bar`, all of which call (two barriers).  Threads 0..255 get the degeneracy
+// and their bin's place in the pattern.
+struct BinPlace {
+  uint32_t off, lk, used;
+};
+template <class Bar>
+__device__ __forceinline__ hist_degeneracy_result block_pattern(uint32_t h, unsigned long long total,
+                                                                uint32_t budget, uint32_t theta_milli, EpiShared& es,
+                                                                int t, Bar bar, BinPlace& place) {
+  const int w = t >> 5, lane = t & 31;
   const bool act = t < HIST_BINS;
   const unsigned full = 0xffffffffu;
-  const uint32_t h = act ? hist[t] : 0u;
   uint32_t lk0 = 0;
   if (act) {
-    if (total == 0) {
-      lk0 = default_lk(t, budget);
-    } else {
-      const unsigned long long spare = budget - HIST_BINS;
-      const float rt = 1.0f / (float)total;
-      const unsigned long long want = 1ull + div_floor(spare * (unsigned long long)h, total, rt);
-      const uint32_t l0 = ilog2_u64(want);
-      lk0 = l0 > 5 ? 5 : l0;
-    }
+    lk0 = total == 0 ? default_lk(t, budget) : pattern_k0(budget - HIST_BINS, h, total);
   }
   if (w < 8) {
     const uint32_t wm = __reduce_max_sync(full, h);
@@ -648,7 +596,7 @@ static __device__ __noinline__ hist_degeneracy_result block_epilogue(const uint3
       for (int f = 0; f < 5; ++f) es.fsum[w][f] = fs[f];
     }
   }
-  __syncthreads();
+  bar.sync();
   uint32_t lk = lk0;
   hist_degeneracy_result r;
   if (act) {
@@ -684,7 +632,7 @@ static __device__ __noinline__ hist_degeneracy_result block_epilogue(const uint3
       if (lane == 0) es.cls[w][c] = __popc(m);
     }
   }
-  __syncthreads();
+  bar.sync();
   if (act) {
     uint32_t base = 0, used = 0, before = 0;
 #pragma unroll
@@ -696,14 +644,40 @@ static __device__ __noinline__ hist_degeneracy_result block_epilogue(const uint3
       used += cnt << c;
     }
     for (int i = 0; i < w; ++i) before += es.cls[i][lk];
-    P.off[t] = (uint16_t)(base + ((before + rank) << lk));
-    P.log2k[t] = (uint8_t)lk;
-    if (t == 0) {
-      P.used = used;
-      P.budget = budget;
-    }
+    place.off = base + ((before + rank) << lk);
+    place.lk = lk;
+    place.used = used;
   }
   return r;
+}
+
+// Bin t's place into pattern P (threads 0..255).
+__device__ __forceinline__ void store_place(hist_pattern& P, int t, uint32_t budget, const BinPlace& place) {
+  P.off[t] = (uint16_t)place.off;
+  P.log2k[t] = (uint8_t)place.lk;
+  if (t == 0) {
+    P.used = place.used;
+    P.budget = budget;
+  }
+}
+
+// The same with the pattern written to P.
+template <class Bar>
+static __device__ __noinline__ hist_degeneracy_result block_epilogue(const uint32_t* hist, unsigned long long total,
+                                                        uint32_t budget, uint32_t theta_milli, hist_pattern& P,
+                                                        EpiShared& es, int t, Bar bar) {
+  BinPlace place;
+  const hist_degeneracy_result r =
+      block_pattern(t < HIST_BINS ? hist[t] : 0u, total, budget, theta_milli, es, t, bar, place);
+  if (t < HIST_BINS) store_place(P, t, budget, place);
+  return r;
+}
+
+// The same by a whole CTA.
+__device__ __forceinline__ hist_degeneracy_result block_epilogue(const uint32_t* hist, unsigned long long total,
+                                                                 uint32_t budget, uint32_t theta_milli,
+                                                                 hist_pattern& P, EpiShared& es) {
+  return block_epilogue(hist, total, budget, theta_milli, P, es, (int)threadIdx.x, CtaBar());
 }
 
 }  // namespace histdev

@@ -70,3 +70,103 @@ def test_oneshot_chain_replayed_from_a_graph(n):
             assert bytes(pat.cpu().numpy()) == oracle.binning_pattern(ref, 1500).to_bytes(), k
             arg, m, t = oracle.degeneracy(ref.astype(np.uint64))
             assert hl.degeneracy_to_host(res) == (arg, m, t, oracle.switch(ref.astype(np.uint64), 450)), k
+
+
+def _sample_flag(x, addr, theta=450):
+    """The switch from a chunk's sample: 256 evenly spaced 16-byte vectors
+    from the first 16-byte boundary of its address, or the whole chunk."""
+    head = min((16 - addr % 16) % 16, x.size)
+    nvec = (x.size - head) // 16
+    if nvec >= 256:
+        v = (np.arange(256, dtype=np.int64) * nvec) // 256
+        x = x[(head + 16 * v)[:, None] + np.arange(16)[None, :]].reshape(-1)
+    return oracle.switch(oracle.hist_u32(x).astype(np.uint64), theta) if x.size else 0
+
+
+# sizes around the sample's (256 vectors after a head of up to 15 bytes), of
+# whole small chunks, and of chunks cut between CTAs
+@pytest.mark.parametrize("sizes,cuts", [
+    ([4095, 4096, 4097, 4110, 4111, 4112, 5000, 8191] * 12, [0, 1, 2, 5, 40, 96]),
+    ([65_536, 70_001, 262_144, 262_145, 17, 0, 4096, 33_333] * 10, [0, 1, 3, 30, 80]),
+    ([1_300_003, 2_000_000, 65_536, 1 << 20, 5, 900_001] * 3, [0, 2, 3, 18]),
+])
+@pytest.mark.parametrize("overlap", [False, True])
+def test_recounted_is_the_samples_misjudgements(sizes, cuts, overlap):
+    """AUTO pushes of one, two and many chunks whose largest bin is near the
+    threshold, so that a chunk's sample and the chunk itself often disagree:
+    recounted equals the disagreements of a host model of the sample (of
+    every chunk but a push's last), the outputs, patterns and switches the
+    oracle's, whichever of them runs in a group, in one CTA or in several."""
+    rng = np.random.default_rng(len(sizes) + overlap)
+    chunks = []
+    for c, n in enumerate(sizes):
+        x = rng.integers(0, 256, n).astype(np.uint8)
+        x[rng.random(n) < 0.4475 + 0.003 * rng.standard_normal()] = c % 200
+        chunks.append(x)
+    offs, pos = [], 0
+    for c, n in enumerate(sizes):
+        pos += int(rng.integers(0, 40))
+        offs.append(pos)
+        pos += n
+    buf = np.zeros(pos + 16, np.uint8)
+    for o, ch in zip(offs, chunks):
+        buf[o:o + ch.size] = ch
+    bd = dev(buf)
+    outs = torch.full((len(sizes), 256), -1, dtype=torch.int32, device="cuda")
+    st = hl.Stream(mode=hl.MODE_AUTO, overlap=overlap)
+    ref = oracle.StreamOracle(8192)
+    expect = 0
+    for lo, hi in zip(cuts[:-1], cuts[1:]):
+        st.push_many(np.uint64(bd.data_ptr()) + np.array(offs[lo:hi], dtype=np.uint64),
+                     np.array(sizes[lo:hi], dtype=np.uint64),
+                     np.array([outs[j].data_ptr() for j in range(lo, hi)], dtype=np.uint64))
+        recs = [ref.push(chunks[j]) for j in range(lo, hi)]
+        for j in range(lo, hi - 1):
+            exact = oracle.switch(oracle.hist_u32(chunks[j]).astype(np.uint64), 450)
+            expect += int(_sample_flag(chunks[j], bd.data_ptr() + offs[j]) != exact)
+        s = st.state()
+        assert bytes(s.pattern) == ref.pattern.to_bytes() and s.flag == ref.flag
+        assert s.last_kernel == recs[-1].kernel
+        assert s.recounted == expect, (lo, hi)
+    got = u32(outs.reshape(-1)).reshape(len(sizes), 256)
+    for j, ch in enumerate(chunks):
+        assert np.array_equal(got[j], oracle.hist_u32(ch)), j
+    assert np.array_equal(np.array(s.totals, np.uint64), ref.totals) and s.status == 0
+    st.close()
+
+
+def test_a_captured_push_replayed():
+    """Pushes of one and of two chunks captured into a graph and replayed over
+    new pixels: totals, the last two patterns and the switch follow the
+    replays."""
+    n = 100_001
+    xd = torch.empty(2 * n, dtype=torch.uint8, device="cuda")
+    for count in (1, 2):
+        st = hl.Stream(budget=960)
+        ref = oracle.StreamOracle(960)
+        s = torch.cuda.Stream()
+        first = [synth.host(n, synth.uniform(), SEED + 95, k) for k in range(count)]
+        with torch.cuda.stream(s):
+            def push():
+                st.push_many([xd.data_ptr() + k * n for k in range(count)], [n] * count)
+            xd[:count * n].copy_(dev(np.concatenate(first)))
+            push()
+            for x in first:
+                ref.push(x)
+            s.synchronize()
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g, stream=s):
+                push()
+            for r in range(5):
+                chunks = [synth.host(n, synth.normal(30 + 20 * r, 3 + r) if (r + k) % 2 else synth.degenerate(5, 0.7),
+                                     SEED + 96 + r, k * n) for k in range(count)]
+                xd[:count * n].copy_(dev(np.concatenate(chunks)))
+                g.replay()
+                s.synchronize()
+                for x in chunks:
+                    rec = ref.push(x)
+            t = st.state()
+        assert np.array_equal(np.array(t.totals, np.uint64), ref.totals)
+        assert bytes(t.pattern) == ref.pattern.to_bytes() and bytes(t.last_pattern) == rec.pattern.to_bytes()
+        assert t.flag == ref.flag and t.last_kernel == rec.kernel and t.chunks == ref.chunks
+        st.close()
