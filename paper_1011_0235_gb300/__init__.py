@@ -183,7 +183,7 @@ def change(acc: torch.Tensor, window: torch.Tensor, tau_milli: int = _abi.HIST_C
     tensors): a device tensor holding one hist_change_result."""
     _dev_buf(acc, 8 * BINS, "acc", 8)
     _dev_buf(window, 8 * BINS, "window", 8)
-    out = torch.zeros(2, dtype=torch.int64, device="cuda")
+    out = torch.empty(2, dtype=torch.int64, device="cuda")
     _abi.check("hist_change", lib().hist_change(acc.data_ptr(), window.data_ptr(), tau_milli, out.data_ptr(),
                                                 _stream_ptr(stream)))
     return out
@@ -345,7 +345,7 @@ class Stream:
     def change(self, tau_milli: int = _abi.HIST_CHANGE_TAU_MILLI_DEFAULT, stream=None) -> torch.Tensor:
         """Change detection between the totals and the moving window: a device
         tensor holding one hist_change_result (see change_to_host)."""
-        out = torch.zeros(2, dtype=torch.int64, device="cuda")
+        out = torch.empty(2, dtype=torch.int64, device="cuda")
         _abi.check("hist_stream_change", lib().hist_stream_change(self._h, tau_milli, out.data_ptr(),
                                                                   _stream_ptr(stream)))
         return out

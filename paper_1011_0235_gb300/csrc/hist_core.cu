@@ -124,13 +124,15 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (t < HIST_BINS && res[t]) atomicAdd(out + t, res[t]);
 }
 
-// Change detection between two uint64 histograms (256 threads).
+// Change detection between two uint64 histograms (256 threads); chained.
 __global__ void __launch_bounds__(HIST_BINS) change_kernel(const unsigned long long* __restrict__ acc,
                                                           const unsigned long long* __restrict__ win,
                                                           uint32_t tau_milli, hist_change_result* __restrict__ res) {
   __shared__ ChangeShared sh;
   const int t = threadIdx.x;
-  const hist_change_result r = change_eval(acc[t], win[t], tau_milli, sh);
+  pdl_launch_dependents();
+  pdl_wait();
+  const hist_change_result r = change_eval(__ldcg(acc + t), __ldcg(win + t), tau_milli, sh);
   if (t == 0) *res = r;
 }
 
@@ -390,10 +392,9 @@ int degeneracy(const uint32_t* d_hist, uint32_t theta_milli, hist_degeneracy_res
 int hist_change(const uint64_t* d_acc, const uint64_t* d_win, uint32_t tau_milli, hist_change_result* d_res,
                 hist_cuda_stream s) {
   if (!d_acc || !d_win || !d_res || tau_milli > 1000) return HIST_EINVAL;
-  change_kernel<<<1, HIST_BINS, 0, (cudaStream_t)s>>>(reinterpret_cast<const unsigned long long*>(d_acc),
-                                                      reinterpret_cast<const unsigned long long*>(d_win), tau_milli,
-                                                      d_res);
-  const cudaError_t e = cudaGetLastError();
+  const cudaError_t e =
+      launch_small(change_kernel, (cudaStream_t)s, reinterpret_cast<const unsigned long long*>(d_acc),
+                   reinterpret_cast<const unsigned long long*>(d_win), tau_milli, d_res);
   return e == cudaSuccess ? HIST_OK : cuda_fail(e);
 }
 

@@ -688,30 +688,23 @@ namespace histdev {
 
 // Shared scratch of change_eval.
 struct ChangeShared {
-  unsigned __int128 term[HIST_BINS];
   unsigned long long sa[8], sm[8];
+  unsigned __int128 term[8];
 };
 
 // Total-variation distance between two histograms normalised to sum 1:
-// D = sum_b |a_b SM - m_b SA| over 2 SA SM.  Threads 0..255 pass bin t of
-// each (a, m); all threads of the CTA call (three barriers).  Thread 0 gets
-// the result: the flag (1000 D >= 2 tau SA SM, exact in 128 bits while
-// SA < 2^56 and SM < 2^40), floor(10^6 D / (2 SA SM)), and whether the sums
-// were in that range.  Either histogram empty: distance 0.
+// D = sum_b |a_b SM - m_b SA| over 2 SA SM.  256 threads pass bin t of each
+// (a, m) and call (two barriers).  Thread 0 gets the result: the flag
+// (1000 D >= 2 tau SA SM, exact in 128 bits while SA < 2^56 and SM < 2^40),
+// floor(10^6 D / (2 SA SM)), and whether the sums were in that range.  Either
+// histogram empty: distance 0.
 __device__ __forceinline__ hist_change_result change_eval(unsigned long long a, unsigned long long m,
                                                           uint32_t tau_milli, ChangeShared& sh) {
   const int t = threadIdx.x, w = t >> 5, lane = t & 31;
-  if (t < HIST_BINS) {
-    unsigned long long x = a, y = m;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      x += __shfl_xor_sync(0xffffffffu, x, o);
-      y += __shfl_xor_sync(0xffffffffu, y, o);
-    }
-    if (lane == 0) {
-      sh.sa[w] = x;
-      sh.sm[w] = y;
-    }
+  const unsigned long long x = warp_sum(a), y = warp_sum(m);
+  if (lane == 0) {
+    sh.sa[w] = x;
+    sh.sm[w] = y;
   }
   __syncthreads();
   unsigned long long SA = 0, SM = 0;
@@ -720,24 +713,40 @@ __device__ __forceinline__ hist_change_result change_eval(unsigned long long a, 
     SA += sh.sa[i];
     SM += sh.sm[i];
   }
-  if (t < HIST_BINS) {
-    const unsigned __int128 p = (unsigned __int128)a * SM, q = (unsigned __int128)m * SA;
-    sh.term[t] = p > q ? p - q : q - p;
+  const unsigned __int128 p = (unsigned __int128)a * SM, q = (unsigned __int128)m * SA;
+  unsigned __int128 d = p > q ? p - q : q - p;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long lo = __shfl_xor_sync(0xffffffffu, (unsigned long long)d, o);
+    const unsigned long long hi = __shfl_xor_sync(0xffffffffu, (unsigned long long)(d >> 64), o);
+    d += ((unsigned __int128)hi << 64) | lo;
   }
+  if (lane == 0) sh.term[w] = d;
   __syncthreads();
-  for (int half = HIST_BINS / 2; half > 0; half >>= 1) {
-    if (t < half) sh.term[t] += sh.term[t + half];
-    __syncthreads();
-  }
   hist_change_result r;
   r.flag = 0;
   r.in_range = (SA < (1ull << 56) && SM < (1ull << 40)) ? 1u : 0u;
   r.dist_ppm = 0;
   if (t == 0 && SA != 0 && SM != 0) {
-    const unsigned __int128 D = sh.term[0];
-    const unsigned __int128 den = (unsigned __int128)SA * SM * 2u;
+    unsigned __int128 D = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) D += sh.term[i];
+    const unsigned __int128 den = (unsigned __int128)SA * SM * 2u, num = D * 1000000u;
     r.flag = (unsigned __int128)1000u * D >= den * tau_milli ? 1u : 0u;
-    r.dist_ppm = (unsigned long long)((D * 1000000u) / den);
+    // the quotient is at most 10^6: in the exact range an FP64 estimate is
+    // within one of it, and one exact step each way settles it
+    if (r.in_range) {
+      const double num_d = (double)(unsigned long long)(num >> 64) * 18446744073709551616.0 +
+                           (double)(unsigned long long)num;
+      const double den_d = (double)(unsigned long long)(den >> 64) * 18446744073709551616.0 +
+                           (double)(unsigned long long)den;
+      unsigned long long k = (unsigned long long)(num_d / den_d);
+      if (den * k > num) k -= 1;
+      else if (den * (k + 1) <= num) k += 1;
+      r.dist_ppm = k;
+    } else {
+      r.dist_ppm = (unsigned long long)(num / den);
+    }
   } else if (t == 0) {
     r.flag = tau_milli == 0 ? 1u : 0u;  // distance 0 reaches only a threshold of 0
   }

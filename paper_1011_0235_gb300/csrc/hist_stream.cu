@@ -865,13 +865,20 @@ __global__ void __launch_bounds__(kThreads, 1) batch_flat_kernel(const __grid_co
 // of the histograms of chunks g-W+1 .. g (chunks before number 0 count as
 // empty; a resumed stream restarts at 0).  The histograms of the last
 // kChunkRing chunks stay in rings, so each chunk's window is summed on its
-// own: one CTA per chunk of the batch, bin b in thread b, W loads per thread
-// with eight in flight, then the window's largest bin and total.
+// own: one CTA per chunk of the batch, thread b + 256 q taking bin b of
+// every fourth run of eight chunks, so that a window of 32 is one round of
+// loads.  Bound by L2 latency: a push of 128 x 1 MiB at W = 32 with its
+// totals, window and change queries takes 40.8 us, 56.0 with 256 threads (four
+// rounds) and the queries each waiting for the launch before it to end.
+constexpr int kWindowThreads = 4 * HIST_BINS;
+constexpr uint32_t kWindowRun = 8;                              // chunks per thread and round
+constexpr uint32_t kWindowRound = kWindowRun * kWindowThreads / HIST_BINS;  // chunks per round
 
-// Largest bin and total of a 256-bin window held one bin per thread (all
-// threads call; two barriers); returned to every thread.
+// Largest bin and total of a 256-bin window held one bin per thread (256
+// threads on barrier 1 call; two barriers); returned to every thread.
 template <class T>
 __device__ __forceinline__ void window_max_sum(T v, T* smax, T* ssum, T& mx, T& sm) {
+  const GroupBar<HIST_BINS> bar = {1};
   const int b = threadIdx.x, w = b >> 5;
   T m = v, s = v;
 #pragma unroll
@@ -884,7 +891,7 @@ __device__ __forceinline__ void window_max_sum(T v, T* smax, T* ssum, T& mx, T& 
     smax[w] = m;
     ssum[w] = s;
   }
-  __syncthreads();
+  bar.sync();
   mx = smax[0];
   sm = ssum[0];
 #pragma unroll
@@ -892,55 +899,66 @@ __device__ __forceinline__ void window_max_sum(T v, T* smax, T* ssum, T& mx, T& 
     mx = smax[i] > mx ? smax[i] : mx;
     sm += ssum[i];
   }
-  __syncthreads();
+  bar.sync();
 }
 
 // The window switches of a launch's chunks, one CTA per chunk, chained after
-// the counting launch.  The CTA of the last chunk
-// writes the window after it and the stream's switch; the one of the chunk
-// before it the kernel the last chunk ran.  In AUTO mode each CTA but the
-// last also takes the same window's switch from the samples, in FP32 (FP64 is
-// slow on this part and the samples are estimates), and counts a chunk whose
-// two switches differ.
-__global__ void __launch_bounds__(HIST_BINS) window_flat_kernel(const PushHead a) {
+// the counting launch.  The CTA of the last chunk writes the window after it
+// and the stream's switch; the one of the chunk before it the kernel the last
+// chunk ran.  In AUTO mode each CTA but the last also takes the same window's
+// switch from the samples, in FP32 and in the chunks' order (FP64 is slow on
+// this part and the samples are estimates), and counts a chunk whose two
+// switches differ.
+__global__ void __launch_bounds__(kWindowThreads) window_flat_kernel(const PushHead a) {
+  __shared__ unsigned long long part[kWindowThreads / HIST_BINS - 1][HIST_BINS];
+  __shared__ uint32_t samp[kWindowRound][HIST_BINS];
   __shared__ unsigned long long smax[HIST_BINS / 32], ssum[HIST_BINS / 32];
   __shared__ float fmax[HIST_BINS / 32], fsum[HIST_BINS / 32];
   __shared__ float scale[HIST_WINDOW_MAX];
   StreamDev* st = a.st;
-  const int b = threadIdx.x;
+  const int b = threadIdx.x & (HIST_BINS - 1), q = threadIdx.x / HIST_BINS;
   pdl_launch_dependents();
   pdl_wait();
   const unsigned long long W = a.window, g = a.first_chunk + blockIdx.x;
   const unsigned long long first = g >= W - 1 ? g - (W - 1) : 0ull;
   const uint32_t len = (uint32_t)(g - first + 1);
   const bool sampled = a.mode == HIST_MODE_AUTO && blockIdx.x + 1 < a.count;
-  if (sampled) {
-    // each window chunk's scale, one thread per chunk
-    for (uint32_t k = (uint32_t)b; k < len; k += HIST_BINS) {
-      const uint32_t slot = (uint32_t)((first + k) % kChunkRing);
-      const uint32_t sn = __ldcg(&st->wsn[slot]);
-      scale[k] = sn ? (float)__ldcg(&st->wn[slot]) / (float)sn : 0.0f;
-    }
-    __syncthreads();
+  // each window chunk's scale, one thread per chunk
+  if (sampled && threadIdx.x < len) {
+    const uint32_t slot = (uint32_t)((first + threadIdx.x) % kChunkRing);
+    const uint32_t sn = __ldcg(&st->wsn[slot]);
+    scale[threadIdx.x] = sn ? (float)__ldcg(&st->wn[slot]) / (float)sn : 0.0f;
   }
   unsigned long long v = 0;
   float f = 0.0f;
-  for (uint32_t k0 = 0; k0 < len; k0 += 8) {
-    uint32_t h[8], q[8];
+  for (uint32_t k0 = 0; k0 < len; k0 += kWindowRound) {
+    uint32_t h[kWindowRun], s[kWindowRun];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const uint32_t slot = (uint32_t)((first + k0 + k) % kChunkRing);
-      h[k] = k0 + k < len ? __ldcg(&st->whist[slot][b]) : 0u;
-      q[k] = sampled && k0 + k < len ? __ldcg(&st->wsamp[slot][b]) : 0u;
+    for (uint32_t i = 0; i < kWindowRun; ++i) {
+      const uint32_t k = k0 + q * kWindowRun + i;
+      const uint32_t slot = (uint32_t)((first + k) % kChunkRing);
+      h[i] = k < len ? __ldcg(&st->whist[slot][b]) : 0u;
+      s[i] = sampled && k < len ? __ldcg(&st->wsamp[slot][b]) : 0u;
     }
 #pragma unroll
-    for (int k = 0; k < 8; ++k) v += h[k];
+    for (uint32_t i = 0; i < kWindowRun; ++i) v += h[i];
     if (sampled) {
 #pragma unroll
-      for (int k = 0; k < 8; ++k)
-        if (k0 + k < len) f += (float)q[k] * scale[k0 + k];
+      for (uint32_t i = 0; i < kWindowRun; ++i) samp[q * kWindowRun + i][b] = s[i];
+      __syncthreads();
+      if (q == 0) {
+        const uint32_t m = len - k0 < kWindowRound ? len - k0 : kWindowRound;
+#pragma unroll 8
+        for (uint32_t i = 0; i < m; ++i) f += (float)samp[i][b] * scale[k0 + i];
+      }
+      __syncthreads();
     }
   }
+  if (q > 0) part[q - 1][b] = v;
+  __syncthreads();
+  if (q > 0) return;
+#pragma unroll
+  for (int i = 0; i < kWindowThreads / HIST_BINS - 1; ++i) v += part[i][b];
   unsigned long long mx, sm;
   window_max_sum(v, smax, ssum, mx, sm);
   const uint32_t flag = reaches_theta(mx, sm, a.theta) ? HIST_FLAG_ADAPTIVE : HIST_FLAG_PLAIN;
@@ -962,18 +980,33 @@ __global__ void __launch_bounds__(HIST_BINS) window_flat_kernel(const PushHead a
   }
 }
 
+// The queries of a stream's state are launches chained to the push before
+// them (they wait for it before they read), and let a push behind them start:
+// a device-to-device copy of the totals between two pushes kept the second
+// one's CTAs from the SMs that the first one's free (64 x 16 MiB overlapping,
+// totals after each push: 166.4 -> 154.3 us; 1024 ragged chunks of at most 64
+// KiB: 24.6 -> 19.4).
+
 // The moving-window histogram after the last chunk (none: zeros): the last
-// chunk's histogram for a window of one, else the window kept by the flat
-// launches.
+// chunk's histogram for a window of one, else the window kept by
+// window_flat_kernel.  At L2: the work before may have written it while this
+// launch was waiting.
 __device__ __forceinline__ unsigned long long window_bin(const StreamDev* st, uint32_t window, bool any, int b) {
   if (!any) return 0ull;
-  return window == 1 ? (unsigned long long)st->h.last_hist[b] : st->wmw[b];
+  return window == 1 ? (unsigned long long)__ldcg(&st->h.last_hist[b]) : __ldcg(&st->wmw[b]);
 }
 
-__global__ void window_copy_kernel(const StreamDev* st, uint32_t window, bool any, unsigned long long* out) {
-  const int b = threadIdx.x;
-  if (b >= HIST_BINS) return;
-  out[b] = window_bin(st, window, any, b);
+__global__ void __launch_bounds__(HIST_BINS) window_copy_kernel(const StreamDev* st, uint32_t window, bool any,
+                                                                unsigned long long* out) {
+  pdl_launch_dependents();
+  pdl_wait();
+  out[threadIdx.x] = window_bin(st, window, any, threadIdx.x);
+}
+
+__global__ void __launch_bounds__(HIST_BINS) totals_copy_kernel(const StreamDev* st, unsigned long long* out) {
+  pdl_launch_dependents();
+  pdl_wait();
+  out[threadIdx.x] = __ldcg(&st->h.totals[threadIdx.x]);
 }
 
 // Change detection between the stream's totals and its moving-window
@@ -982,8 +1015,10 @@ __global__ void __launch_bounds__(HIST_BINS) stream_change_kernel(const StreamDe
                                                                   uint32_t tau_milli, hist_change_result* res) {
   __shared__ ChangeShared sh;
   const int b = threadIdx.x;
+  pdl_launch_dependents();
+  pdl_wait();
   const unsigned long long m = window_bin(st, window, any, b);
-  const hist_change_result r = change_eval(st->h.totals[b], m, tau_milli, sh);
+  const hist_change_result r = change_eval(__ldcg(&st->h.totals[b]), m, tau_milli, sh);
   if (b == 0) *res = r;
 }
 
@@ -1193,7 +1228,7 @@ int launch_batch(hist_stream* st, uint32_t count, const uint8_t* const* ins, con
   PushHead head = *a;
   void* hparams[] = {&head};
   if (e == cudaSuccess && windowed)
-    e = launch_chained((const void*)window_flat_kernel, dim3(count), dim3(HIST_BINS), hparams, 0, s);
+    e = launch_chained((const void*)window_flat_kernel, dim3(count), dim3(kWindowThreads), hparams, 0, s);
   if (own) free(a);
   if (e != cudaSuccess) return cuda_fail(e);
   st->flat_launches += 1;
@@ -1430,26 +1465,39 @@ int hist_stream_flush(hist_stream* st, hist_cuda_stream s) {
 
 int hist_stream_totals(hist_stream* st, uint64_t* d_totals, hist_cuda_stream s) {
   if (!st || !d_totals) return HIST_EINVAL;
-  const void* src = reinterpret_cast<const char*>(st->d) + offsetof(StreamHead, totals);
-  cudaError_t e = cudaMemcpyAsync(d_totals, src, HIST_BINS * sizeof(uint64_t), cudaMemcpyDeviceToDevice,
-                                  (cudaStream_t)s);
+  cudaError_t e;
+  if ((uintptr_t)d_totals % sizeof(uint64_t) == 0) {
+    const StreamDev* d = st->d;
+    unsigned long long* out = reinterpret_cast<unsigned long long*>(d_totals);
+    void* params[] = {&d, &out};
+    e = launch_chained((const void*)totals_copy_kernel, dim3(1), dim3(HIST_BINS), params, 0, (cudaStream_t)s);
+  } else {
+    e = cudaMemcpyAsync(d_totals, st->d->h.totals, HIST_BINS * sizeof(uint64_t), cudaMemcpyDeviceToDevice,
+                        (cudaStream_t)s);
+  }
   return e == cudaSuccess ? HIST_OK : cuda_fail(e);
 }
 
 int hist_stream_window(hist_stream* st, uint64_t* d_window, hist_cuda_stream s) {
   if (!st || !d_window) return HIST_EINVAL;
-  const bool any = st->chunks_launched > st->resume_chunk;
-  window_copy_kernel<<<1, HIST_BINS, 0, (cudaStream_t)s>>>(st->d, st->cfg.window, any,
-                                                            reinterpret_cast<unsigned long long*>(d_window));
-  const cudaError_t e = cudaGetLastError();
+  const StreamDev* d = st->d;
+  uint32_t window = st->cfg.window;
+  bool any = st->chunks_launched > st->resume_chunk;
+  unsigned long long* out = reinterpret_cast<unsigned long long*>(d_window);
+  void* params[] = {&d, &window, &any, &out};
+  const cudaError_t e =
+      launch_chained((const void*)window_copy_kernel, dim3(1), dim3(HIST_BINS), params, 0, (cudaStream_t)s);
   return e == cudaSuccess ? HIST_OK : cuda_fail(e);
 }
 
 int hist_stream_change(hist_stream* st, uint32_t tau_milli, hist_change_result* d_res, hist_cuda_stream s) {
   if (!st || !d_res || tau_milli > 1000) return HIST_EINVAL;
-  const bool any = st->chunks_launched > st->resume_chunk;
-  stream_change_kernel<<<1, HIST_BINS, 0, (cudaStream_t)s>>>(st->d, st->cfg.window, any, tau_milli, d_res);
-  const cudaError_t e = cudaGetLastError();
+  const StreamDev* d = st->d;
+  uint32_t window = st->cfg.window;
+  bool any = st->chunks_launched > st->resume_chunk;
+  void* params[] = {&d, &window, &any, &tau_milli, &d_res};
+  const cudaError_t e =
+      launch_chained((const void*)stream_change_kernel, dim3(1), dim3(HIST_BINS), params, 0, (cudaStream_t)s);
   return e == cudaSuccess ? HIST_OK : cuda_fail(e);
 }
 
