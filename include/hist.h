@@ -321,11 +321,15 @@ int hist_stream_set_state(hist_stream* st, const hist_stream_state* h_state, his
  * d_ptrs / d_sizes are DEVICE arrays of `count` image pointers and sizes
  * (each image below 2^32 bytes, any alignment); d_out is count x uint32_t[256]
  * on the device, overwritten: histogram i is d_out[256 i .. 256 i + 255].
- * Work: a memset of d_out and one kernel per HIST_BATCH_MAX_IMAGES images.
- * Each CTA takes an equal share of the images' concatenated bytes and counts
- * it in a lane-private sub-bin table (k = 32 sub-bins per bin), or with
- * 2^small_log2k sub-bins for images below small_bytes; a CTA adds into an
- * image's output where its share leaves the image.  No scratch memory. */
+ * Work, per HIST_BATCH_MAX_IMAGES images: with every image in the
+ * lane-private layout (the default) two kernels, one for the small images and
+ * one for the rest; else a memset of d_out and one kernel.  Each CTA takes an
+ * equal share of the images' cost (bytes and a fixed cost per image) and
+ * counts it in a lane-private sub-bin table (k = 32 sub-bins per bin; images
+ * of at most 4 KiB in one table per warp), or with 2^small_log2k sub-bins for
+ * images below small_bytes; a CTA adds into an image's output where its share
+ * leaves the image.  ctas_per_sm and unroll shape the second kind only.  No
+ * scratch memory. */
 #define HIST_BATCH_MAX_IMAGES 4096u
 
 typedef struct hist_batch_tuning {
@@ -342,7 +346,7 @@ void hist_batch_tuning_init(hist_batch_tuning* t);
 int hist_batch(const uint8_t* const* d_ptrs, const size_t* d_sizes, uint32_t count, uint32_t* d_out,
                const hist_batch_tuning* tuning, hist_cuda_stream s);
 
-/* The same batch as an instantiated CUDA graph (memset + kernels), for
+/* The same batch as an instantiated CUDA graph, for
  * replaying over new contents of the same device arrays and buffers.  The
  * caller owns the graph (hist_batch_graph_destroy). */
 typedef struct hist_batch_graph hist_batch_graph;
@@ -408,15 +412,15 @@ void hist_batch_table_init(hist_batch_table* t);
 int hist_batch_classify(const uint8_t* const* d_ptrs, const size_t* d_sizes, uint32_t count, uint32_t theta_milli,
                         uint8_t* d_regime, hist_cuda_stream s);
 
-/* hist_batch with a per-regime table: a memset of d_out, hist_batch_classify
- * into d_regime (count bytes on the device, the caller's; the regimes stay
- * there), then one counting kernel per HIST_BATCH_MAX_IMAGES images in which
- * each image is counted with its regime's setting.  No other device memory.
+/* hist_batch with a per-regime table: hist_batch_classify into d_regime
+ * (count bytes on the device, the caller's; the regimes stay there), then
+ * hist_batch's launches, in which each image is counted with its regime's
+ * setting.  No other device memory.
  * table null = hist_batch_table_init.  HIST_EINVAL for a bad table. */
 int hist_batch_regimes(const uint8_t* const* d_ptrs, const size_t* d_sizes, uint32_t count, uint32_t* d_out,
                        uint8_t* d_regime, const hist_batch_table* table, hist_cuda_stream s);
 
-/* The same as an instantiated CUDA graph (memset, classification, counting),
+/* The same as an instantiated CUDA graph (classification, counting),
  * destroyed with hist_batch_graph_destroy. */
 int hist_batch_regimes_capture(const uint8_t* const* d_ptrs, const size_t* d_sizes, uint32_t count,
                                uint32_t* d_out, uint8_t* d_regime, const hist_batch_table* table,

@@ -166,6 +166,377 @@ __global__ void __launch_bounds__(kThreads, MINB) batch_images_kernel(BatchImgAr
   }
 }
 
+// ------------------------------------------------ the lane-private kernels --
+//
+// A batch whose images are all counted in the lane-private table (layout 5,
+// the default) is two launches of batch_lane_kernel, each of one CTA of 1024
+// threads per SM, each CTA taking an equal share of the cost of the launch's
+// images, a contiguous range of them placed end to end.
+//
+// The first launch counts whole images of at most kLaneSmall bytes: those of
+// at most kLaneTiny by a warp each, in a 256-bin table of its own, the others
+// by four groups of eight warps, an image at a time each, a thread per bin,
+// in a lane-private table each.  It also clears the outputs of the other
+// images.  The second launch counts those, piece by piece, the whole CTA on
+// each, which has the start of the next piece fetched into L2 while it
+// reduces the table; its CTAs start on the SMs that the first's leave and
+// wait for it before they write.  Two launches because the groups' tables
+// (128 KiB) would take the L1 cache from the large images' loads (64 stream
+// chunks of 16 MiB: 161 us with 80 KiB of shared memory, 176 with 146), and
+// because one kernel with both loops spills registers.
+//
+// Bound by the HBM read on large images, by the prologue (sizes, two scans,
+// the window's list: 3.5 us) and latency on small ones.  On the GPU, replayed
+// from a graph, before (one CTA-wide loop over all images, two CTAs per SM)
+// and now: 4096 images of 64 .. 4096 a side (9.97 GB) 1491 -> 1406 us (7.09
+// TB/s), 464 of 314 .. 2303 (0.68 GB) 123 -> 113, 2048 of 16 .. 256 (29 MB)
+// 38.8 -> 19.5, 4096 of 8 .. 22 51 -> 8.5 us.
+
+constexpr uint32_t kLaneGroups = 4;
+constexpr int kLaneGroupThreads = kThreads / (int)kLaneGroups;
+static_assert(kLaneGroupThreads == HIST_BINS, "one bin per thread of a group");
+constexpr int kLaneWindow = 64;  // images of the range taken at a time
+constexpr uint32_t kLanePer = kBatchMaxImages / kThreads;  // images per thread in the cost prefix
+template <bool SMALL>
+__host__ __device__ constexpr size_t lane_smem() {
+  return (size_t)(SMALL ? kLaneGroups : 1u) * kTableWords * 4;
+}
+
+// Largest image a group counts whole.
+constexpr uint32_t kLaneSmall = 128u << 10;
+// Largest image a warp counts alone.  Its increments meet in banks (3.5
+// wavefronts per 32 uniform pixels), but a lane-private table takes 512
+// wavefronts to sum and clear: as many as 6.5 KB of uniform pixels, or more
+// of peaked ones, lose to conflicts.
+constexpr uint32_t kLaneTiny = 4u << 10;
+constexpr int kTinyLoads = 2;  // vectors in flight per lane
+// Fixed cost of an image beside its bytes: what a group or a CTA counts in
+// the time of an image's reduction.
+constexpr unsigned long long kLaneSmallCost = 24ull << 10;
+template <bool SMALL>
+__device__ __forceinline__ unsigned long long lane_cost(unsigned long long n) {
+  return n + (SMALL ? kLaneSmallCost : kImageCost);
+}
+
+struct LanePiece {
+  const uint8_t* base;
+  uint32_t len;
+  uint32_t image;  // bit 31: the whole image
+};
+struct alignas(16) LaneItem {
+  const uint4* body;
+  uint32_t nvec;
+  uint32_t image;
+  uint32_t head, tail;
+};
+
+struct LaneArgs {
+  const uint8_t* const* ptrs;
+  const size_t* sizes;
+  uint32_t* out;
+  unsigned long long inv;  // floor((2^64 - 1) / grid)
+  uint32_t count;
+};
+
+template <bool SMALL>
+struct LaneShared {
+  unsigned long long wsum[kWarps];
+  unsigned long long lo, hi;    // the CTA's cost range
+  unsigned long long share;     // the batch's bytes / grid
+  unsigned long long next_pos;  // cost position of the next window's first image
+  uint32_t i0;                  // the range's first image
+  uint32_t n;                   // entries of the window's list, the tiny images' first
+  uint32_t tiny;                // of them the tiny ones
+  uint32_t wcount[2][2];
+  LanePiece piece[SMALL ? 1 : kLaneWindow];
+  LaneItem item[SMALL ? kLaneWindow : 1];
+  uint32_t res[SMALL ? 1 : HIST_BINS];
+  uint32_t eh[SMALL ? kLaneGroups : 1][HIST_BINS];  // edge bytes
+};
+
+// Whether an image of n bytes is the SMALL launch's: tiny, or at most
+// kLaneSmall bytes and half of a CTA's share of the batch (with fewer bytes
+// the images are better spread over the SMs in pieces: 26 images of 61 ..
+// 2615 a side 16.6 us, 18.8 if each of at most a share is counted whole, and
+// 2048 thumbnails 22.5 us if only those of a quarter are, 19.5 at half).
+__device__ __forceinline__ bool lane_small(unsigned long long n, unsigned long long share) {
+  return n <= kLaneTiny || (n <= kLaneSmall && n * 2 <= share);
+}
+
+// Inclusive block scan of v; the block's sum in `total` (one barrier; the
+// caller puts one before wsum is written again).
+__device__ __forceinline__ unsigned long long warp_scan(unsigned long long v) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned long long y = __shfl_up_sync(0xffffffffu, v, o);
+    if (lane >= o) v += y;
+  }
+  return v;
+}
+__device__ __forceinline__ unsigned long long block_scan(unsigned long long v, unsigned long long* wsum,
+                                                         unsigned long long& total) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const unsigned long long x = warp_scan(v);
+  if (lane == 31) wsum[w] = x;
+  __syncthreads();
+  const unsigned long long s = warp_scan(wsum[lane]);  // kWarps == 32
+  total = __shfl_sync(0xffffffffu, s, 31);
+  const unsigned long long before = __shfl_sync(0xffffffffu, s, (w + 31) & 31);
+  return (w ? before : 0ull) + x;
+}
+static_assert(kWarps == 32, "a lane per warp in block_scan");
+
+// floor(x / grid) or a little less, for inv = floor((2^64 - 1) / grid): every
+// CTA takes the same cuts from it, without the 64-bit division's 150
+// instructions in 32 warps (2 us).
+__device__ __forceinline__ unsigned long long grid_share(unsigned long long x, unsigned long long inv) {
+  return __umul64hi(x, inv);
+}
+
+// The window of images from i0 on, whose first has cost position
+// ls.next_pos: warps 0 and 1 (an image per lane) list what this CTA counts of
+// them.  All threads call (barriers before and after are the caller's).
+template <bool SMALL>
+__device__ __forceinline__ void lane_window(const LaneArgs& a, uint32_t i0, LaneShared<SMALL>& ls) {
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+  if (t >= kLaneWindow) return;
+  const GroupBar<kLaneWindow> bar = {15};
+  const uint32_t i = i0 + (uint32_t)t;
+  const bool in = i < a.count;
+  const unsigned long long n = in ? (unsigned long long)a.sizes[i] : 0ull;
+  const uint8_t* p = in ? a.ptrs[i] : nullptr;
+  const bool mine = n && lane_small(n, ls.share) == SMALL;
+  const unsigned long long c = mine ? lane_cost<SMALL>(n) : 0ull;
+  const unsigned long long x = warp_scan(c);
+  const unsigned long long pos = ls.next_pos;
+  if (lane == 31) ls.wsum[w] = x;
+  bar.sync();
+  const unsigned long long p0 = pos + (w ? ls.wsum[0] : 0ull) + x - c;
+  unsigned long long b0 = 0, e0 = 0;
+  if (mine && p0 < ls.hi) {
+    if (SMALL) {
+      // the range holding its first cost position counts it
+      if (p0 >= ls.lo) e0 = n;
+    } else {
+      b0 = ls.lo > p0 ? split_point(p, ls.lo - p0) : 0ull;
+      e0 = split_point(p, ls.hi - p0);
+      if (e0 > n) e0 = n;
+    }
+  }
+  const bool tiny = SMALL && b0 < e0 && n <= kLaneTiny, other = b0 < e0 && !tiny;
+  const unsigned mt = __ballot_sync(0xffffffffu, tiny), mo = __ballot_sync(0xffffffffu, other);
+  if (lane == 0) {
+    ls.wcount[w][0] = __popc(mt);
+    ls.wcount[w][1] = __popc(mo);
+  }
+  bar.sync();
+  const uint32_t ntiny = ls.wcount[0][0] + ls.wcount[1][0];
+  if (tiny || other) {
+    const unsigned lt = (1u << lane) - 1u;
+    const uint32_t k = tiny ? (w ? ls.wcount[0][0] : 0u) + __popc(mt & lt)
+                            : ntiny + (w ? ls.wcount[0][1] : 0u) + __popc(mo & lt);
+    if (SMALL) {
+      // (a warp's vectors need no whole lines)
+      const Split sp = split_bytes_at(p, (size_t)n, tiny ? 16 : kLineBytes);
+      LaneItem& q = ls.item[k];
+      q.body = reinterpret_cast<const uint4*>(p + sp.head);
+      q.nvec = (uint32_t)sp.nvec;
+      q.image = i;
+      q.head = (uint32_t)sp.head;
+      q.tail = (uint32_t)sp.tail;
+    } else {
+      LanePiece& q = ls.piece[k];
+      q.base = p + b0;
+      q.len = (uint32_t)(e0 - b0);
+      q.image = i | (b0 == 0 && e0 == n ? 1u << 31 : 0u);
+    }
+  }
+  if (t == kLaneWindow - 1) {
+    ls.next_pos = p0 + c;
+    ls.tiny = ntiny;
+    ls.n = ntiny + ls.wcount[0][1] + ls.wcount[1][1];
+  }
+}
+
+// Count the window's pieces, the whole CTA, into the table (clear before and
+// after).
+__device__ __forceinline__ void lane_pieces(const LaneArgs& a, uint32_t* table, LaneShared<false>& ls) {
+  const int t = threadIdx.x;
+  for (uint32_t k = 0; k < ls.n; ++k) {
+    piece_count(ls.piece[k].base, ls.piece[k].len, table, ls.eh[0], nullptr, nullptr);
+    if (k + 1 < ls.n) {
+      const uint32_t at = (uint32_t)t * kLineBytes;
+      if (at < ls.piece[k + 1].len) asm volatile("prefetch.global.L2 [%0];" ::"l"(ls.piece[k + 1].base + at));
+    }
+    __syncthreads();
+    lane_reduce<kThreads, true>(table, ls.res, t);
+    __syncthreads();
+    if (t < HIST_BINS) {
+      const uint32_t h = ls.res[t] + ls.eh[0][t];
+      ls.eh[0][t] = 0;
+      if (k == 0) pdl_wait();  // the output is clear
+      const uint32_t image = ls.piece[k].image;
+      uint32_t* o = a.out + (size_t)(image & 0x7fffffffu) * HIST_BINS + t;
+      if (image >> 31) *o = h;
+      else if (h) atomicAdd(o, h);
+    }
+    __syncthreads();
+  }
+}
+
+// Count the window's tiny images, a warp each, in the warp's 256 words of the
+// first table (clear before and after).
+__device__ __forceinline__ void lane_tiny(const LaneArgs& a, uint32_t* tables, const LaneShared<true>& ls) {
+  const uint32_t w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  uint32_t* h = tables + w * HIST_BINS;
+  for (uint32_t i = w; i < ls.tiny; i += kWarps) {
+    const LaneItem& it = ls.item[i];
+    const uint8_t* in = reinterpret_cast<const uint8_t*>(it.body) - it.head;
+    uint32_t edge = 0x100u;
+    if (lane < it.head) edge = in[lane];
+    else if (lane - it.head < it.tail) edge = reinterpret_cast<const uint8_t*>(it.body + it.nvec)[lane - it.head];
+    LaneRange r = lane_range(it.body, 0, it.nvec, (int)lane);
+    uint4 v[kTinyLoads];
+    lane_load<kTinyLoads, 32>(v, r);
+    if (edge < 0x100u) atomicAdd(&h[edge], 1u);
+    while (r.left) {
+#pragma unroll
+      for (int u = 0; u < kTinyLoads; ++u)
+        if ((uint32_t)(u * 32) < r.left) vec_count(v[u], h);
+      r.q += kTinyLoads * 32;
+      r.left = r.left > kTinyLoads * 32 ? r.left - kTinyLoads * 32 : 0u;
+      lane_load<kTinyLoads, 32>(v, r);
+    }
+    __syncwarp();
+    uint32_t* out = a.out + (size_t)it.image * HIST_BINS;
+#pragma unroll
+    for (int k = 0; k < HIST_BINS / 32; ++k) {
+      out[lane + 32 * k] = h[lane + 32 * k];
+      h[lane + 32 * k] = 0;
+    }
+    __syncwarp();
+  }
+}
+
+// Count the window's other images, a group each at a time (the tables clear
+// before and after).
+__device__ __forceinline__ void lane_items(const LaneArgs& a, uint32_t* tables, LaneShared<true>& ls) {
+  const uint32_t g = threadIdx.x / kLaneGroupThreads;
+  const int t = threadIdx.x % kLaneGroupThreads;
+  const GroupBar<kLaneGroupThreads> bar = {1 + (int)g};
+  uint32_t* table = tables + g * kTableWords;
+  const uint32_t base = smem_addr(table) + ((t & 31) << 2);
+  const uint32_t n = ls.n;
+  uint32_t i = ls.tiny + g;
+  if (i >= n) return;
+  uint4 v[kLaneLoads];
+  lane_load<kLaneLoads, kLaneGroupThreads>(v, lane_range(ls.item[i].body, 0, ls.item[i].nvec, t));
+  auto edge_of = [&](const LaneItem& it) -> uint32_t {
+    if ((uint32_t)t >= it.head + it.tail) return 0x100u;
+    return (uint32_t)t < it.head ? *(reinterpret_cast<const uint8_t*>(it.body) - it.head + t)
+                                 : reinterpret_cast<const uint8_t*>(it.body + it.nvec)[t - it.head];
+  };
+  uint32_t edge = edge_of(ls.item[i]);
+  for (; i < n; i += kLaneGroups) {
+    const LaneItem& it = ls.item[i];
+    if (edge < 0x100u) atomicAdd(&ls.eh[g][edge], 1u);
+    edge = 0x100u;
+    LaneRange next = {nullptr, 0};
+    if (i + kLaneGroups < n) {
+      const LaneItem& it2 = ls.item[i + kLaneGroups];
+      edge = edge_of(it2);
+      next = lane_range(it2.body, 0, it2.nvec, t);
+    }
+    lane_count<kLaneLoads, kLaneGroupThreads>(v, lane_range(it.body, 0, it.nvec, t), base, next);
+    bar.sync();
+    uint32_t h = lane_row(table, t);
+    if (it.head + it.tail) {
+      h += ls.eh[g][t];
+      ls.eh[g][t] = 0;
+    }
+    a.out[(size_t)it.image * HIST_BINS + t] = h;
+    bar.sync();
+  }
+}
+
+template <bool SMALL>
+__global__ void __launch_bounds__(kThreads, 1) batch_lane_kernel(const __grid_constant__ LaneArgs a) {
+  extern __shared__ __align__(16) uint32_t tables[];
+  __shared__ LaneShared<SMALL> ls;
+  const int t = threadIdx.x;
+  pdl_launch_dependents();
+  // the batch's bytes: thread t holds images kLanePer t ...
+  unsigned long long n[kLanePer], local = 0, total;
+#pragma unroll
+  for (uint32_t k = 0; k < kLanePer; ++k) {
+    const uint32_t i = (uint32_t)t * kLanePer + k;
+    n[k] = i < a.count ? (unsigned long long)a.sizes[i] : 0ull;
+    local += n[k];
+  }
+  // one image per warp of the grid (the grid has at least kBatchMaxImages
+  // warps: launch_batch_lane)
+  const uint32_t zi = blockIdx.x * kWarps + ((uint32_t)t >> 5);
+  const unsigned long long zsize = SMALL && zi < a.count ? (unsigned long long)a.sizes[zi] : 0ull;
+  {
+    uint4* t4 = reinterpret_cast<uint4*>(tables);
+    for (int i = t; i < (int)(lane_smem<SMALL>() / 16); i += kThreads) t4[i] = make_uint4(0, 0, 0, 0);
+  }
+  if (t < (int)(sizeof(ls.eh) / 4)) (&ls.eh[0][0])[t] = 0;
+  if (t == 0) ls.i0 = a.count;
+  block_scan(local, ls.wsum, total);
+  const unsigned long long share = grid_share(total, a.inv);
+  if (SMALL && zi < a.count && !(zsize && lane_small(zsize, share))) {
+    // an output that is not this launch's to write
+#pragma unroll
+    for (int k = 0; k < HIST_BINS / 32; ++k) a.out[(size_t)zi * HIST_BINS + (t & 31) + 32 * k] = 0;
+  }
+  // this launch's images' costs, and the one that holds cost position lo
+  local = 0;
+#pragma unroll
+  for (uint32_t k = 0; k < kLanePer; ++k) {
+    n[k] = n[k] && lane_small(n[k], share) == SMALL ? lane_cost<SMALL>(n[k]) : 0ull;
+    local += n[k];
+  }
+  if (!__syncthreads_or(local != 0)) {  // (and wsum is read)
+    if (!SMALL) pdl_wait();  // the launch ends after the first
+    return;
+  }
+  unsigned long long pos = block_scan(local, ls.wsum, total) - local;
+  const unsigned long long lo = grid_share(total * blockIdx.x, a.inv);
+  if (t == 0) {
+    ls.lo = lo;
+    ls.hi = blockIdx.x + 1 == gridDim.x ? total : grid_share(total * (blockIdx.x + 1), a.inv);
+    ls.share = share;
+  }
+#pragma unroll
+  for (uint32_t k = 0; k < kLanePer; ++k) {
+    if (n[k] && pos <= lo && lo < pos + n[k]) {
+      ls.i0 = (uint32_t)t * kLanePer + k;
+      ls.next_pos = pos;
+    }
+    pos += n[k];
+  }
+  __syncthreads();
+  for (uint32_t i0 = ls.i0; i0 < a.count; i0 += kLaneWindow) {
+    lane_window<SMALL>(a, i0, ls);
+    __syncthreads();
+    const bool last = ls.next_pos >= ls.hi;
+    if constexpr (SMALL) {
+      if (ls.tiny) {
+        lane_tiny(a, tables, ls);
+        __syncthreads();
+      }
+      lane_items(a, tables, ls);
+    } else {
+      lane_pieces(a, tables, ls);
+    }
+    __syncthreads();  // the window's list is read
+    if (last) break;
+  }
+  if (!SMALL) pdl_wait();  // (a CTA with nothing to write)
+}
+
 // The regime of image blockIdx.x (rule in hist.h): 256 threads; thread t
 // takes run t of the sample (16 consecutive pixels from floor(t n / 256)),
 // or pixels t, t + 256, ... of an image of at most 4096 pixels, loading all
@@ -248,9 +619,57 @@ RegimeLayouts layouts_of(const hist_batch_table& tb) {
   return l;
 }
 
+// Whether a batch counts every image in the lane-private table.
+bool lane_layouts(const RegimeLayouts& l) {
+  for (uint32_t r = 0; r < HIST_REGIMES; ++r)
+    if (l.layout[r] != 5 || (l.small_bytes[r] && l.small_layout[r] != 5)) return false;
+  return true;
+}
+
+// The launches of batch_lane_kernel.  The first starts when the work before it
+// is complete; the second reads nothing that the first writes, and writes
+// after it.
+int launch_batch_lane(const uint8_t* const* d_ptrs, const size_t* d_sizes, uint32_t count, uint32_t* d_out,
+                      cudaStream_t s) {
+  static int attr[kMaxDevices];
+  const int rc = ensure_smem_attr_bytes((const void*)batch_lane_kernel<true>, attr, lane_smem<true>());
+  if (rc) return rc;
+  for (uint32_t first = 0; first < count; first += kBatchMaxImages) {
+    LaneArgs a;
+    a.ptrs = d_ptrs + first;
+    a.sizes = d_sizes + first;
+    a.out = d_out + (size_t)first * HIST_BINS;
+    a.count = count - first < kBatchMaxImages ? count - first : kBatchMaxImages;
+    cudaLaunchConfig_t lc = {};
+    cudaLaunchAttribute at[1];
+    // (at least kBatchMaxImages warps in all)
+    const int sms = sm_count(), least = (int)kBatchMaxImages / kWarps;
+    lc.gridDim = dim3((unsigned)(sms > least ? sms : least));
+    lc.blockDim = dim3(kThreads);
+    lc.stream = s;
+    a.inv = ~0ull / lc.gridDim.x;
+    lc.dynamicSmemBytes = lane_smem<true>();
+    cudaError_t e = cudaLaunchKernelEx(&lc, batch_lane_kernel<true>, a);
+    if (e != cudaSuccess) return cuda_fail(e);
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    lc.attrs = at;
+    lc.numAttrs = 1;
+    lc.dynamicSmemBytes = lane_smem<false>();
+    e = cudaLaunchKernelEx(&lc, batch_lane_kernel<false>, a);
+    if (e != cudaSuccess) return cuda_fail(e);
+  }
+  return HIST_OK;
+}
+
 int launch_batch_images(const hist_batch_tuning& tu, const RegimeLayouts& lay, const uint8_t* regime,
                         const uint8_t* const* d_ptrs, const size_t* d_sizes, uint32_t count, uint32_t* d_out,
                         cudaStream_t s) {
+  if (lane_layouts(lay)) return launch_batch_lane(d_ptrs, d_sizes, count, d_out, s);
+  if (count) {  // (no images: only the kernel's attributes are set up)
+    const cudaError_t e = cudaMemsetAsync(d_out, 0, (size_t)count * HIST_BINS * sizeof(uint32_t), s);
+    if (e != cudaSuccess) return cuda_fail(e);
+  }
   // one CTA per SM with 64 registers (2 or 4 loads in flight), or two with 32
   // registers (2 loads in flight)
   static int attr21[kMaxDevices], attr41[kMaxDevices], attr22[kMaxDevices];
@@ -317,8 +736,6 @@ hist_batch_tuning shape_of(const hist_batch_table& t) {
 int batch_regimes(const uint8_t* const* d_ptrs, const size_t* d_sizes, uint32_t count, uint32_t* d_out,
                   uint8_t* d_regime, const hist_batch_table& tb, cudaStream_t s) {
   if (count == 0) return HIST_OK;
-  cudaError_t e = cudaMemsetAsync(d_out, 0, (size_t)count * HIST_BINS * sizeof(uint32_t), s);
-  if (e != cudaSuccess) return cuda_fail(e);
   int rc = launch_regimes(d_ptrs, d_sizes, count, tb.theta_milli, d_regime, s);
   if (rc) return rc;
   return launch_batch_images(shape_of(tb), layouts_of(tb), d_regime, d_ptrs, d_sizes, count, d_out, s);
@@ -377,8 +794,6 @@ int hist_batch(const uint8_t* const* d_ptrs, const size_t* d_sizes, uint32_t cou
   else hist_batch_tuning_init(&tu);
   if (!tuning_ok(&tu) || (count && (!d_ptrs || !d_sizes || !d_out))) return HIST_EINVAL;
   if (count == 0) return HIST_OK;
-  cudaError_t e = cudaMemsetAsync(d_out, 0, (size_t)count * HIST_BINS * sizeof(uint32_t), (cudaStream_t)s);
-  if (e != cudaSuccess) return cuda_fail(e);
   return launch_batch_images(tu, layouts_of(tu), nullptr, d_ptrs, d_sizes, count, d_out, (cudaStream_t)s);
 }
 
@@ -616,8 +1031,6 @@ extern "C" int hist_batch_autotune_regimes(const uint8_t* const* d_ptrs, const s
       }
       const float ms = time_runs(
           [&]() {
-            cudaError_t me = cudaMemsetAsync(dout, 0, (size_t)rc_n * HIST_BINS * sizeof(uint32_t), s);
-            if (me != cudaSuccess) return cuda_fail(me);
             return launch_batch_images(shape, lay, nullptr, dp, dz, rc_n, dout, s);
           },
           s, e0, e1, repeats, &rc);

@@ -61,6 +61,12 @@ __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)
 __device__ __forceinline__ void shared_inc(uint32_t a) {
   asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(a) : "memory");
 }
+// The same by v.
+__device__ __forceinline__ void shared_add(uint32_t a, uint32_t v) {
+  asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+}
+struct IncOne {};
+__device__ __forceinline__ void shared_add(uint32_t a, IncOne) { shared_inc(a); }
 __device__ __forceinline__ uint32_t shared_ld(uint32_t a) {
   uint32_t v;
   asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
@@ -263,23 +269,31 @@ __device__ __forceinline__ void lane_load(uint4 (&v)[U], const LaneRange& r) {
     if ((uint32_t)(u * NTHR) < r.left) v[u] = ldg_stream(r.q + u * NTHR);
 }
 
+// The 16 pixels of a vector into the lane-private table at `base` (this
+// lane's column), each as `inc`.
+template <class Inc>
+__device__ __forceinline__ void lane_vec(const uint4& q, uint32_t base, Inc inc) {
+  const uint32_t w4[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+  for (int k = 0; k < 16; ++k) shared_add(base + (((w4[k >> 2] >> (8 * (k & 3))) & 0xffu) << 7), inc);
+}
+
 // Count this thread's vectors of r, whose first U are loaded in v
 // (lane_load), keeping U loads in flight while it counts: the next ones of
 // its own, and at its end the first U of r2, the range that comes next (left
-// = 0: none), which v holds on return.  (Refilling each vector's registers as
+// = 0: none), which v holds on return.  A pixel adds `inc`.  (Refilling each vector's registers as
 // soon as it is counted, with 4 to 8 vectors, put every load behind 16
 // increments in the memory queue: 64 chunks of 16 MiB 161 -> 168-172 us,
 // 1024 of 64 KiB 24 -> 32 us.)
-template <int U, int NTHR>
+template <int U, int NTHR, class Inc = IncOne>
 __device__ __forceinline__ void lane_count(uint4 (&v)[U], LaneRange r, uint32_t base,
-                                           const LaneRange& r2 = LaneRange{nullptr, 0}) {
-  const LaneOrder o = {0, 0};  // the natural order: every lane has its own bank
+                                           const LaneRange& r2 = LaneRange{nullptr, 0}, Inc inc = Inc()) {
   uint4 w[U];
   while (r.left > (uint32_t)((2 * U - 1) * NTHR)) {  // this round and the next are whole
 #pragma unroll
     for (int u = 0; u < U; ++u) w[u] = ldg_stream(r.q + (U + u) * NTHR);
 #pragma unroll
-    for (int u = 0; u < U; ++u) count_vec<PATH_SHIFT, 5>(v[u], base, 0, 0, o);
+    for (int u = 0; u < U; ++u) lane_vec(v[u], base, inc);
 #pragma unroll
     for (int u = 0; u < U; ++u) v[u] = w[u];
     r.q += U * NTHR;
@@ -291,7 +305,7 @@ __device__ __forceinline__ void lane_count(uint4 (&v)[U], LaneRange r, uint32_t 
     lane_load<U, NTHR>(w, next);
 #pragma unroll
     for (int u = 0; u < U; ++u)
-      if ((uint32_t)(u * NTHR) < r.left) count_vec<PATH_SHIFT, 5>(v[u], base, 0, 0, o);
+      if ((uint32_t)(u * NTHR) < r.left) lane_vec(v[u], base, inc);
 #pragma unroll
     for (int u = 0; u < U; ++u) v[u] = w[u];
     if (!more) return;
@@ -521,6 +535,28 @@ __device__ __forceinline__ void count_edges_into(const uint8_t* a, const Split& 
   const int t = threadIdx.x, L = (int)kLineBytes;
   if (t < (int)sp.head) atomicAdd(&h[a[t]], 1u);
   else if (t >= L && t < L + (int)sp.tail) atomicAdd(&h[a[sp.head + sp.nvec * 16 + (t - L)]], 1u);
+}
+
+// The 16 pixels of a vector into a 256-bin shared histogram.
+__device__ __forceinline__ void vec_count(const uint4& q, uint32_t* h) {
+  const uint32_t w4[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+  for (int k = 0; k < 16; ++k) atomicAdd(&h[(w4[k >> 2] >> (8 * (k & 3))) & 0xffu], 1u);
+}
+
+// Count len bytes at `base` into the lane-private table and the edge
+// histogram eh: the whole CTA, four loads in flight per thread; vec (null:
+// none): one more vector of this thread's, counted into samp.
+__device__ __forceinline__ void piece_count(const uint8_t* base, uint32_t len, uint32_t* table, uint32_t* eh,
+                                            const uint8_t* vec, uint32_t* samp) {
+  const Split sp = split_bytes(base, len);
+  uint4 v[kLaneLoads];
+  const LaneRange r =
+      lane_range(reinterpret_cast<const uint4*>(base + sp.head), 0, (uint32_t)sp.nvec, threadIdx.x);
+  lane_load<kLaneLoads, kThreads>(v, r);
+  count_edges_into(base, sp, eh);
+  if (vec) vec_count(ldg_stream(reinterpret_cast<const uint4*>(vec)), samp);
+  lane_count<kLaneLoads, kThreads>(v, r, smem_addr(table) + ((threadIdx.x & 31) << 2));
 }
 
 // Count head and tail bytes of a split into cs.res (threads 0..143).

@@ -284,12 +284,6 @@ __device__ __forceinline__ uint32_t sample_at(const uint8_t* in, uint32_t n, uin
   if (sp.nvec < kSampleVecs) return 0xffffffffu;
   return (uint32_t)(sp.head + 16 * ((size_t)k * sp.nvec / kSampleVecs));
 }
-__device__ __forceinline__ void sample_count(const uint4& q, uint32_t* h) {
-  const uint32_t w4[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-  for (int k = 0; k < 16; ++k) atomicAdd(&h[(w4[k >> 2] >> (8 * (k & 3))) & 0xffu], 1u);
-}
-
 // The larger of the warps' maxima m[0..7].
 __device__ __forceinline__ uint32_t max8(const uint32_t* m) {
   uint32_t mx = m[0];
@@ -518,19 +512,11 @@ __device__ __noinline__ void flat_flush(const A& a, const FlatDesc& d, uint32_t 
   __syncthreads();
 }
 
-// Count len bytes at `base` into the table and the edge histogram eh: the
-// whole CTA, four loads in flight per thread; vec (threads 0..255, null:
-// none): a sample vector among those bytes, counted into samp.
+// piece_count as a call of its own, which keeps the counting loop's registers
+// from what surrounds it.
 static __device__ __noinline__ void flat_count(const uint8_t* base, uint32_t len, uint32_t* table, uint32_t* eh,
                                                const uint8_t* vec, uint32_t* samp) {
-  const Split sp = split_bytes(base, len);
-  uint4 v[kLaneLoads];
-  const LaneRange r =
-      lane_range(reinterpret_cast<const uint4*>(base + sp.head), 0, (uint32_t)sp.nvec, threadIdx.x);
-  lane_load<kLaneLoads, kThreads>(v, r);
-  count_edges_into(base, sp, eh);
-  if (vec) sample_count(ldg_stream(reinterpret_cast<const uint4*>(vec)), samp);
-  lane_count<kLaneLoads, kThreads>(v, r, smem_addr(table) + ((threadIdx.x & 31) << 2));
+  piece_count(base, len, table, eh, vec, samp);
 }
 
 // Count bytes [b0, e0) of chunk d (not empty) into the table, which is clear
@@ -709,7 +695,7 @@ __device__ __noinline__ void group_count(const A& a, uint32_t count, bool releas
       // read after the chunk, so that its lines are in L2: ahead of it each
       // 16-byte vector is a DRAM access of its own
       const uint8_t* in = reinterpret_cast<const uint8_t*>(it.body) - (it.edges & 0xffu);
-      sample_count(ldg_stream(reinterpret_cast<const uint4*>(in + sample_at(in, it.n, t))), fs.gsamp[g]);
+      vec_count(ldg_stream(reinterpret_cast<const uint4*>(in + sample_at(in, it.n, t))), fs.gsamp[g]);
     }
     bar.sync();
     if (prev_n && t == 0) flat_compare(a, prev_n, max8(fs.gmax[g][0]), max8(fs.gmax[g][1]));

@@ -170,3 +170,47 @@ def test_a_captured_push_replayed():
         assert bytes(t.pattern) == ref.pattern.to_bytes() and bytes(t.last_pattern) == rec.pattern.to_bytes()
         assert t.flag == ref.flag and t.last_kernel == rec.kernel and t.chunks == ref.chunks
         st.close()
+
+
+def _batch(sizes, seed, spread, out_shift=0):
+    """hist_batch on random images of these sizes, at every alignment; the
+    output rows start out_shift words into a buffer of rubbish."""
+    rng = np.random.default_rng(seed)
+    offs, pos = [], 0
+    for n in sizes:
+        pos += int(rng.integers(0, spread))
+        offs.append(pos)
+        pos += n
+    x = rng.integers(0, 256, pos + 16, dtype=np.uint8)
+    x[rng.random(pos + 16) < 0.3] = 77
+    xd = dev(x)
+    ptrs = torch.tensor([xd.data_ptr() + o for o in offs], dtype=torch.int64, device="cuda")
+    szs = torch.tensor(list(sizes), dtype=torch.int64, device="cuda")
+    buf = torch.full((len(sizes) * 256 + out_shift,), -5, dtype=torch.int32, device="cuda")
+    out = buf[out_shift:]
+    rc = hl.lib().hist_batch(ptrs.data_ptr(), szs.data_ptr(), len(sizes), out.data_ptr(), None,
+                             torch.cuda.current_stream().cuda_stream)
+    assert rc == 0
+    got = u32(out).reshape(len(sizes), 256)
+    for i, (o, n) in enumerate(zip(offs, sizes)):
+        assert np.array_equal(got[i], oracle.hist_u32(x[o:o + n])), (i, n)
+    assert (buf[:out_shift] == -5).all()
+
+
+@pytest.mark.parametrize("name,sizes,out_shift", [
+    # on both sides of the warps', the groups' and the whole-image limits
+    ("edges", [0, 1, 15, 16, 127, 128, 143, 4095, 4096, 4097, 131_071, 131_072, 131_073, 500_000] * 40, 1),
+    # a few images, all cut between CTAs
+    ("few", [300_000, 131_072, 70_001, 5000, 4096, 3], 0),
+    # one range holds hundreds of tiny images (many windows of 64) between
+    # pieces of large ones
+    ("long", [20_000_000] + [9] * 700 + [5000] * 300 + [30_000_001] + [0] * 100 + [4097] * 200, 3),
+    # more images than one launch takes, tiny and not
+    ("many", [100 + 37 * (i % 300) for i in range(4096 + 70)], 2),
+    ("empty", [0, 0, 0], 0),
+    ("one", [1], 0),
+])
+def test_batch_lane_launches(name, sizes, out_shift):
+    """The default batch's two launches against the oracle, image by image:
+    sizes around every limit of their rule, outputs at any word."""
+    _batch(sizes, 17, 40, out_shift)
