@@ -207,7 +207,7 @@ void hist_config_init(hist_config* cfg);
 
 typedef struct hist_stream hist_stream;
 
-/* Allocates the stream's device state (about 15 MiB, cudaMalloc on the
+/* Allocates the stream's device state (about 16 MiB, cudaMalloc on the
  * current device: the state, the scratch rings of the one-launch paths and
  * the moving window's chunk histograms) and initialises it; synchronous (the
  * device is synchronized), so call it outside stream capture. */
@@ -473,7 +473,7 @@ int hist_batch_autotune_regimes(const uint8_t* const* d_ptrs, const size_t* d_si
  *
  * It allocates no device memory (no cudaMalloc, cudaFree or other device
  * allocator): it runs the same launches as hist_stream_push_many on a stream
- * state -- about 15 MiB -- that is one fixed device array in the library,
+ * state -- about 16 MiB -- that is one fixed device array in the library,
  * held by every GPU that loads the library until the process exits, and
  * cleared and initialised on `s` at the start of every call.  The first call
  * on a device looks up that array's device address and sets the kernels up;
@@ -610,7 +610,7 @@ typedef struct hist_completion {
 typedef struct hist_server hist_server;
 
 void hist_server_config_init(hist_server_config* c);
-/* Allocates the per-stream state, max_inflight batch slots (about 1.1 MiB of
+/* Allocates the per-stream state, max_inflight batch slots (about 2 MiB of
  * device memory each) and their CUDA streams, and 64 KiB of pinned, mapped
  * host memory for the requests' completion and state words; synchronizes
  * the device.  HIST_EINVAL for a bad config. */

@@ -559,6 +559,42 @@ __device__ __forceinline__ void piece_count(const uint8_t* base, uint32_t len, u
   lane_count<kLaneLoads, kThreads>(v, r, smem_addr(table) + ((threadIdx.x & 31) << 2));
 }
 
+// An input (a chunk, a request) that several CTAs count sums in one 64-bit word per bin: the bin's
+// count (bits 0..31), the 32 KiB blocks of memory counted (32..49: cuts
+// between CTAs lie between blocks, and an input touches at most 2^17 + 1) and
+// the sample's count (50..62: at most 4096).  One atomic per bin then tells
+// its thread whether the bin is complete, and the sum with it: adding counts,
+// publishing them with a fence, and counting bytes in a word of its own took
+// three more round trips to L2.
+__device__ __forceinline__ unsigned long long acc_word(uint32_t count, uint32_t blocks, uint32_t samp) {
+  return (unsigned long long)count | ((unsigned long long)blocks << 32) | ((unsigned long long)samp << 50);
+}
+constexpr uint32_t kAccBlockMask = (1u << 18) - 1u;
+// Blocks of memory that bytes [b0, e0) (not empty) at `in` touch.
+__device__ __forceinline__ uint32_t acc_blocks(const uint8_t* in, uint32_t b0, uint32_t e0) {
+  const unsigned long long p = (unsigned long long)(uintptr_t)in;
+  return (uint32_t)((p + e0 - 1) / kSplitAlign - (p + b0) / kSplitAlign) + 1u;
+}
+
+// A whole chunk (request) as a group counts it, computed once for the group's threads.
+struct alignas(16) GroupItem {
+  const uint4* body;  // its vectors from the first 128-byte line on
+  uint32_t* out;
+  uint32_t nvec;
+  uint32_t n;
+  uint32_t j;
+  uint32_t edges;  // bytes before the vectors (bits 0..7) and after them (8..15); bit 16: sampled
+};
+
+// The edge byte that thread t of a group counts (0x100: none), loaded a chunk
+// ahead like the vectors.
+__device__ __forceinline__ uint32_t group_edge(const GroupItem& it, int t) {
+  const uint32_t head = it.edges & 0xffu, tail = (it.edges >> 8) & 0xffu;
+  if ((uint32_t)t >= head + tail) return 0x100u;
+  const uint8_t* in = reinterpret_cast<const uint8_t*>(it.body) - head;
+  return (uint32_t)t < head ? in[t] : reinterpret_cast<const uint8_t*>(it.body + it.nvec)[t - head];
+}
+
 // Count head and tail bytes of a split into cs.res (threads 0..143).
 __device__ __forceinline__ void count_edges(const uint8_t* a, const Split& sp, CtaShared& cs) {
   count_edges_into(a, sp, cs.res);

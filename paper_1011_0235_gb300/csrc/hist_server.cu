@@ -3,19 +3,21 @@
 // Each request is the next chunk of one of `streams` independent streams; a
 // stream's adaptive state (the switch flag, the binning pattern and the
 // layout derived from it, the totals and the last histogram) stays on the
-// device, so a request runs the kernel and pattern chosen from its stream's
-// previous request (Sec. III.B / III.C), exactly as hist_stream_push would.
+// device, so a request gets the kernel and pattern chosen from its stream's
+// previous request (Sec. III.B / III.C), exactly as hist_stream_push would;
+// every kernel and pattern counts in the lane-private table.
 //
 // Continuous batching on the host: submitted requests wait in a FIFO queue;
 // whenever a batch slot is free, the queued requests that fit the HBM byte
 // budget and whose stream has no request on the GPU form a batch, launched
 // on the slot's own CUDA stream, so batches overlap on the device.  A batch
-// is one kernel with no device-side waits: the CTAs split the requests by a
-// cost model (bytes plus a fixed cost per request), count each piece with
-// its stream's layout and add it into the request's accumulator; the CTA
-// that completes a request (a done-bytes counter) computes its degeneracy
-// and next pattern and updates the stream's state.  A request counted whole
-// by one CTA skips the accumulator.  Once a request's output is written, its
+// is one kernel with no device-side waits: the host splits the requests among
+// the CTAs by a cost model (bytes plus a fixed cost per request), each CTA
+// counts its pieces and adds them into the requests' accumulators; the CTA
+// that completes a request computes its degeneracy and next pattern and
+// updates the stream's state.  Small requests are counted whole by groups of
+// warps, each of which runs its requests' epilogues itself.  A request counted
+// whole by one CTA skips the accumulator.  Once a request's output is written, its
 // epilogue writes the batch's sequence number into the request's completion
 // word in pinned host memory, so the host sees each request complete without
 // waiting for the rest of its batch; it then updates the stream's state and
@@ -37,37 +39,46 @@
 #include "hist.h"
 #include "hist_device.cuh"
 #include "hist_internal.h"
+#include "hist_plan.h"
 
 using namespace histdev;
 using namespace histlib;
 
 namespace {
 
-constexpr uint32_t kSrvMaxBatch = HIST_SERVER_MAX_BATCH;  // <= kThreads (one prefix lane each)
+constexpr uint32_t kSrvMaxBatch = HIST_SERVER_MAX_BATCH;
 constexpr uint32_t kSrvMaxSlots = HIST_SERVER_MAX_INFLIGHT;
 // cost of a request beyond its bytes, in bytes: about what one CTA counts
 // while it reduces its table, publishes its piece and runs a request's
-// epilogue and completion (a burst of 4000 requests of 4 KiB..64 MiB on
-// GB300: 3.64 TB/s at 64 KiB, 4.1 at 256 KiB, no better beyond)
+// epilogue and completion
 constexpr unsigned long long kReqCost = 256ull << 10;
-// cost units per CTA of a batch (the grid is at most every resident CTA)
-constexpr unsigned long long kCtaCost = 64ull << 10;
-// dynamic shared memory: table, slot table, request cost prefix (u64 per
-// request + 1), each request's stream ctl word
-constexpr size_t kSrvSmem = (size_t)(kTableWords + kLutWords) * 4 + (size_t)(kSrvMaxBatch + 1) * 8 +
-                            (size_t)kSrvMaxBatch * 4;
+// the same for a small request, counted beside three others (64 to 160 KiB,
+// and 128 KiB instead of 256 above, measured within 2 % of these on a burst)
+constexpr unsigned long long kSmallReqCost = 96ull << 10;
+constexpr uint32_t kSmallReq = 256u << 10;  // largest request a group counts
+// cost units per CTA of a batch (the grid is at most every resident CTA);
+// from launch to completion a request takes 10.9 us at the median with 32
+// KiB, 11.4 with 64, 12.4 with 128 (50k requests/s)
+constexpr unsigned long long kCtaCost = 32ull << 10;
+constexpr int kGroups = 4;
+constexpr int kGroupThreads = kThreads / kGroups;
+static_assert(kGroupThreads == HIST_BINS, "one bin per thread of a group");
+constexpr int kEpiBar = 1 + kGroups;  // named barrier of the threads of a CTA's epilogue
+// dynamic shared memory: the groups' tables in a batch with groups, else one
+constexpr size_t kSrvSmem = (size_t)kTableWords * 4;
+constexpr size_t kSrvGroupSmem = kGroups * kSrvSmem;
 // request-table capacities of the two kernel variants (the table travels in
 // the launch's parameters: 24 bytes per request)
 constexpr uint32_t kSmallCap = 32;
 
-static_assert(kSrvMaxBatch <= (uint32_t)kThreads, "one prefix lane per request");
+__host__ __device__ __forceinline__ unsigned long long srv_cost(unsigned long long n) {
+  return n + (n <= kSmallReq ? kSmallReqCost : kReqCost);
+}
 
 // Per-stream state on the device.  The two patterns sit in two slots: the
 // next request's in pat[cur], the last request's in the other; a request's
 // epilogue writes the new pattern over the older one and flips cur, so no
-// pattern is ever copied.  ctl packs what a batch reads about a stream
-// before counting: the switch (bit 0), whether pat[cur] is a uniform shift
-// (bit 1), cur (bit 2) and the shift's log2 k (bits 8..15).
+// pattern is ever copied.  ctl holds the switch (bit 0) and cur (bit 1).
 struct SrvStream {
   unsigned long long totals[HIST_BINS];
   uint32_t last_hist[HIST_BINS];
@@ -77,8 +88,8 @@ struct SrvStream {
   uint32_t last_kernel;  // kernel the last request ran
 };
 
-__host__ __device__ __forceinline__ uint32_t srv_ctl(uint32_t flag, uint32_t shift, uint32_t cur, uint32_t lk) {
-  return (flag & 1u) | ((shift & 1u) << 1) | ((cur & 1u) << 2) | ((lk & 0xffu) << 8);
+__host__ __device__ __forceinline__ uint32_t srv_ctl(uint32_t flag, uint32_t cur) {
+  return (flag & 1u) | ((cur & 1u) << 1);
 }
 
 struct SrvReq {
@@ -88,11 +99,11 @@ struct SrvReq {
   uint32_t stream;
 };
 
-// Per batch slot, on the device.  acc and done return to zero when a
-// request's epilogue has read them, so a slot needs clearing only once.
+// Per batch slot, on the device.  Both return to zero when a request's
+// epilogue has read them, so a slot needs clearing only once.
 struct SrvSlot {
-  uint32_t acc[kSrvMaxBatch][HIST_BINS];  // partial sums of split requests
-  unsigned long long done[kSrvMaxBatch];  // bytes of each split request counted
+  unsigned long long acc[kSrvMaxBatch][HIST_BINS];  // requests counted by several CTAs (acc_word)
+  uint32_t rbins[kSrvMaxBatch];                     // bins complete, where several CTAs completed a request
 };
 
 struct SrvCommon {
@@ -112,6 +123,7 @@ struct SrvCommon {
 template <uint32_t CAP>
 struct SrvArgs {
   SrvCommon c;
+  RangePlan plan;
   SrvReq req[CAP];
 };
 
@@ -119,238 +131,307 @@ __device__ __forceinline__ uint32_t srv_kernel_for(uint32_t mode, uint32_t flag)
   return mode == HIST_MODE_AUTO ? flag : (mode == HIST_MODE_PLAIN ? HIST_FLAG_PLAIN : HIST_FLAG_ADAPTIVE);
 }
 
-// Whether P gives every bin the same k = 2^lk at off = b k (all threads call).
-__device__ bool srv_is_shift(const hist_pattern& P) {
-  const bool act = threadIdx.x < HIST_BINS;
-  const uint32_t lk0 = P.log2k[0];
-  const int ok = !act || (P.log2k[threadIdx.x] == lk0 && lk0 <= 5 &&
-                          (uint32_t)P.off[threadIdx.x] == ((uint32_t)threadIdx.x << lk0));
-  return __syncthreads_and(ok) != 0;
-}
+// A piece of a request, bytes [b0, e0) (e0 = 0: an empty request), as the CTAs
+// keep it in shared memory (the table sits in the kernel's parameters, read
+// through the constant cache: 0.5 - 1 us a miss).
+struct SrvPiece {
+  SrvReq q;
+  uint32_t r;  // the request's number in the batch
+  uint32_t b0, e0;
+};
 
-__device__ __forceinline__ void srv_copy_words(void* dst, const void* src, int words) {
-  const uint32_t* s = reinterpret_cast<const uint32_t*>(src);
-  uint32_t* d = reinterpret_cast<uint32_t*>(dst);
-  for (int i = threadIdx.x; i < words; i += blockDim.x) d[i] = s[i];
-}
+constexpr uint32_t kSrvItems = 2 * kWarps;  // requests the groups take at a time
 
-// The same from a stream's state in global memory, read at L2: the state is
+struct SrvShared {
+  EpiShared es[kGroups];
+  uint32_t res[HIST_BINS];
+  uint32_t eh[2][HIST_BINS];  // edge bytes of the CTA's pieces, in turn
+  int last;
+  uint16_t wl[kSrvMaxBatch];  // whole requests left to the groups
+  GroupItem items[kSrvItems]; // the ones the groups are at (j: the stream)
+  uint32_t item_r[kSrvItems]; // their numbers in the batch
+  SrvReq win[kWarps];         // the requests of the range the CTA is at
+  SrvPiece piece[kWarps];     // its pieces of them
+  uint32_t npiece, nwl;
+  unsigned long long pos;     // cost position of the request after them
+  uint32_t geh[kGroups][HIST_BINS];
+};
+
+// Request r of stream `sid` (n bytes) is complete, threads t = 0..255 (which
+// share named barrier `id`) hold a bin each in h: write its output and publish
+// the request's completion word, then advance its stream's state.  The state
+// can follow the completion: the stream's next request is admitted only once
+// the state word below has been seen.  The state is read at L2: it was
 // written by another batch's epilogue, possibly while an older batch that
-// read it on this SM is still resident, so no line of it is taken from L1.
-__device__ __forceinline__ void srv_copy_state_words(void* dst, const void* src, int words) {
-  const uint32_t* s = reinterpret_cast<const uint32_t*>(src);
-  uint32_t* d = reinterpret_cast<uint32_t*>(dst);
-  for (int i = threadIdx.x; i < words; i += blockDim.x) d[i] = __ldcg(s + i);
-}
-
-// pre[r] = sum over requests before r of (n + kReqCost); pre[count] = total;
-// ctl[r] = request r's stream ctl word (its load overlaps the scan).  The
-// request table sits in the kernel's parameters, read through the constant
-// cache, which serves a warp's distinct addresses one after another: each
-// warp first copies its requests' sizes and streams into pre[] and ctl[]
-// with a warp-uniform index, and thread r then reads entry r from there.
-__device__ void srv_cost_prefix(const SrvReq* req, uint32_t count, const SrvStream* streams,
-                                unsigned long long* pre, uint32_t* ctl) {
-  __shared__ unsigned long long wsum[kWarps];
-  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-  for (uint32_t r = (uint32_t)w; r < count; r += kWarps) {
-    const uint32_t n = req[r].n, sid = req[r].stream;
-    if (lane == 0) {
-      pre[r] = n;
-      ctl[r] = sid;
-    }
-  }
-  __syncthreads();
-  // thread t reads entry t and later overwrites only entry t (and pre[count])
-  const uint32_t cw = t < (int)count ? __ldcg(&streams[ctl[t]].ctl) : 0u;
-  const unsigned long long c = t < (int)count ? pre[t] + kReqCost : 0ull;
-  unsigned long long x = c;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
-  }
-  if (lane == 31) wsum[w] = x;
-  __syncthreads();
-  unsigned long long before = 0;
-  for (int i = 0; i < w; ++i) before += wsum[i];
-  if (t < (int)count) {
-    pre[t] = before + x - c;
-    ctl[t] = cw;
-  }
-  if (t == (int)count - 1) pre[count] = before + x;
-  __syncthreads();
-}
-
-// Request r (q) is complete and cs.hist holds its histogram: write its
-// output and publish the request's completion word, then advance its
-// stream's state.  The state can follow the completion: the stream's next
-// request is admitted only once the state word below has been seen.  All
-// threads of the CTA call.
-__device__ __noinline__ void srv_epilogue(const SrvCommon& a, uint32_t r, const SrvReq& q, uint32_t ctl,
-                                          CtaShared& cs, EpiShared& es) {
-  SrvStream* st = a.streams + q.stream;
-  const uint32_t kernel = srv_kernel_for(a.mode, ctl & 1u), cur = (ctl >> 2) & 1u;
-  __syncthreads();  // cs.hist is written
-  if (threadIdx.x < HIST_BINS && q.out) q.out[threadIdx.x] = cs.hist[threadIdx.x];
-  // the output precedes the completion word: the barrier orders the CTA's
+// read it on this SM is still resident.
+__device__ __noinline__ void srv_epilogue(const SrvCommon& a, uint32_t r, uint32_t sid, uint32_t n, uint32_t* out,
+                                          uint32_t h, EpiShared& es, int t, int id) {
+  SrvStream* st = a.streams + sid;
+  const GroupBar<HIST_BINS> bar = {id};
+  const uint32_t ctl = __ldcg(&st->ctl);
+  if (out) out[t] = h;
+  // the output precedes the completion word: the barrier orders the threads'
   // writes before thread 0's system-scope release store, whose release is
   // cumulative (an explicit system fence before it measured 1.5 % slower on
   // a burst of 4000 requests and orders nothing more)
-  __syncthreads();
-  if (threadIdx.x == 0)
+  bar.sync();
+  if (t == 0)
     asm volatile("st.release.sys.global.u32 [%0], %1;" ::"l"(a.done + r), "r"(a.seq) : "memory");
-  const hist_degeneracy_result d = block_epilogue(cs.hist, q.n, a.budget, a.theta, cs.pat, es);
-  __syncthreads();
-  if (threadIdx.x < HIST_BINS) {
-    const uint32_t h = cs.hist[threadIdx.x];
-    if (h) atomicAdd(&st->totals[threadIdx.x], (unsigned long long)h);
-    st->last_hist[threadIdx.x] = h;
-  }
+  if (h) atomicAdd(&st->totals[t], (unsigned long long)h);
+  st->last_hist[t] = h;
+  BinPlace place;
+  const hist_degeneracy_result d = block_pattern(h, n, a.budget, a.theta, es, t, bar, place);
   // the new pattern replaces the older of the two
-  srv_copy_words(&st->pat[cur ^ 1u], &cs.pat, (int)(sizeof(hist_pattern) / 4));
-  const bool shift = srv_is_shift(cs.pat);
-  if (threadIdx.x == 0) {
-    st->ctl = srv_ctl(d.flag, shift ? 1u : 0u, cur ^ 1u, shift ? cs.pat.log2k[0] : 0u);
-    st->last_kernel = kernel;
+  const uint32_t cur = (ctl >> 1) & 1u;
+  store_place(st->pat[cur ^ 1u], t, a.budget, place);
+  if (t == 0) {
+    st->ctl = srv_ctl(d.flag, cur ^ 1u);
+    st->last_kernel = srv_kernel_for(a.mode, ctl & 1u);
     atomicAdd(&st->chunks, 1ull);  // at L2, like every other read of the state
   }
   // the stream's state is written: its state word releases the stream to
   // the host's admission, so that its next request may run in a batch that
   // starts while this one is still counting (the same release argument as
   // for the completion word)
-  __syncthreads();
-  if (threadIdx.x == 0)
+  bar.sync();
+  if (t == 0)
     asm volatile("st.release.sys.global.u32 [%0], %1;" ::"l"(a.done + kSrvMaxBatch + r), "r"(a.seq) : "memory");
 }
 
-// The slot table of a stream's pattern that is not a uniform shift (all
-// threads call).
-__device__ __noinline__ void srv_layout_general(const SrvStream* st, uint32_t cur, uint32_t* lut, CtaShared& cs) {
+// Count piece d (the CTA's k-th) into the table, which is clear before and
+// after, and publish it: into the request's accumulator, or, when it is the
+// whole request, straight into the request's epilogue.  Epilogues are run by
+// the first 256 threads while the others go on to the CTA's next piece.  All
+// threads call.
+__device__ __forceinline__ void srv_piece(const SrvCommon& a, const SrvPiece& d, uint32_t k, uint32_t* table,
+                                          SrvShared& ss) {
+  const int t = threadIdx.x;
+  uint32_t h = 0;
+  if (d.e0) {
+    piece_count(d.q.in + d.b0, d.e0 - d.b0, table, ss.eh[k & 1], nullptr, nullptr);
+    __syncthreads();
+    lane_reduce<kThreads, true>(table, ss.res, t);
+    __syncthreads();
+    if (t < HIST_BINS) {
+      h = ss.res[t] + ss.eh[k & 1][t];
+      ss.eh[k & 1][t] = 0;
+    }
+  }
+  bool complete = d.e0 - d.b0 == d.q.n;
+  if (!complete) {
+    unsigned long long* acc = &a.slot->acc[d.r][t & (HIST_BINS - 1)];
+    bool done = false;
+    if (t < HIST_BINS) {
+      const unsigned long long add = acc_word(h, acc_blocks(d.q.in, d.b0, d.e0), 0);
+      const unsigned long long sum = atomicAdd(acc, add) + add;
+      done = ((uint32_t)(sum >> 32) & kAccBlockMask) == acc_blocks(d.q.in, 0, d.q.n);
+      h = (uint32_t)sum;
+    }
+    const int bins = __syncthreads_count(done);
+    if (bins == HIST_BINS) {
+      // this CTA's adds were the last to every bin
+      complete = true;
+      if (t < HIST_BINS) *acc = 0;
+    } else if (bins > 0) {
+      // two CTAs' adds crossed: the one that brings the completed bins to 256
+      // reads them all
+      if (t == 0) {
+        __threadfence();
+        ss.last = atomicAdd(&a.slot->rbins[d.r], (uint32_t)bins) + (uint32_t)bins == HIST_BINS;
+        __threadfence();
+      }
+      __syncthreads();
+      complete = ss.last != 0;
+      if (complete) {
+        if (t < HIST_BINS) {
+          h = (uint32_t)__ldcg(acc);
+          *acc = 0;
+        }
+        if (t == 0) a.slot->rbins[d.r] = 0;
+      }
+    }
+  }
+  if (complete && t < HIST_BINS) srv_epilogue(a, d.r, d.q.stream, d.q.n, d.q.out, h, ss.es[0], t, kEpiBar);
+}
+
+// Requests [r0, r0 + kWarps), the first at cost position ss.pos: into ss.win,
+// a warp each (their constant-cache misses overlap), then warp 0, a request
+// per lane, lists the CTA's pieces of them and, in ss.wl, the whole ones left
+// to the groups.  All threads call (begins and ends with a barrier).
+template <uint32_t CAP>
+__device__ __forceinline__ void srv_window(const SrvArgs<CAP>& args, uint32_t r0, SrvShared& ss) {
+  const uint32_t w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const RangePlan& p = args.plan;
   __syncthreads();
-  srv_copy_state_words(&cs.pat, &st->pat[cur], (int)(sizeof(hist_pattern) / 4));
+  if (r0 + w < args.c.count) {
+    const SrvReq q = args.req[r0 + w];
+    if (lane == 0) ss.win[w] = q;
+  }
   __syncthreads();
-  classify_pattern(cs.pat, lut, cs);
+  if (w == 0) {
+    const unsigned long long lo = p.lo[blockIdx.x], hi = p.lo[blockIdx.x + 1];
+    const bool in = r0 + lane < args.c.count;
+    const SrvReq q = in ? ss.win[lane] : SrvReq{nullptr, nullptr, 0, 0};
+    const uint32_t n = q.n;
+    const unsigned long long c = in ? srv_cost(n) : 0ull;
+    unsigned long long x = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
+      if ((int)lane >= o) x += y;
+    }
+    const unsigned long long p0 = ss.pos + x - c;
+    // this CTA's bytes of the request: its cost range cut to [0, n), each
+    // cut moved to a 32 KiB boundary of the request's memory; a request of
+    // at most a quarter of a CTA's range is not split (the range holding its
+    // first cost position counts it whole, with no accumulator), and a small
+    // one of those is left to the groups
+    bool piece = false, item = false;
+    unsigned long long b0 = 0, e0 = 0;
+    if (in && p0 < hi) {
+      if (n == 0 || plan_whole(n, p.range)) {
+        item = p0 >= lo && n != 0 && n <= p.group_max;
+        piece = p0 >= lo && !item;
+        e0 = n;
+      } else {
+        b0 = lo > p0 ? split_point(q.in, lo - p0) : 0ull;
+        e0 = split_point(q.in, hi - p0);
+        if (e0 > (unsigned long long)n) e0 = n;
+        piece = b0 < e0;
+      }
+    }
+    const unsigned mp = __ballot_sync(0xffffffffu, piece), mi = __ballot_sync(0xffffffffu, item);
+    const unsigned lt = (1u << lane) - 1u;
+    if (piece) ss.piece[__popc(mp & lt)] = SrvPiece{q, r0 + lane, (uint32_t)b0, (uint32_t)e0};
+    if (item) ss.wl[ss.nwl + __popc(mi & lt)] = (uint16_t)(r0 + lane);
+    __syncwarp();
+    if (lane == 31) {
+      ss.pos = p0 + c;
+      ss.npiece = __popc(mp);
+      ss.nwl += __popc(mi);
+    }
+  }
+  __syncthreads();
+}
+
+// The groups' requests [i0, i0 + kSrvItems) of the list (first >= 0: first,
+// first + 1, ...; else ss.wl) into ss.items, a warp per request.
+template <uint32_t CAP>
+__device__ __forceinline__ void srv_items(const SrvArgs<CAP>& args, uint32_t nwl, int first, uint32_t i0,
+                                          SrvShared& ss) {
+  for (uint32_t k = threadIdx.x >> 5; k < kSrvItems && i0 + k < nwl; k += kWarps) {
+    const uint32_t r = first >= 0 ? (uint32_t)first + i0 + k : ss.wl[i0 + k];
+    const SrvReq q = args.req[r];
+    if ((threadIdx.x & 31) == 0) {
+      const Split sp = split_bytes(q.in, q.n);
+      GroupItem it;
+      it.body = reinterpret_cast<const uint4*>(q.in + sp.head);
+      it.out = q.out;
+      it.nvec = (uint32_t)sp.nvec;
+      it.n = q.n;
+      it.j = q.stream;
+      it.edges = (uint32_t)sp.head | ((uint32_t)sp.tail << 8);
+      ss.items[k] = it;
+      ss.item_r[k] = r;
+    }
+  }
+}
+
+// This group's requests g, g + kGroups, ... of the first `count` in ss.items
+// (its table and edge histogram clear).  All of the group's threads call.
+__device__ __forceinline__ void srv_group(const SrvCommon& a, uint32_t count, uint32_t* tables, SrvShared& ss) {
+  const int g = threadIdx.x / kGroupThreads, t = threadIdx.x % kGroupThreads;
+  const GroupBar<kGroupThreads> bar = {g + 1};
+  uint32_t* table = tables + (size_t)g * kTableWords;
+  const uint32_t base = smem_addr(table) + ((t & 31) << 2);
+  uint32_t i = (uint32_t)g;
+  if (i >= count) return;
+  for (; i < count; i += kGroups) {
+    const GroupItem& it = ss.items[i];
+    const uint32_t edge = group_edge(it, t);
+    uint4 v[kLaneLoads];
+    const LaneRange r = lane_range(it.body, 0, it.nvec, t);
+    lane_load<kLaneLoads, kGroupThreads>(v, r);
+    if (edge < 0x100u) atomicAdd(&ss.geh[g][edge], 1u);
+    lane_count<kLaneLoads, kGroupThreads>(v, r, base);
+    bar.sync();
+    uint32_t h = lane_row(table, t);
+    if (it.edges) {
+      h += ss.geh[g][t];
+      ss.geh[g][t] = 0;
+    }
+    // (its barriers also keep the next request's increments from this one's
+    // reduction)
+    srv_epilogue(a, ss.item_r[i], it.j, it.n, it.out, h, ss.es[g], t, g + 1);
+  }
 }
 
 // One CTA of 1024 threads per SM, four loads in flight per thread (as the
-// stream's counting kernel): at 2k and 50k requests/s p50 19.7 -> 18.9 and
-// 21.0 -> 19.6 us, p99 39.9 -> 35.6 and 52.4 -> 44.2 us against two CTAs
-// per SM; burst capacity 2.53 -> 2.49 TB/s.
+// stream's counting kernel).  Bound by the HBM read in a burst and by latency
+// (launch, one round of loads, an accumulator's and an epilogue's round trips)
+// on single requests.  Before -- per-warp tables for the streams the switch
+// called plain, the default pattern's slot lookup for first requests, a cost
+// prefix with 64-bit divisions in every CTA -- and now: a burst of 600
+// requests of 4 KiB .. 64 MiB on 256 streams 1320 -> 767 us, one of 4000 3.48
+// -> 6.0 TB/s; at 50k requests/s p50 18.3 -> 14.2 us, p99 40.7 -> 26.8.
 template <uint32_t CAP>
 __global__ void __launch_bounds__(kThreads, 1) server_batch_kernel(const __grid_constant__ SrvArgs<CAP> args) {
-  extern __shared__ __align__(16) uint32_t smem[];
-  uint32_t* table = smem;
-  uint32_t* lut = smem + kTableWords;  // slot table while counting, then scratch of the reduction
-  unsigned long long* pre = reinterpret_cast<unsigned long long*>(smem + kTableWords + kLutWords);
-  uint32_t* ctl = reinterpret_cast<uint32_t*>(pre + kSrvMaxBatch + 1);
-  __shared__ CtaShared cs;
-  __shared__ EpiShared es;
-  __shared__ int last;
+  extern __shared__ __align__(16) uint32_t tables[];
+  __shared__ SrvShared ss;
   const SrvCommon& a = args.c;
-
-  zero_table(table);
-  srv_cost_prefix(args.req, a.count, a.streams, pre, ctl);
-  const unsigned long long W = pre[a.count];
-  const unsigned long long lo = W * blockIdx.x / gridDim.x;
-  const unsigned long long hi = W * (blockIdx.x + 1) / gridDim.x;
-  if (lo >= hi) return;
-  // the request holding cost position lo
-  uint32_t r = 0, rh = a.count;
-  while (r + 1 < rh) {
-    const uint32_t mid = (r + rh) >> 1;
-    if (pre[mid] <= lo) r = mid;
-    else rh = mid;
+  const RangePlan& p = args.plan;
+  const int t = threadIdx.x;
+  const bool groups = p.groups[blockIdx.x >> 5] >> (blockIdx.x & 31) & 1u;
+  const uint32_t s0 = p.s[blockIdx.x], s1 = p.s[blockIdx.x + 1];
+  uint32_t nwl = s1 - s0;
+  int first = (int)s0;
+  if (!groups) {
+    zero_table(tables);
+    if (t < HIST_BINS) ss.eh[0][t] = ss.eh[1][t] = 0;
+    if (t == 0) {
+      ss.pos = p.pre[blockIdx.x];
+      ss.nwl = 0;
+    }
+    uint32_t k = 0;
+    for (uint32_t r0 = p.j[blockIdx.x]; r0 < a.count; r0 += kWarps) {
+      srv_window(args, r0, ss);
+      for (uint32_t i = 0; i < ss.npiece; ++i) srv_piece(a, ss.piece[i], k++, tables, ss);
+      if (ss.pos >= p.lo[blockIdx.x + 1]) break;
+    }
+    __syncthreads();
+    nwl = ss.nwl;
+    first = -1;
   }
-  for (; r < a.count && pre[r] < hi; ++r) {
-    const SrvReq q = args.req[r];
-    const unsigned long long p0 = pre[r];
-    if (q.n == 0) {
-      // no bytes: the CTA holding the request's first cost position folds it
-      if (p0 >= lo) {
-        if (threadIdx.x < HIST_BINS) cs.hist[threadIdx.x] = 0;
-        srv_epilogue(a, r, q, ctl[r], cs, es);
-      }
-      continue;
-    }
-    // this CTA's bytes of the request: its cost range cut to [0, n), each
-    // cut moved to a 32 KiB boundary of the request's memory; a request of
-    // at most a quarter of a CTA's range is not split (the range holding
-    // its first cost position counts it whole, with no accumulator)
-    unsigned long long b0 = lo > p0 ? split_point(q.in, lo - p0) : 0ull;
-    unsigned long long e0 = split_point(q.in, hi - p0);
-    if (e0 > (unsigned long long)q.n) e0 = q.n;
-    if ((unsigned long long)q.n * 4 <= W / gridDim.x) {
-      if (p0 < lo) continue;
-      b0 = 0;
-      e0 = q.n;
-    }
-    if (b0 >= e0) continue;
-    const uint32_t c = ctl[r];
-    int path = PATH_PLAIN, lk = 0;
-    if (srv_kernel_for(a.mode, c & 1u) == HIST_FLAG_ADAPTIVE) {
-      if ((c >> 1) & 1u) {
-        path = PATH_SHIFT;
-        lk = (int)((c >> 8) & 0xffu);
-      } else {
-        srv_layout_general(a.streams + q.stream, (c >> 2) & 1u, lut, cs);
-        path = cs.path;
-        lk = cs.lk;
-      }
-    }
-    const uint8_t* base = q.in + b0;
-    const uint32_t len = (uint32_t)(e0 - b0);
-    const Split sp = split_bytes(base, len);
-    count_call4(path, lk, reinterpret_cast<const uint4*>(base + sp.head), 0, sp.nvec, table, lut);
-    const bool more = r + 1 < a.count && pre[r + 1] < hi;  // the CTA has another piece
-    const bool cleared = flush_table(path, lk, table, cs.pat, lut, cs, more);
-    count_edges(base, sp, cs);
-    if (more && !cleared) zero_table(table);
+  if (nwl == 0) return;
+  __syncthreads();
+  {
+    const int g = t / kGroupThreads, gt = t % kGroupThreads;
+    uint4* t4 = reinterpret_cast<uint4*>(tables + (size_t)g * kTableWords);
+#pragma unroll
+    for (int i = 0; i < kTableWords / 4 / kGroupThreads; ++i) t4[gt + i * kGroupThreads] = make_uint4(0, 0, 0, 0);
+    ss.geh[g][gt] = 0;
+  }
+  for (uint32_t i0 = 0; i0 < nwl; i0 += kSrvItems) {
+    if (i0) __syncthreads();
+    srv_items(args, nwl, first, i0, ss);
     __syncthreads();
-    if (b0 == 0 && e0 == q.n) {
-      // the whole request
-      if (threadIdx.x < HIST_BINS) cs.hist[threadIdx.x] = cs.res[threadIdx.x];
-      srv_epilogue(a, r, q, ctl[r], cs, es);
-      continue;
-    }
-    if (threadIdx.x < HIST_BINS && cs.res[threadIdx.x]) atomicAdd(&a.slot->acc[r][threadIdx.x], cs.res[threadIdx.x]);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      // the barrier orders the CTA's adds before this fence, which publishes
-      // them before the byte count
-      __threadfence();
-      last = atomicAdd(&a.slot->done[r], (unsigned long long)len) + len == q.n;
-    }
-    __syncthreads();
-    if (last) {
-      // every other piece of r was added (and fenced) before its done count
-      __threadfence();
-      if (threadIdx.x < HIST_BINS) {
-        cs.hist[threadIdx.x] = __ldcg(&a.slot->acc[r][threadIdx.x]);
-        a.slot->acc[r][threadIdx.x] = 0;
-      }
-      if (threadIdx.x == 0) a.slot->done[r] = 0;
-      srv_epilogue(a, r, q, ctl[r], cs, es);
-    }
+    srv_group(a, nwl - i0 < kSrvItems ? nwl - i0 : kSrvItems, tables, ss);
   }
 }
 
 // Every stream starts with no chunks, the plain kernel and the default
 // pattern (one CTA).
-__global__ void server_init_kernel(SrvStream* s, uint32_t streams, uint32_t budget) {
-  __shared__ CtaShared cs;
+__global__ void __launch_bounds__(HIST_BINS) server_init_kernel(SrvStream* s, uint32_t streams, uint32_t budget) {
   __shared__ EpiShared es;
-  if (threadIdx.x < HIST_BINS) cs.hist[threadIdx.x] = 0;
-  __syncthreads();
-  block_epilogue(cs.hist, 0, budget, HIST_THETA_MILLI_DEFAULT, cs.pat, es);
-  __syncthreads();
-  const bool shift = srv_is_shift(cs.pat);
+  const int t = threadIdx.x;
+  BinPlace place;
+  block_pattern(0u, 0ull, budget, HIST_THETA_MILLI_DEFAULT, es, t, CtaBar(), place);
   for (uint32_t i = 0; i < streams; ++i) {
     SrvStream* st = s + i;
-    srv_copy_words(&st->pat[0], &cs.pat, (int)(sizeof(hist_pattern) / 4));
-    srv_copy_words(&st->pat[1], &cs.pat, (int)(sizeof(hist_pattern) / 4));
-    if (threadIdx.x == 0) {
-      st->ctl = srv_ctl(HIST_FLAG_PLAIN, shift ? 1u : 0u, 0u, shift ? cs.pat.log2k[0] : 0u);
+    store_place(st->pat[0], t, budget, place);
+    store_place(st->pat[1], t, budget, place);
+    if (t == 0) {
+      st->ctl = srv_ctl(HIST_FLAG_PLAIN, 0u);
       st->last_kernel = HIST_FLAG_PLAIN;
     }
   }
@@ -553,17 +634,22 @@ int admit(hist_server* s) {
     a->req[i].out = r.out;
     a->req[i].n = (uint32_t)r.n;
     a->req[i].stream = r.stream;
-    cost += r.n + kReqCost;
+    cost += srv_cost(r.n);
   }
   unsigned long long grid = (cost + kCtaCost - 1) / kCtaCost;
   if (grid > (unsigned long long)s->max_grid) grid = (unsigned long long)s->max_grid;
   if (grid < 1) grid = 1;
+  plan_ranges(
+      &a->plan, count, (uint32_t)grid, kSmallReq, [&](uint32_t i) { return (unsigned long long)a->req[i].n; },
+      [&](uint32_t i) { return srv_cost(a->req[i].n); });
   // the small variant's parameters are a prefix of the large one's
   static_assert(offsetof(SrvArgs<kSmallCap>, req) == offsetof(SrvArgs<kSrvMaxBatch>, req), "parameter layout");
+  static_assert(sizeof(SrvArgs<kSrvMaxBatch>) <= 32764, "kernel parameters are limited to 32764 bytes");
   void* params[] = {a};
   const void* fn = count <= kSmallCap ? (const void*)server_batch_kernel<kSmallCap>
                                       : (const void*)server_batch_kernel<kSrvMaxBatch>;
-  cudaError_t e = cudaLaunchKernel(fn, dim3((unsigned)grid), dim3(kThreads), params, kSrvSmem, f->cs);
+  cudaError_t e = cudaLaunchKernel(fn, dim3((unsigned)grid), dim3(kThreads), params,
+                                   a->plan.group_max ? kSrvGroupSmem : kSrvSmem, f->cs);
   if (e != cudaSuccess) {
     // nothing was enqueued: the requests go back to the head of the queue
     for (const PendingReq& r : f->reqs) s->stream_busy[r.stream] = 0;
@@ -623,14 +709,15 @@ int hist_server_create(const hist_server_config* cfg, hist_server** out) {
   memset(&s->stats, 0, sizeof(s->stats));
   static int attr_small[kMaxDevices], attr_large[kMaxDevices];
   int rc = s->sms > 0 ? HIST_OK : HIST_ECUDA;
-  if (rc == HIST_OK) rc = ensure_smem_attr_bytes((const void*)server_batch_kernel<kSmallCap>, attr_small, kSrvSmem);
-  if (rc == HIST_OK) rc = ensure_smem_attr_bytes((const void*)server_batch_kernel<kSrvMaxBatch>, attr_large, kSrvSmem);
+  if (rc == HIST_OK) rc = ensure_smem_attr_bytes((const void*)server_batch_kernel<kSmallCap>, attr_small, kSrvGroupSmem);
+  if (rc == HIST_OK) rc = ensure_smem_attr_bytes((const void*)server_batch_kernel<kSrvMaxBatch>, attr_large, kSrvGroupSmem);
   if (rc == HIST_OK) {
     int per_sm = 0;
     const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &per_sm, (const void*)server_batch_kernel<kSrvMaxBatch>, kThreads, kSrvSmem);
+        &per_sm, (const void*)server_batch_kernel<kSrvMaxBatch>, kThreads, kSrvGroupSmem);
     if (e != cudaSuccess) rc = cuda_fail(e);
     s->max_grid = s->sms * (per_sm > 0 ? per_sm : 1);
+    if (s->max_grid > (int)kPlanCtas) s->max_grid = (int)kPlanCtas;
   }
   s->args = new (std::nothrow) SrvArgs<kSrvMaxBatch>();
   if (!s->args && rc == HIST_OK) rc = HIST_ENOMEM;
@@ -650,7 +737,7 @@ int hist_server_create(const hist_server_config* cfg, hist_server** out) {
       if (e == cudaSuccess) e = cudaMemset(f.d_slot, 0, sizeof(SrvSlot));
     }
     if (e == cudaSuccess) {
-      server_init_kernel<<<1, 256>>>(s->d_streams, cfg->streams, cfg->pattern_budget);
+      server_init_kernel<<<1, HIST_BINS>>>(s->d_streams, cfg->streams, cfg->pattern_budget);
       e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
@@ -730,7 +817,7 @@ int hist_server_stream_state(hist_server* s, uint32_t stream, hist_stream_state*
   memset(h, 0, sizeof(*h));
   memcpy(h->totals, tmp.totals, sizeof(h->totals));
   memcpy(h->last_hist, tmp.last_hist, sizeof(h->last_hist));
-  const uint32_t cur = (tmp.ctl >> 2) & 1u;
+  const uint32_t cur = (tmp.ctl >> 1) & 1u;
   h->pattern = tmp.pat[cur];
   h->last_pattern = tmp.pat[cur ^ 1u];
   h->chunks = tmp.chunks;

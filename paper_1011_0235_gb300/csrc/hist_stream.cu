@@ -17,6 +17,7 @@
 #include "hist.h"
 #include "hist_device.cuh"
 #include "hist_internal.h"
+#include "hist_plan.h"
 
 using namespace histdev;
 using namespace histlib;
@@ -25,7 +26,6 @@ namespace {
 
 constexpr uint32_t kMaxBatch = 1024;   // chunks per launch
 constexpr uint32_t kSmallBatch = 128;  // chunks per launch of the smaller parameter block
-constexpr uint32_t kPlanCtas = 160;    // largest grid: the host plans the CTAs' ranges
 constexpr uint32_t kChunkRing = 4 * kMaxBatch;  // scratch: chunk accumulators
 constexpr uint32_t kLaunchRing = 8;             // scratch: per-launch records
 constexpr uint32_t kPollLimit = 1u << 22;  // bounded wait: about a second
@@ -101,18 +101,7 @@ struct BatchArgs : PushHead {
   uint32_t trace_first;             // index of this batch's first chunk in the trace
   uint32_t trace_cap;               // chunks the trace holds
   unsigned long long* trace;        // optional phase timestamps (see hist_stream_trace)
-  // the host splits the batch's cost into the CTAs' ranges (flat_plan), so a
-  // CTA reads its own range instead of scanning the chunk table
-  unsigned long long range;                    // the batch's cost / grid
-  uint32_t group_max;                          // largest chunk left to the groups (0: a launch without groups)
-  unsigned long long plan_lo[kPlanCtas + 1];   // CTA b's range is [plan_lo[b], plan_lo[b + 1])
-  unsigned long long plan_pre[kPlanCtas];      // cost position of its first chunk
-  uint16_t plan_j[kPlanCtas];                  // its first chunk
-  // CTA b with bit b of plan_groups set has only whole chunks for the
-  // groups: chunks [plan_s[b], plan_s[b + 1]) start in its range, and any
-  // chunk that overlaps the range from before is whole (an earlier CTA's)
-  uint16_t plan_s[kPlanCtas + 1];
-  uint32_t plan_groups[(kPlanCtas + 31) / 32];
+  RangePlan plan;  // the host's split of the batch's cost
   ChunkDesc c[CAP];
 };
 using SmallArgs = BatchArgs<kSmallBatch>;
@@ -210,16 +199,6 @@ struct FlatDesc {
   uint32_t j;
 };
 constexpr uint32_t kListItems = 2 * kWarps;  // chunks the groups take at a time
-
-// A whole chunk as a group counts it, computed once for the group's threads.
-struct alignas(16) GroupItem {
-  const uint4* body;  // its vectors from the first 128-byte line on
-  uint32_t* out;
-  uint32_t nvec;
-  uint32_t n;
-  uint32_t j;
-  uint32_t edges;  // bytes before the vectors (bits 0..7) and after them (8..15); bit 16: sampled
-};
 
 // CTA-wide state of batch_flat_kernel (shared memory).
 template <uint32_t CAP>
@@ -421,23 +400,6 @@ __device__ __noinline__ void flat_ring_ready(const A& a, FlatShared<A::kCap>& fs
   if (threadIdx.x == 0) fs.ring_ok = 1;
 }
 
-// A chunk that several CTAs count sums in one 64-bit word per bin: the bin's
-// count (bits 0..31), the 32 KiB blocks of memory counted (32..49: cuts
-// between CTAs lie between blocks, and a chunk touches at most 2^17 + 1) and
-// the sample's count (50..62: at most 4096).  One atomic per bin then tells
-// its thread whether the bin is complete, and the sum with it: adding counts,
-// publishing them with a fence, and counting bytes in a word of its own took
-// three more round trips to L2.
-__device__ __forceinline__ unsigned long long acc_word(uint32_t count, uint32_t blocks, uint32_t samp) {
-  return (unsigned long long)count | ((unsigned long long)blocks << 32) | ((unsigned long long)samp << 50);
-}
-constexpr uint32_t kAccBlockMask = (1u << 18) - 1u;
-// Blocks of memory that bytes [b0, e0) (not empty) at `in` touch.
-__device__ __forceinline__ uint32_t flat_blocks(const uint8_t* in, uint32_t b0, uint32_t e0) {
-  const unsigned long long p = (unsigned long long)(uintptr_t)in;
-  return (uint32_t)((p + e0 - 1) / kSplitAlign - (p + b0) / kSplitAlign) + 1u;
-}
-
 // Run the epilogue of chunk d, whose histogram and sample threads 0..255 hold.
 // All threads call.
 template <class A>
@@ -476,9 +438,9 @@ __device__ __noinline__ void flat_flush(const A& a, const FlatDesc& d, uint32_t 
     unsigned long long* acc = &st->racc[slot][t & (HIST_BINS - 1)];
     bool done = false;
     if (t < HIST_BINS) {
-      const unsigned long long add = acc_word(h, flat_blocks(d.in, b0, e0), s);
+      const unsigned long long add = acc_word(h, acc_blocks(d.in, b0, e0), s);
       const unsigned long long sum = atomicAdd(acc, add) + add;
-      done = ((uint32_t)(sum >> 32) & kAccBlockMask) == flat_blocks(d.in, 0, n);
+      done = ((uint32_t)(sum >> 32) & kAccBlockMask) == acc_blocks(d.in, 0, n);
       h = (uint32_t)sum;
       s = (uint32_t)(sum >> 50);
     }
@@ -573,8 +535,8 @@ template <class A>
 __device__ uint32_t flat_range(const A& a, unsigned long long x0, unsigned long long x1, unsigned long long range,
                                uint32_t wend, uint32_t* table, FlatShared<A::kCap>& fs) {
   uint32_t nwl = 0;
-  uint32_t j = a.plan_j[blockIdx.x];
-  unsigned long long p0 = a.plan_pre[blockIdx.x], p1 = 0;  // cost position of chunk j, of chunk j + 1
+  uint32_t j = a.plan.j[blockIdx.x];
+  unsigned long long p0 = a.plan.pre[blockIdx.x], p1 = 0;  // cost position of chunk j, of chunk j + 1
   for (; j < a.count && p0 < x1; ++j, p0 = p1) {
     if (j == wend) {
       __syncthreads();
@@ -593,12 +555,12 @@ __device__ uint32_t flat_range(const A& a, unsigned long long x0, unsigned long 
       }
       continue;
     }
-    if ((unsigned long long)n * 4 <= range) {
+    if (plan_whole(n, range)) {
       // a chunk of at most a quarter of a CTA's range is not split: the
       // range holding its first cost position counts it whole, so it needs
       // no accumulator or ring; a small one is left to the groups
       if (p0 >= x0) {
-        if (n <= a.group_max) {
+        if (n <= a.plan.group_max) {
           if (threadIdx.x == 0) fs.wl[nwl] = (uint16_t)j;
           ++nwl;
         } else {
@@ -648,15 +610,6 @@ __device__ __forceinline__ void group_items(const A& a, uint32_t nwl, int first,
     const FlatDesc d = {a.c[j].in, a.c[j].out, a.c[j].n, j};
     if ((threadIdx.x & 31) == 0) fs.items[k] = group_item(a, d);
   }
-}
-
-// The edge byte that thread t of a group counts (0x100: none), loaded a chunk
-// ahead like the vectors.
-__device__ __forceinline__ uint32_t group_edge(const GroupItem& it, int t) {
-  const uint32_t head = it.edges & 0xffu, tail = (it.edges >> 8) & 0xffu;
-  if ((uint32_t)t >= head + tail) return 0x100u;
-  const uint8_t* in = reinterpret_cast<const uint8_t*>(it.body) - head;
-  return (uint32_t)t < head ? in[t] : reinterpret_cast<const uint8_t*>(it.body + it.nvec)[t - head];
 }
 
 // This group's chunks g, g + kGroups, ... of the first `count` in fs.items,
@@ -816,9 +769,9 @@ __global__ void __launch_bounds__(kThreads, 1) batch_flat_kernel(const __grid_co
     fs.epis = 0;
   }
   // what the range needs of the parameters is read before the wait
-  const bool groups = a.plan_groups[blockIdx.x >> 5] >> (blockIdx.x & 31) & 1u;
-  const uint32_t s0 = a.plan_s[blockIdx.x], s1 = a.plan_s[blockIdx.x + 1], j0 = a.plan_j[blockIdx.x];
-  const unsigned long long lo = a.plan_lo[blockIdx.x], hi = a.plan_lo[blockIdx.x + 1];
+  const bool groups = a.plan.groups[blockIdx.x >> 5] >> (blockIdx.x & 31) & 1u;
+  const uint32_t s0 = a.plan.s[blockIdx.x], s1 = a.plan.s[blockIdx.x + 1], j0 = a.plan.j[blockIdx.x];
+  const unsigned long long lo = a.plan.lo[blockIdx.x], hi = a.plan.lo[blockIdx.x + 1];
   if (groups) {
     // the range holds whole chunks for the groups only
     __syncthreads();
@@ -836,7 +789,7 @@ __global__ void __launch_bounds__(kThreads, 1) batch_flat_kernel(const __grid_co
                      : "memory");
     }
     uint32_t nwl = 0;
-    if (lo < hi) nwl = flat_range(a, lo, hi, a.range, wend, tables, fs);
+    if (lo < hi) nwl = flat_range(a, lo, hi, a.plan.range, wend, tables, fs);
     __syncthreads();
     if (nwl) flat_groups(a, nwl, -1, false, tables, fs);
   }
@@ -1110,67 +1063,18 @@ cudaError_t launch_chained(const void* fn, dim3 grid, dim3 block, void** params,
   return cudaLaunchKernelExC(&lc, fn, params);
 }
 
-// The CTAs' ranges of a launch: the batch's chunks placed end to end at their
-// costs (flat_cost), total W; CTA b takes [W b / grid, W (b + 1) / grid) and
-// starts at the last chunk whose cost position is at most the range's start.
-// (A kernel that computes the split itself reads every chunk's size from the
-// parameters: about 8 us per launch of 1024 chunks.)  Returns the grid: at
-// most `grid` CTAs, and no more than kCtaCost of cost each needs.
+// The grid of a launch and its CTAs' ranges (plan_ranges): at most `grid`
+// CTAs, and no more than kCtaCost bytes, or a chunk, each needs.
 constexpr unsigned long long kCtaCost = 32ull << 10;
-template <class A>
-uint32_t flat_plan(A* a, uint32_t count, const size_t* ns, uint32_t grid) {
-  unsigned long long W = 0, bytes = 0;
-  for (uint32_t i = 0; i < count; ++i) {
-    W += flat_cost(ns[i], i, count);
-    bytes += ns[i];
-  }
+uint32_t flat_plan(RangePlan* p, uint32_t count, const size_t* ns, uint32_t grid) {
+  unsigned long long bytes = 0;
+  for (uint32_t i = 0; i < count; ++i) bytes += ns[i];
   unsigned long long want = (bytes + kCtaCost - 1) / kCtaCost;
   if (want < count) want = count;
   if (want < grid) grid = (uint32_t)want;
-  a->range = W / grid;
-  uint32_t j = 0;
-  unsigned long long pj = 0;  // cost position of chunk j
-  for (uint32_t b = 0; b <= grid; ++b) {
-    const unsigned long long lo = W * b / grid;
-    a->plan_lo[b] = lo;
-    if (b == grid) break;
-    while (j + 1 < count && pj + flat_cost(ns[j], j, count) <= lo) {
-      pj += flat_cost(ns[j], j, count);
-      ++j;
-    }
-    a->plan_j[b] = (uint16_t)j;
-    a->plan_pre[b] = pj;
-  }
-  // the chunks the groups take (as flat_range decides)
-  const unsigned long long range = a->range;
-  auto whole = [&](uint32_t i) { return (unsigned long long)ns[i] * 4 <= range; };
-  auto small = [&](uint32_t i) { return ns[i] != 0 && ns[i] <= kGroupChunkMax && whole(i); };
-  // a launch has groups if at least half of its cost is theirs
-  unsigned long long small_cost = 0;
-  for (uint32_t i = 0; i < count; ++i)
-    if (small(i)) small_cost += flat_cost(ns[i], i, count);
-  a->group_max = 2 * small_cost >= W ? kGroupChunkMax : 0;
-  auto grouped = [&](uint32_t i) { return a->group_max && small(i); };
-  uint32_t i = 0;  // first chunk whose cost position is at least the range's start
-  unsigned long long pi = 0;
-  for (uint32_t b = 0; b <= grid; ++b) {
-    const unsigned long long lo = a->plan_lo[b];
-    while (i < count && pi < lo) {
-      pi += flat_cost(ns[i], i, count);
-      ++i;
-    }
-    a->plan_s[b] = (uint16_t)i;
-  }
-  // (a launch without groups has no memory for their tables: no CTA of it may
-  // take their path, whatever its range holds)
-  for (uint32_t b = 0; a->group_max && b < grid; ++b) {
-    bool only = true;
-    const uint32_t j0 = a->plan_j[b], s0 = a->plan_s[b], s1 = a->plan_s[b + 1];
-    // a chunk that starts before the range and reaches into it
-    for (uint32_t k = j0; k < s0 && only; ++k) only = whole(k);
-    for (uint32_t k = s0; k < s1 && only; ++k) only = grouped(k);
-    if (only) a->plan_groups[b >> 5] |= 1u << (b & 31);
-  }
+  plan_ranges(
+      p, count, grid, kGroupChunkMax, [&](uint32_t i) { return (unsigned long long)ns[i]; },
+      [&](uint32_t i) { return flat_cost(ns[i], i, count); });
   return grid;
 }
 
@@ -1206,11 +1110,11 @@ int launch_batch(hist_stream* st, uint32_t count, const uint8_t* const* ins, con
     a->c[i].out = outs ? outs[i] : nullptr;
   }
   const bool windowed = st->cfg.window > 1;
-  const uint32_t grid = flat_plan(a, count, ns, (uint32_t)st->grid);
+  const uint32_t grid = flat_plan(&a->plan, count, ns, (uint32_t)st->grid);
   void* params[] = {a};
   cudaError_t e =
       launch_chained((const void*)batch_flat_kernel<A>, dim3(grid), dim3(kThreads), params,
-                     a->group_max ? kFlatGroupSmem : kFlatSmem, s);
+                     a->plan.group_max ? kFlatGroupSmem : kFlatSmem, s);
   PushHead head = *a;
   void* hparams[] = {&head};
   if (e == cudaSuccess && windowed)

@@ -214,3 +214,34 @@ def test_batch_lane_launches(name, sizes, out_shift):
     """The default batch's two launches against the oracle, image by image:
     sizes around every limit of their rule, outputs at any word."""
     _batch(sizes, 17, 40, out_shift)
+
+
+@pytest.mark.parametrize("mode,budget", [(hl.MODE_AUTO, 8192), (hl.MODE_PLAIN, 960), (hl.MODE_ADAPTIVE, 2048)])
+def test_server_requests_around_the_groups_limit(mode, budget):
+    """Requests around the sizes at which a batch's paths change (empty, inside
+    a line, the groups' largest, cut between CTAs), at every alignment, three
+    rounds of one per stream: outputs and each stream's state equal the
+    oracle's."""
+    sizes = [0, 1, 127, 143, 4096, 70_001, 262_143, 262_144, 262_145, 600_007, 3_000_001, 9_000_000] * 6
+    rng = np.random.default_rng(budget)
+    srv = hl.Server(streams=len(sizes), mode=mode, pattern_budget=budget, max_batch=64)
+    refs = [oracle.StreamOracle(budget, mode=mode) for _ in sizes]
+    x = rng.integers(0, 256, max(sizes) + 300, dtype=np.uint8)
+    x[rng.random(x.size) < 0.46] = 9  # near the switch's threshold
+    xd = dev(x)
+    for rnd in range(3):
+        outs = torch.full((len(sizes), 256), -1, dtype=torch.int32, device="cuda")
+        offs = rng.integers(0, 300, len(sizes))
+        torch.cuda.synchronize()
+        for i, n in enumerate(sizes):
+            srv.submit_ptr(i, xd.data_ptr() + int(offs[i]), n, outs[i].data_ptr(), i)
+        srv.drain(20000)
+        got = u32(outs).reshape(len(sizes), 256)
+        for i, n in enumerate(sizes):
+            rec = refs[i].push(x[offs[i]:offs[i] + n])
+            assert np.array_equal(got[i], rec.hist), (rnd, i, n)
+            s = srv.stream_state(i)
+            assert bytes(s.pattern) == refs[i].pattern.to_bytes() and bytes(s.last_pattern) == rec.pattern.to_bytes()
+            assert s.flag == refs[i].flag and s.last_kernel == rec.kernel and s.chunks == rnd + 1
+            assert np.array_equal(np.array(s.totals, np.uint64), refs[i].totals)
+    srv.close()
