@@ -134,7 +134,7 @@ int degeneracy_u64(const uint64_t* d_hist, uint32_t theta_milli, hist_degeneracy
  * in shared memory, no pattern, merged per bin.  The sub-histograms are one
  * per lane (32 of 256 bins, shared by the CTA's warps) rather than one per
  * warp: the same 32 KiB, and a warp's increments fall in 32 banks whatever
- * the pixels are (64 MiB of uniform pixels: 2.2 -> 4.6 TB/s).  The per-warp
+ * the pixels are (64 MiB of uniform pixels: 2.2 -> 5.1 TB/s).  The per-warp
  * layout itself is measured by hist_ablation without a pattern.  d_out:
  * uint32_t[256], overwritten.  n >= 2^32 -> HIST_EINVAL.  d_in may be null
  * only if n == 0. */

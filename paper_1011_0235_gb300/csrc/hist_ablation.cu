@@ -38,6 +38,17 @@ using namespace histlib;
 
 namespace {
 
+// First vector of CTA b's part of nvec vectors: b nvec / parts moved up to a
+// multiple of g vectors, g the largest power of two up to 2048 and up to 1/32
+// of a part, at least 8.
+__device__ __forceinline__ size_t stage_begin(size_t nvec, size_t parts, size_t b) {
+  const size_t per = nvec / parts;
+  size_t g = 2048;
+  while (g > 8 && g * 32 > per) g >>= 1;
+  const size_t r = (nvec * b / parts + g - 1) & ~(g - 1);
+  return r < nvec ? r : nvec;
+}
+
 // Sub-bin address of pixel v (PATH/LK as in count_word), or the increment.
 template <int STAGE, int PATH, int LK>
 __device__ __forceinline__ void ablate_word(uint32_t w, uint32_t base, uint32_t lutb, uint32_t table, uint32_t& acc) {
@@ -244,8 +255,8 @@ __global__ void __launch_bounds__(kThreads, 2)
   }
   const Split sp = split_bytes(in, n);
   const uint4* body = reinterpret_cast<const uint4*>(in + sp.head);
-  const size_t begin = part_begin(sp.nvec, gridDim.x, blockIdx.x);
-  const size_t end = part_begin(sp.nvec, gridDim.x, blockIdx.x + 1);
+  const size_t begin = stage_begin(sp.nvec, gridDim.x, blockIdx.x);
+  const size_t end = stage_begin(sp.nvec, gridDim.x, blockIdx.x + 1);
   uint32_t acc = 0;
   if (STAGE == 7) {
     __shared__ __align__(8) unsigned long long full[kStageBufs];

@@ -189,8 +189,9 @@ __global__ void __launch_bounds__(kThreads, MINB) batch_images_kernel(BatchImgAr
 // the window's list: 3.5 us) and latency on small ones.  On the GPU, replayed
 // from a graph, before (one CTA-wide loop over all images, two CTAs per SM)
 // and now: 4096 images of 64 .. 4096 a side (9.97 GB) 1491 -> 1406 us (7.09
-// TB/s), 464 of 314 .. 2303 (0.68 GB) 123 -> 113, 2048 of 16 .. 256 (29 MB)
-// 38.8 -> 19.5, 4096 of 8 .. 22 51 -> 8.5 us.
+// TB/s), 464 of 314 .. 2303 (0.68 GB) 123 -> 112, 2048 of 16 .. 256 (29 MB)
+// 38.8 -> 18.8, 4096 of 8 .. 22 51 -> 7.5 us.  Both launches are chained: the
+// first clears its tables while the work before the call ends.
 
 constexpr uint32_t kLaneGroups = 4;
 constexpr int kLaneGroupThreads = kThreads / (int)kLaneGroups;
@@ -465,6 +466,15 @@ __global__ void __launch_bounds__(kThreads, 1) batch_lane_kernel(const __grid_co
   extern __shared__ __align__(16) uint32_t tables[];
   __shared__ LaneShared<SMALL> ls;
   const int t = threadIdx.x;
+  {
+    uint4* t4 = reinterpret_cast<uint4*>(tables);
+    for (int i = t; i < (int)(lane_smem<SMALL>() / 16); i += kThreads) t4[i] = make_uint4(0, 0, 0, 0);
+  }
+  if (t < (int)(sizeof(ls.eh) / 4)) (&ls.eh[0][0])[t] = 0;
+  if (t == 0) ls.i0 = a.count;
+  // the work before the call is complete from here on: it may have written
+  // the arrays and the images, and the second launch reads both
+  if (SMALL) pdl_wait();
   pdl_launch_dependents();
   // the batch's bytes: thread t holds images kLanePer t ...
   unsigned long long n[kLanePer], local = 0, total;
@@ -478,12 +488,6 @@ __global__ void __launch_bounds__(kThreads, 1) batch_lane_kernel(const __grid_co
   // warps: launch_batch_lane)
   const uint32_t zi = blockIdx.x * kWarps + ((uint32_t)t >> 5);
   const unsigned long long zsize = SMALL && zi < a.count ? (unsigned long long)a.sizes[zi] : 0ull;
-  {
-    uint4* t4 = reinterpret_cast<uint4*>(tables);
-    for (int i = t; i < (int)(lane_smem<SMALL>() / 16); i += kThreads) t4[i] = make_uint4(0, 0, 0, 0);
-  }
-  if (t < (int)(sizeof(ls.eh) / 4)) (&ls.eh[0][0])[t] = 0;
-  if (t == 0) ls.i0 = a.count;
   block_scan(local, ls.wsum, total);
   const unsigned long long share = grid_share(total, a.inv);
   if (SMALL && zi < a.count && !(zsize && lane_small(zsize, share))) {
@@ -626,9 +630,9 @@ bool lane_layouts(const RegimeLayouts& l) {
   return true;
 }
 
-// The launches of batch_lane_kernel.  The first starts when the work before it
-// is complete; the second reads nothing that the first writes, and writes
-// after it.
+// The launches of batch_lane_kernel.  The first waits for the work before it
+// before it reads; the second starts after that, reads nothing that the first
+// writes, and writes after it.
 int launch_batch_lane(const uint8_t* const* d_ptrs, const size_t* d_sizes, uint32_t count, uint32_t* d_out,
                       cudaStream_t s) {
   static int attr[kMaxDevices];
@@ -648,13 +652,13 @@ int launch_batch_lane(const uint8_t* const* d_ptrs, const size_t* d_sizes, uint3
     lc.blockDim = dim3(kThreads);
     lc.stream = s;
     a.inv = ~0ull / lc.gridDim.x;
-    lc.dynamicSmemBytes = lane_smem<true>();
-    cudaError_t e = cudaLaunchKernelEx(&lc, batch_lane_kernel<true>, a);
-    if (e != cudaSuccess) return cuda_fail(e);
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     lc.attrs = at;
     lc.numAttrs = 1;
+    lc.dynamicSmemBytes = lane_smem<true>();
+    cudaError_t e = cudaLaunchKernelEx(&lc, batch_lane_kernel<true>, a);
+    if (e != cudaSuccess) return cuda_fail(e);
     lc.dynamicSmemBytes = lane_smem<false>();
     e = cudaLaunchKernelEx(&lc, batch_lane_kernel<false>, a);
     if (e != cudaSuccess) return cuda_fail(e);

@@ -45,22 +45,25 @@ __device__ __forceinline__ uint32_t cluster_ld(uint32_t a, uint32_t rank) {
 // equal part, and the CTAs sum each other's tables through distributed
 // shared memory: no cleared output, no global atomics, one launch.  Bound by
 // latency (launch, one round of loads, two barriers of the cluster): 1 MiB of
-// uniform pixels 10.3 -> 8.2 us a call in a row (a clearing memset and 16
-// CTAs of per-warp tables before), 5.9 us of it on the GPU; 4 KiB 8.0 -> 3.6
-// us on the GPU.
+// uniform pixels 10.3 -> 4.8 us a call in a row (a clearing memset and 16
+// CTAs of per-warp tables before), 3.9 us of it on the GPU; 4 KiB 8.0 -> 1.5
+// us on the GPU.  Chained: the tables are cleared while the work before ends.
 __global__ void __launch_bounds__(kThreads, 1)
-    oneshot_cluster_kernel(const uint8_t* __restrict__ in, size_t n, uint32_t* __restrict__ out) {
+    oneshot_cluster_kernel(const uint8_t* __restrict__ in, uint32_t n, uint32_t* __restrict__ out, const Parts parts) {
   extern __shared__ __align__(16) uint32_t smem[];
   __shared__ uint32_t res[HIST_BINS];
   const int t = threadIdx.x;
   const uint32_t C = cluster_size(), rank = cluster_rank();
   const Split sp = split_bytes(in, n);
   const uint4* body = reinterpret_cast<const uint4*>(in + sp.head);
-  const uint32_t begin = (uint32_t)part_begin(sp.nvec, C, rank), end = (uint32_t)part_begin(sp.nvec, C, rank + 1);
+  const uint32_t nvec = (uint32_t)sp.nvec;
+  const uint32_t begin = part_begin(parts, nvec, rank), end = part_begin(parts, nvec, rank + 1);
   uint4 v[kLaneLoads];
   const LaneRange r = lane_range(body, begin, end, t);
-  lane_load<kLaneLoads, kThreads>(v, r);
   zero_table(smem);
+  pdl_wait();
+  pdl_launch_dependents();
+  lane_load<kLaneLoads, kThreads>(v, r);
   __syncthreads();
   lane_count<kLaneLoads, kThreads>(v, r, smem_addr(smem) + ((t & 31) << 2));
   __syncthreads();
@@ -84,10 +87,10 @@ __global__ void __launch_bounds__(kThreads, 1)
 }
 
 // A longer input: out is cleared by a launch of its own, which lets the
-// counting launch start at once; that one waits for it only before it adds.
-// The clearing launch itself starts when the work before it has completed,
-// so the pixels are there before either starts.
+// counting launch start once the work before the call has completed (the
+// pixels are there then); that one waits for the clear only before it adds.
 __global__ void __launch_bounds__(HIST_BINS) oneshot_clear_kernel(uint32_t* __restrict__ out) {
+  pdl_wait();
   pdl_launch_dependents();
   out[threadIdx.x] = 0;
 }
@@ -95,18 +98,18 @@ __global__ void __launch_bounds__(HIST_BINS) oneshot_clear_kernel(uint32_t* __re
 // One CTA of 1024 threads per SM with four loads in flight per thread: as
 // many bytes in flight as two CTAs with two loads each, without two CTAs on
 // one SM finishing their ranges apart.  Bound by the HBM read.  On the GPU,
-// clearing launch included: 64 MiB of uniform pixels 30.7 -> 14.7 us, 256 MiB
-// 98.4 -> 43.1 us (6.2 TB/s; per-warp tables before).
+// clearing launch included: 64 MiB of uniform pixels 30.7 -> 13.1 us, 256 MiB
+// 98.4 -> 40.1 us (6.7 TB/s; per-warp tables before).
 __global__ void __launch_bounds__(kThreads, 1)
-    oneshot_kernel(const uint8_t* __restrict__ in, size_t n, uint32_t* __restrict__ out) {
+    oneshot_kernel(const uint8_t* __restrict__ in, uint32_t n, uint32_t* __restrict__ out, const Parts parts) {
   extern __shared__ __align__(16) uint32_t smem[];
   __shared__ uint32_t res[HIST_BINS];
   const int t = threadIdx.x;
   pdl_launch_dependents();
   const Split sp = split_bytes(in, n);
   const uint4* body = reinterpret_cast<const uint4*>(in + sp.head);
-  const uint32_t begin = (uint32_t)part_begin(sp.nvec, gridDim.x, blockIdx.x);
-  const uint32_t end = (uint32_t)part_begin(sp.nvec, gridDim.x, blockIdx.x + 1);
+  const uint32_t nvec = (uint32_t)sp.nvec;
+  const uint32_t begin = part_begin(parts, nvec, blockIdx.x), end = part_begin(parts, nvec, blockIdx.x + 1);
   uint4 v[kLaneLoads];
   const LaneRange r = lane_range(body, begin, end, t);
   lane_load<kLaneLoads, kThreads>(v, r);
@@ -270,9 +273,9 @@ int ensure_wide_cluster(const void* fn, int* done) {
 constexpr size_t kClusterStep = (size_t)kThreads * 16;
 // Longest input of the cluster path: one round of four loads per thread of 16
 // CTAs.  Calls in a row on 1 MiB (the second launch costs the host 2.5 us):
-// 8.2 us against 9.7 with the clearing and the counting launch; replayed from
-// a graph 5.9 against 5.65, and 7.7 against 5.8 at 2 MiB, where 16 SMs are
-// too few.
+// 7.7 us against 10.5 with the clearing and the counting launch at 1.5 MiB;
+// replayed from a graph both take 3.8 - 3.9 us, and at 2 MiB the cluster 2 us
+// more, where 16 SMs are too few.
 constexpr size_t kClusterMax = 16 * 4 * kClusterStep;
 constexpr size_t kOneshotSmem = (size_t)kTableWords * 4;
 
@@ -284,11 +287,13 @@ int oneshot(const uint8_t* d_in, size_t n, uint32_t* d_out, cudaStream_t s) {
     return e == cudaSuccess ? HIST_OK : cuda_fail(e);
   }
   cudaLaunchConfig_t lc = {};
-  cudaLaunchAttribute at[1];
-  lc.blockDim = dim3(kThreads);
-  lc.dynamicSmemBytes = kOneshotSmem;
+  cudaLaunchAttribute at[2];
   lc.stream = s;
   lc.attrs = at;
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  lc.numAttrs = 1;
+  const uint32_t nvec = (uint32_t)split_bytes(d_in, n).nvec;
   if (n <= kClusterMax) {
     unsigned c = 1;
     while (c < 16 && c * kClusterStep < n) c <<= 1;
@@ -298,21 +303,26 @@ int oneshot(const uint8_t* d_in, size_t n, uint32_t* d_out, cudaStream_t s) {
       if (rc) return rc;
     }
     lc.gridDim = dim3(c);
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = c;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    lc.numAttrs = c > 1 ? 1 : 0;
-    e = cudaLaunchKernelEx(&lc, oneshot_cluster_kernel, d_in, n, d_out);
+    lc.blockDim = dim3(kThreads);
+    lc.dynamicSmemBytes = kOneshotSmem;
+    if (c > 1) {
+      at[1].id = cudaLaunchAttributeClusterDimension;
+      at[1].val.clusterDim.x = c;
+      at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+      lc.numAttrs = 2;
+    }
+    e = cudaLaunchKernelEx(&lc, oneshot_cluster_kernel, d_in, (uint32_t)n, d_out, make_parts(nvec, c));
     return e == cudaSuccess ? HIST_OK : cuda_fail(e);
   }
-  oneshot_clear_kernel<<<1, HIST_BINS, 0, s>>>(d_out);
-  e = cudaGetLastError();
+  lc.gridDim = dim3(1);
+  lc.blockDim = dim3(HIST_BINS);
+  e = cudaLaunchKernelEx(&lc, oneshot_clear_kernel, d_out);
   if (e != cudaSuccess) return cuda_fail(e);
-  lc.gridDim = dim3((unsigned)sm_count());
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  lc.numAttrs = 1;
-  e = cudaLaunchKernelEx(&lc, oneshot_kernel, d_in, n, d_out);
+  const uint32_t grid = (uint32_t)sm_count();
+  lc.gridDim = dim3(grid);
+  lc.blockDim = dim3(kThreads);
+  lc.dynamicSmemBytes = kOneshotSmem;
+  e = cudaLaunchKernelEx(&lc, oneshot_kernel, d_in, (uint32_t)n, d_out, make_parts(nvec, grid));
   return e == cudaSuccess ? HIST_OK : cuda_fail(e);
 }
 

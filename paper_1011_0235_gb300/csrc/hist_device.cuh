@@ -61,12 +61,6 @@ __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)
 __device__ __forceinline__ void shared_inc(uint32_t a) {
   asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(a) : "memory");
 }
-// The same by v.
-__device__ __forceinline__ void shared_add(uint32_t a, uint32_t v) {
-  asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
-}
-struct IncOne {};
-__device__ __forceinline__ void shared_add(uint32_t a, IncOne) { shared_inc(a); }
 __device__ __forceinline__ uint32_t shared_ld(uint32_t a) {
   uint32_t v;
   asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
@@ -176,13 +170,6 @@ static __device__ void count_range(const uint4* __restrict__ p, size_t begin, si
   for (; i < end; i += nthr) count_vec<PATH, LK>(ldg_stream(p + i), base, lutb, tab, o);
 }
 
-// The whole CTA, two loads in flight.
-template <int PATH, int LK>
-static __device__ void count_slice(const uint4* __restrict__ p, size_t begin, size_t end, uint32_t* table,
-                                   const uint32_t* lut) {
-  count_range<PATH, LK, 2>(p, begin, end, table, lut, threadIdx.x, kThreads);
-}
-
 // Layout dispatch for count_range.
 template <int UNROLL>
 __device__ __forceinline__ void count_range_dispatch(int path, int lk, const uint4* p, size_t begin, size_t end,
@@ -200,39 +187,6 @@ __device__ __forceinline__ void count_range_dispatch(int path, int lk, const uin
       default: count_range<PATH_SHIFT, 0, UNROLL>(p, begin, end, table, lut, tid, nthr); break;
     }
   }
-}
-
-__device__ __forceinline__ void count_dispatch(int path, int lk, const uint4* p, size_t begin,
-                                               size_t end, uint32_t* table, const uint32_t* lut) {
-  if (begin >= end) return;
-  if (path == PATH_PLAIN) count_slice<PATH_PLAIN, 0>(p, begin, end, table, lut);
-  else if (path == PATH_LUT) count_slice<PATH_LUT, 0>(p, begin, end, table, lut);
-  else {
-    switch (lk) {
-      case 5: count_slice<PATH_SHIFT, 5>(p, begin, end, table, lut); break;
-      case 4: count_slice<PATH_SHIFT, 4>(p, begin, end, table, lut); break;
-      case 3: count_slice<PATH_SHIFT, 3>(p, begin, end, table, lut); break;
-      case 2: count_slice<PATH_SHIFT, 2>(p, begin, end, table, lut); break;
-      case 1: count_slice<PATH_SHIFT, 1>(p, begin, end, table, lut); break;
-      default: count_slice<PATH_SHIFT, 0>(p, begin, end, table, lut); break;
-    }
-  }
-}
-
-// count_dispatch as a call of its own, for kernels that run at 32 registers
-// with other phases that need more: those spill around the call, and the
-// counting loop keeps its registers.
-static __device__ __noinline__ void count_call(int path, int lk, const uint4* p, size_t begin, size_t end,
-                                               uint32_t* table, const uint32_t* lut) {
-  count_dispatch(path, lk, p, begin, end, table, lut);
-}
-
-// The whole CTA with four loads in flight per thread, for kernels that run
-// one CTA of 1024 threads per SM (64 registers): the SM then keeps as many
-// bytes in flight as two CTAs with two loads each.
-static __device__ __noinline__ void count_call4(int path, int lk, const uint4* p, size_t begin, size_t end,
-                                                uint32_t* table, const uint32_t* lut) {
-  count_range_dispatch<4>(path, lk, p, begin, end, table, lut, threadIdx.x, kThreads);
 }
 
 // ------------------------------------------------- the lane-private table --
@@ -270,30 +224,29 @@ __device__ __forceinline__ void lane_load(uint4 (&v)[U], const LaneRange& r) {
 }
 
 // The 16 pixels of a vector into the lane-private table at `base` (this
-// lane's column), each as `inc`.
-template <class Inc>
-__device__ __forceinline__ void lane_vec(const uint4& q, uint32_t base, Inc inc) {
+// lane's column).
+__device__ __forceinline__ void lane_vec(const uint4& q, uint32_t base) {
   const uint32_t w4[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
-  for (int k = 0; k < 16; ++k) shared_add(base + (((w4[k >> 2] >> (8 * (k & 3))) & 0xffu) << 7), inc);
+  for (int k = 0; k < 16; ++k) shared_inc(base + (((w4[k >> 2] >> (8 * (k & 3))) & 0xffu) << 7));
 }
 
 // Count this thread's vectors of r, whose first U are loaded in v
 // (lane_load), keeping U loads in flight while it counts: the next ones of
 // its own, and at its end the first U of r2, the range that comes next (left
-// = 0: none), which v holds on return.  A pixel adds `inc`.  (Refilling each vector's registers as
+// = 0: none), which v holds on return.  (Refilling each vector's registers as
 // soon as it is counted, with 4 to 8 vectors, put every load behind 16
 // increments in the memory queue: 64 chunks of 16 MiB 161 -> 168-172 us,
 // 1024 of 64 KiB 24 -> 32 us.)
-template <int U, int NTHR, class Inc = IncOne>
+template <int U, int NTHR>
 __device__ __forceinline__ void lane_count(uint4 (&v)[U], LaneRange r, uint32_t base,
-                                           const LaneRange& r2 = LaneRange{nullptr, 0}, Inc inc = Inc()) {
+                                           const LaneRange& r2 = LaneRange{nullptr, 0}) {
   uint4 w[U];
   while (r.left > (uint32_t)((2 * U - 1) * NTHR)) {  // this round and the next are whole
 #pragma unroll
     for (int u = 0; u < U; ++u) w[u] = ldg_stream(r.q + (U + u) * NTHR);
 #pragma unroll
-    for (int u = 0; u < U; ++u) lane_vec(v[u], base, inc);
+    for (int u = 0; u < U; ++u) lane_vec(v[u], base);
 #pragma unroll
     for (int u = 0; u < U; ++u) v[u] = w[u];
     r.q += U * NTHR;
@@ -305,7 +258,7 @@ __device__ __forceinline__ void lane_count(uint4 (&v)[U], LaneRange r, uint32_t 
     lane_load<U, NTHR>(w, next);
 #pragma unroll
     for (int u = 0; u < U; ++u)
-      if ((uint32_t)(u * NTHR) < r.left) lane_vec(v[u], base, inc);
+      if ((uint32_t)(u * NTHR) < r.left) lane_vec(v[u], base);
 #pragma unroll
     for (int u = 0; u < U; ++u) v[u] = w[u];
     if (!more) return;
@@ -313,13 +266,12 @@ __device__ __forceinline__ void lane_count(uint4 (&v)[U], LaneRange r, uint32_t 
   }
 }
 
-// The per-bin sums of a lane-private table into res[0..255] (with ADD: added
-// to it), by NTHR threads (t: 0 .. NTHR - 1), and with CLEAR the table set to
+// The per-bin sums of a lane-private table into res[0..255], by NTHR threads (t: 0 .. NTHR - 1), and with CLEAR the table set to
 // zero.  Four threads take a row, each 8 words of it as two 16-byte reads;
 // the rows of odd index take them the other way round, so that the 8 lanes
 // of a 128-byte wavefront (two rows) read 32 banks.  The caller's barriers
 // stand before and after.
-template <int NTHR, bool CLEAR, bool ADD = false>
+template <int NTHR, bool CLEAR>
 __device__ __forceinline__ void lane_reduce(uint32_t* table, uint32_t* res, int t) {
 #pragma unroll
   for (int r0 = 0; r0 < HIST_BINS; r0 += NTHR / 4) {
@@ -330,7 +282,7 @@ __device__ __forceinline__ void lane_reduce(uint32_t* table, uint32_t* res, int 
     uint32_t sum = x.x + x.y + x.z + x.w + y.x + y.y + y.z + y.w;
     sum += __shfl_xor_sync(0xffffffffu, sum, 1);
     sum += __shfl_xor_sync(0xffffffffu, sum, 2);
-    if (q == 0) res[row] = ADD ? res[row] + sum : sum;
+    if (q == 0) res[row] = sum;
   }
 }
 
@@ -513,18 +465,28 @@ __device__ __forceinline__ unsigned long long split_point(const uint8_t* p, unsi
   return ((a + b + kSplitAlign - 1) & ~(kSplitAlign - 1)) - a;
 }
 
-// First vector of part b when nvec vectors are cut into `parts` contiguous
-// ranges (b = parts gives nvec): b nvec / parts moved up to a multiple of g
-// vectors, g the largest power of two up to 2048 (32 KiB) and up to 1/32 of
-// a part, at least 8 (a 128-byte line).  One-shot launches over 1 GiB:
-// the full table 6.61 -> 6.95 TB/s, the per-warp tables 5.44 -> 5.77 TB/s
-// against equal parts cut anywhere (cuts on 128-byte lines alone gave
-// 6.34 - 6.61 and 5.76).
-__host__ __device__ __forceinline__ size_t part_begin(size_t nvec, size_t parts, size_t b) {
+// How nvec vectors are cut into `parts` contiguous ranges (computed on the
+// host: a 64-bit division costs every warp of a CTA 150 instructions): part b
+// begins at b nvec / parts, or one vector less, moved up to a multiple of g
+// vectors, g the largest power of two up to 2048 (32 KiB) and up to 1/32 of a
+// part, at least 8 (a 128-byte line).  One-shot launches over 1 GiB: the full
+// table 6.61 -> 6.95 TB/s against equal parts cut anywhere.
+struct Parts {
+  unsigned long long inv;  // floor((2^64 - 1) / parts)
+  uint32_t parts, g;
+};
+inline Parts make_parts(size_t nvec, uint32_t parts) {
+  Parts p;
+  p.inv = ~0ull / parts;
+  p.parts = parts;
   const size_t per = nvec / parts;
-  size_t g = 2048;
-  while (g > 8 && g * 32 > per) g >>= 1;
-  const size_t r = (nvec * b / parts + g - 1) & ~(g - 1);
+  p.g = 2048;
+  while (p.g > 8 && (size_t)p.g * 32 > per) p.g >>= 1;
+  return p;
+}
+__device__ __forceinline__ uint32_t part_begin(const Parts& p, uint32_t nvec, uint32_t b) {
+  if (b == p.parts) return nvec;
+  const uint32_t r = ((uint32_t)__umul64hi((unsigned long long)nvec * b, p.inv) + p.g - 1) & ~(p.g - 1);
   return r < nvec ? r : nvec;
 }
 

@@ -72,6 +72,47 @@ def test_oneshot_chain_replayed_from_a_graph(n):
             assert hl.degeneracy_to_host(res) == (arg, m, t, oracle.switch(ref.astype(np.uint64), 450)), k
 
 
+@pytest.mark.parametrize("n", [700, 400_003, 3_000_017])
+def test_calls_behind_a_copy_in_a_graph(n):
+    """One-shot, batch and stream launches captured behind a memcpy that writes
+    their pixels (work that is no kernel), replayed over new pixels."""
+    src = torch.empty(n, dtype=torch.uint8, device="cuda")
+    xd = torch.empty(n, dtype=torch.uint8, device="cuda")
+    mid = torch.empty(n, dtype=torch.uint8, device="cuda")
+    out = hl.empty_hist()
+    rows = torch.empty((2, 256), dtype=torch.int32, device="cuda")
+    ptrs = torch.tensor([xd.data_ptr(), xd.data_ptr() + 5], dtype=torch.int64, device="cuda")
+    szs = torch.tensor([n, min(n - 5, 3000)], dtype=torch.int64, device="cuda")
+    st = hl.Stream(mode=hl.MODE_AUTO)
+    push_out = torch.empty(256, dtype=torch.int32, device="cuda")
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        def step():
+            xd.copy_(src)
+            hl.hist_plain(xd, out)
+            mid.copy_(xd)
+            assert hl.lib().hist_batch(ptrs.data_ptr(), szs.data_ptr(), 2, rows.data_ptr(), None, s.cuda_stream) == 0
+            mid.copy_(xd)
+            st.push(xd, push_out)
+        src.zero_()
+        step()
+        s.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s):
+            step()
+        for k, law in enumerate([synth.normal(60, 9), synth.uniform(), synth.degenerate(3, 0.9)]):
+            x = synth.host(n, law, SEED + 97, k * n)
+            src.copy_(torch.from_numpy(x))
+            g.replay()
+            s.synchronize()
+            ref = oracle.hist_u32(x)
+            assert np.array_equal(u32(out), ref) and np.array_equal(u32(push_out), ref), k
+            got = u32(rows).reshape(2, 256)
+            assert np.array_equal(got[0], ref), k
+            assert np.array_equal(got[1], oracle.hist_u32(x[5:5 + min(n - 5, 3000)])), k
+    st.close()
+
+
 def _sample_flag(x, addr, theta=450):
     """The switch from a chunk's sample: 256 evenly spaced 16-byte vectors
     from the first 16-byte boundary of its address, or the whole chunk."""
