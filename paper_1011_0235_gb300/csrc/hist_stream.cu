@@ -152,7 +152,7 @@ __device__ __forceinline__ unsigned long long ld_acquire(const unsigned long lon
 // chunk before, weighed and laid out the chunks by it and counted the
 // mispredicted ones again: 64 chunks of 16 MiB took 208 us a push of N(128,
 // 8) and 287 us on the degenerate workload, in a 960-slot adaptive stream 435
-// us; all now take what the full table takes, 160 us.
+// us; all now take what the full table takes, 159 us.
 
 // Cost of a chunk beyond its bytes.  Launches of 1024 x 16 KiB, 100 x 64 KiB
 // and 512 x 256 KiB chunks: 12.1, 10.8 and 38.6 us with 32 KiB, 10.7, 8.1 and
@@ -198,6 +198,11 @@ struct FlatDesc {
   uint32_t n;
   uint32_t j;
 };
+// A piece of a chunk: bytes [b0, e0) (e0 = 0: an empty chunk).
+struct FlatPiece {
+  FlatDesc d;
+  uint32_t b0, e0;
+};
 constexpr uint32_t kListItems = 2 * kWarps;  // chunks the groups take at a time
 
 // CTA-wide state of batch_flat_kernel (shared memory).
@@ -205,16 +210,18 @@ template <uint32_t CAP>
 struct FlatShared {
   alignas(16) unsigned long long ring_seen[2];  // launches_done as the launch started (cp.async)
   EpiShared es[kGroups];
-  uint32_t res[HIST_BINS];   // sums of the piece in the table
-  uint32_t eh[HIST_BINS];    // its unaligned edge bytes
-  uint32_t samp[HIST_BINS];  // AUTO: the sample's pixels in it
+  uint32_t res[HIST_BINS];      // sums of the piece in the table
+  uint32_t eh[2][HIST_BINS];    // unaligned edge bytes of the CTA's pieces, in turn
+  uint32_t samp[2][HIST_BINS];  // AUTO: the sample's pixels in them
   int last;
   int released;  // this CTA has waited for the previous launch
-  int ring_ok;   // the chunk ring slots of this launch are free
   uint32_t epis; // chunk epilogues this CTA ran
+  FlatDesc win[kWarps];         // the chunks of the range the CTA is at
+  FlatPiece piece[kWarps];      // its pieces of them
+  uint32_t npiece, nwl;
+  unsigned long long pos;       // cost position of the chunk after them
   uint16_t wl[CAP];             // whole chunks left to the groups, in batch order
   GroupItem items[kListItems];  // the chunks the groups are at
-  FlatDesc win[kWarps];         // chunk j in entry j mod kWarps (flat_descs)
   uint32_t gmax[kGroups][2][HIST_BINS / 32];  // each group's largest bins per warp: chunk, sample
   uint32_t geh[kGroups][HIST_BINS];    // each group's edge bytes
   uint32_t gsamp[kGroups][HIST_BINS];  // and sample
@@ -356,99 +363,92 @@ __device__ __forceinline__ void flat_finish(const A& a, uint32_t epis) {
 // before it reads a chunk byte: that work may be the kernel that wrote the
 // chunk, and only the wait makes its writes visible.  A CTA also waits for
 // the previous launch to complete before its first epilogue, which reads
-// and writes the stream state (flat_release), and before it first adds
-// into a chunk ring slot, the last user of the slot -- a launch at least
-// kChunkRing / kMaxBatch - 1 launches back -- must be complete
-// (flat_ring_ready, a bounded wait for the number that each launch writes
-// once it knows the launch before it to be complete).  All threads call
-// both.
+// and writes the stream state, and before it first adds into a chunk ring
+// slot, the last user of the slot -- a launch at least kChunkRing / kMaxBatch
+// - 1 launches back -- must be complete (flat_ring_ready, a bounded wait for
+// the number that each launch writes once it knows the launch before it to be
+// complete).
 __device__ __forceinline__ void flat_prev_done(const PushHead& a) {
   asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(&a.st->h.launches_done), "l"(a.prev) : "memory");
 }
-template <class A>
-__device__ __forceinline__ void flat_release(const A& a, FlatShared<A::kCap>& fs) {
-  if (!fs.released) pdl_wait();
-  __syncthreads();
-  if (threadIdx.x == 0 && !fs.released) {
-    fs.released = 1;
-    flat_prev_done(a);
-  }
-}
 
+// Thread 0.  (A launch that waited at its start has its slots: for it this
+// only checks the number, as it stood then.)
 template <class A>
 __device__ __noinline__ void flat_ring_ready(const A& a, FlatShared<A::kCap>& fs) {
-  // fs.ring_ok is read between the first two barriers and written after the
-  // second, so every thread takes the same branch
-  __syncthreads();
-  if (fs.ring_ok) return;
   constexpr unsigned long long back = kChunkRing / kMaxBatch - 1;
-  if (threadIdx.x == 0) {
-    asm volatile("cp.async.wait_all;" ::: "memory");
-    // as the launch started (a launch that waited there needs no more)
-    if (a.early || fs.ring_seen[0] + back < a.launch) {
-      uint32_t it = 0;
-      while (a.launch > back && ld_acquire(&a.st->h.launches_done) < a.launch - back) {
-        if (++it >= kPollLimit) {
-          atomicOr(&a.st->h.status, kStatusTimeout);
-          break;
-        }
-        __nanosleep(256);
-      }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  if (!a.early && fs.ring_seen[0] + back >= a.launch) return;
+  uint32_t it = 0;
+  while (a.launch > back && ld_acquire(&a.st->h.launches_done) < a.launch - back) {
+    if (++it >= kPollLimit) {
+      atomicOr(&a.st->h.status, kStatusTimeout);
+      break;
     }
+    __nanosleep(256);
   }
-  __syncthreads();
-  if (threadIdx.x == 0) fs.ring_ok = 1;
 }
 
-// Run the epilogue of chunk d, whose histogram and sample threads 0..255 hold.
-// All threads call.
+// Count piece k of the window's (the CTA's number `turn`; `ring`: whether the
+// ring check is behind) into the table, which is clear before and after, and
+// publish it: into the chunk's accumulator, or, when it is the whole chunk,
+// straight into the chunk's epilogue.  The CTA that completes a chunk runs
+// its epilogue, by the first 256 threads while the others go on to the CTA's
+// next piece, whose first 128 KiB are fetched into L2 while this one's table
+// is reduced.  All threads call.
 template <class A>
-__device__ __forceinline__ void flat_complete(const A& a, const FlatDesc& d, uint32_t h, uint32_t s,
-                                              FlatShared<A::kCap>& fs) {
-  flat_release(a, fs);
-  if (threadIdx.x < HIST_BINS) flat_epilogue(a, d, h, s, fs.es[0], threadIdx.x, kEpiBar);
-  if (threadIdx.x == 0) fs.epis += 1;
-}
-
-// Reduce the table, which holds bytes [b0, e0) of chunk d, and publish the
-// piece: into the chunk's accumulator, or, when it is the whole chunk,
-// straight into the chunk's epilogue.  The CTA that completes the chunk runs
-// the epilogue.  The table is left clear.  All threads call.
-template <class A>
-__device__ __noinline__ void flat_flush(const A& a, const FlatDesc& d, uint32_t b0, uint32_t e0, uint32_t* table,
-                                        FlatShared<A::kCap>& fs) {
-  __syncthreads();
+__device__ __forceinline__ void flat_piece(const A& a, uint32_t k, uint32_t turn, bool& ring, uint32_t* table,
+                                           FlatShared<A::kCap>& fs) {
   StreamDev* st = a.st;
   const int t = threadIdx.x;
-  const uint32_t n = d.n, j = d.j;
-  lane_reduce<kThreads, true>(table, fs.res, t);
-  __syncthreads();
+  const FlatPiece& p = fs.piece[k];
   uint32_t h = 0, s = 0;
-  if (t < HIST_BINS) {
-    h = fs.res[t] + fs.eh[t];
-    s = fs.samp[t];
-    fs.eh[t] = fs.samp[t] = 0;
+  flat_mark(a, p.d.j, 0);
+  if (p.e0) {
+    const uint8_t* vec = nullptr;
+    if (flat_sampled(a, p.d.j) && t < (int)kSampleVecs) {
+      // (every cut between pieces is a multiple of 16 bytes in memory)
+      const uint32_t at = sample_at(p.d.in, p.d.n, t);
+      if (at != 0xffffffffu && at >= p.b0 && at < p.e0) vec = p.d.in + at;
+    }
+    piece_count(p.d.in + p.b0, p.e0 - p.b0, table, fs.eh[turn & 1], vec, fs.samp[turn & 1]);
+    if (k + 1 < fs.npiece) {
+      const FlatPiece& q = fs.piece[k + 1];
+      const uint32_t at = (uint32_t)t * kLineBytes;
+      if (at < q.e0 - q.b0) asm volatile("prefetch.global.L2 [%0];" ::"l"(q.d.in + q.b0 + at));
+    }
+    __syncthreads();
+    lane_reduce<kThreads, true>(table, fs.res, t);
+    __syncthreads();
+    if (t < HIST_BINS) {
+      h = fs.res[t] + fs.eh[turn & 1][t];
+      s = fs.samp[turn & 1][t];
+      fs.eh[turn & 1][t] = fs.samp[turn & 1][t] = 0;
+    }
+    flat_mark(a, p.d.j, 5);
   }
-  flat_mark(a, j, 5);
-  if (e0 - b0 == n) {
-    flat_complete(a, d, h, s, fs);
-  } else {
-    flat_ring_ready(a, fs);
-    const uint32_t slot = (uint32_t)((a.first_chunk + j) % kChunkRing);
+  bool complete = p.e0 - p.b0 == p.d.n;
+  if (!complete) {
+    if (!ring) {
+      if (t == 0) flat_ring_ready(a, fs);
+      if (a.early) __syncthreads();
+      ring = true;
+    }
+    const uint32_t slot = (uint32_t)((a.first_chunk + p.d.j) % kChunkRing);
     unsigned long long* acc = &st->racc[slot][t & (HIST_BINS - 1)];
     bool done = false;
     if (t < HIST_BINS) {
-      const unsigned long long add = acc_word(h, acc_blocks(d.in, b0, e0), s);
+      const unsigned long long add = acc_word(h, acc_blocks(p.d.in, p.b0, p.e0), s);
       const unsigned long long sum = atomicAdd(acc, add) + add;
-      done = ((uint32_t)(sum >> 32) & kAccBlockMask) == acc_blocks(d.in, 0, n);
+      done = ((uint32_t)(sum >> 32) & kAccBlockMask) == acc_blocks(p.d.in, 0, p.d.n);
       h = (uint32_t)sum;
       s = (uint32_t)(sum >> 50);
     }
     const int bins = __syncthreads_count(done);
     if (bins == HIST_BINS) {
       // this CTA's adds were the last to every bin
+      complete = true;
       if (t < HIST_BINS) *acc = 0;
-      flat_complete(a, d, h, s, fs);
     } else if (bins > 0) {
       // two CTAs' adds crossed: the one that brings the completed bins to 256
       // reads them all
@@ -458,7 +458,8 @@ __device__ __noinline__ void flat_flush(const A& a, const FlatDesc& d, uint32_t 
         __threadfence();
       }
       __syncthreads();
-      if (fs.last) {
+      complete = fs.last != 0;
+      if (complete) {
         if (t < HIST_BINS) {
           const unsigned long long sum = __ldcg(acc);
           h = (uint32_t)sum;
@@ -466,51 +467,87 @@ __device__ __noinline__ void flat_flush(const A& a, const FlatDesc& d, uint32_t 
           *acc = 0;
         }
         if (t == 0) st->rbins[slot] = 0;
-        flat_complete(a, d, h, s, fs);
       }
     }
   }
-  flat_mark(a, j, 7);
-  __syncthreads();
-}
-
-// piece_count as a call of its own, which keeps the counting loop's registers
-// from what surrounds it.
-static __device__ __noinline__ void flat_count(const uint8_t* base, uint32_t len, uint32_t* table, uint32_t* eh,
-                                               const uint8_t* vec, uint32_t* samp) {
-  piece_count(base, len, table, eh, vec, samp);
-}
-
-// Count bytes [b0, e0) of chunk d (not empty) into the table, which is clear
-// (a CTA's range holds one piece of a chunk), and publish the piece.  All
-// threads call.
-template <class A>
-__device__ __forceinline__ void flat_piece(const A& a, const FlatDesc& d, uint32_t b0, uint32_t e0, uint32_t* table,
-                                           FlatShared<A::kCap>& fs) {
-  flat_mark(a, d.j, 0);
-  const uint8_t* vec = nullptr;
-  if (flat_sampled(a, d.j) && threadIdx.x < kSampleVecs) {
-    // (every cut between pieces is a multiple of 16 bytes in memory)
-    const uint32_t at = sample_at(d.in, d.n, threadIdx.x);
-    if (at != 0xffffffffu && at >= b0 && at < e0) vec = d.in + at;
+  if (t < HIST_BINS) {
+    if (complete) {
+      if (a.early) {
+        pdl_wait();
+        if (t == 0 && !fs.released) {
+          fs.released = 1;
+          flat_prev_done(a);
+        }
+      }
+      flat_epilogue(a, p.d, h, s, fs.es[0], t, kEpiBar);
+      if (t == 0) fs.epis += 1;
+    }
+    flat_mark(a, p.d.j, 7);
   }
-  flat_count(d.in + b0, e0 - b0, table, fs.eh, vec, fs.samp);
-  flat_flush(a, d, b0, e0, table, fs);
 }
 
-// Chunks [j0, j0 + kWarps) into fs.win, warp w reading chunk j0 + w's entry
-// with a warp-uniform index, so that the warps' constant-cache misses
-// overlap; returns the end of the chunks read.  All threads call (ends with a
-// barrier).
+// Chunks [j0, j0 + kWarps), the first at cost position fs.pos: into fs.win, a
+// warp each with a warp-uniform index (their constant-cache misses overlap),
+// then warp 0, a chunk per lane, lists the CTA's pieces of them and, in fs.wl,
+// the whole ones left to the groups.  Chunk j's byte b sits at its cost
+// position + b (after the tail cost for the last two chunks); a range takes
+// the bytes whose cost position it holds.  All threads call (begins and ends
+// with a barrier).
 template <class A>
-__device__ __noinline__ uint32_t flat_descs(const A& a, uint32_t j0, FlatShared<A::kCap>& fs) {
-  const uint32_t j = j0 + (threadIdx.x >> 5);
-  if (j < a.count) {
-    const FlatDesc d = {a.c[j].in, a.c[j].out, a.c[j].n, j};
-    if ((threadIdx.x & 31) == 0) fs.win[j % kWarps] = d;
+__device__ __forceinline__ void flat_window(const A& a, uint32_t j0, FlatShared<A::kCap>& fs) {
+  const uint32_t w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  __syncthreads();
+  if (j0 + w < a.count) {
+    const FlatDesc d = {a.c[j0 + w].in, a.c[j0 + w].out, a.c[j0 + w].n, j0 + w};
+    if (lane == 0) fs.win[w] = d;
   }
   __syncthreads();
-  return j0 + kWarps;
+  if (w == 0) {
+    const unsigned long long lo = a.plan.lo[blockIdx.x], hi = a.plan.lo[blockIdx.x + 1];
+    const bool in = j0 + lane < a.count;
+    const FlatDesc d = in ? fs.win[lane] : FlatDesc{nullptr, nullptr, 0, 0};
+    const uint32_t n = d.n;
+    const unsigned long long c = in ? flat_cost(n, d.j, a.count) : 0ull;
+    unsigned long long x = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
+      if ((int)lane >= o) x += y;
+    }
+    const unsigned long long p0 = fs.pos + x - c;
+    // a chunk of at most a quarter of a CTA's range is not split: the range
+    // holding its first cost position counts it whole, so it needs no
+    // accumulator or ring; a small one is left to the groups
+    bool piece = false, item = false;
+    unsigned long long b0 = 0, e0 = 0;
+    if (in && p0 < hi) {
+      if (n == 0 || plan_whole(n, a.plan.range)) {
+        item = p0 >= lo && n != 0 && n <= a.plan.group_max;
+        piece = p0 >= lo && !item;
+        e0 = n;
+      } else {
+        // byte b sits at cost q0 + b, after the chunk's tail cost
+        const unsigned long long q0 = p0 + flat_tail(n, d.j, a.count);
+        if (hi > q0) {
+          b0 = lo > q0 ? split_point(d.in, lo - q0) : 0ull;
+          e0 = split_point(d.in, hi - q0);
+          if (e0 > (unsigned long long)n) e0 = n;
+          piece = b0 < e0;
+        }
+      }
+    }
+    const unsigned mp = __ballot_sync(0xffffffffu, piece), mi = __ballot_sync(0xffffffffu, item);
+    const unsigned lt = (1u << lane) - 1u;
+    if (piece) fs.piece[__popc(mp & lt)] = FlatPiece{d, (uint32_t)b0, (uint32_t)e0};
+    if (item) fs.wl[fs.nwl + __popc(mi & lt)] = (uint16_t)d.j;
+    __syncwarp();
+    if (lane == 31) {
+      fs.pos = p0 + c;
+      fs.npiece = __popc(mp);
+      fs.nwl += __popc(mi);
+    }
+  }
+  __syncthreads();
 }
 
 __device__ __forceinline__ GroupItem group_item(const PushHead& a, const FlatDesc& d) {
@@ -524,60 +561,6 @@ __device__ __forceinline__ GroupItem group_item(const PushHead& a, const FlatDes
   it.edges = (uint32_t)sp.head | ((uint32_t)sp.tail << 8) |
              (flat_sampled(a, d.j) && !sample_whole(d.in, d.n) ? 1u << 16 : 0u);
   return it;
-}
-
-// Count the cost range [x0, x1) of the batch.  Chunk j's byte b sits at its
-// cost position + b (after the tail cost for the last two chunks); a range
-// takes the bytes whose cost position it holds.  The chunks before wend are
-// read (flat_descs).  Returns the number of whole chunks left to the groups
-// (fs.wl).  All threads call.
-template <class A>
-__device__ uint32_t flat_range(const A& a, unsigned long long x0, unsigned long long x1, unsigned long long range,
-                               uint32_t wend, uint32_t* table, FlatShared<A::kCap>& fs) {
-  uint32_t nwl = 0;
-  uint32_t j = a.plan.j[blockIdx.x];
-  unsigned long long p0 = a.plan.pre[blockIdx.x], p1 = 0;  // cost position of chunk j, of chunk j + 1
-  for (; j < a.count && p0 < x1; ++j, p0 = p1) {
-    if (j == wend) {
-      __syncthreads();
-      wend = flat_descs(a, j, fs);
-    }
-    const FlatDesc d = fs.win[j % kWarps];
-    const uint32_t n = d.n;
-    p1 = p0 + flat_cost(n, j, a.count);
-    if (n == 0) {
-      // no bytes: the range holding the chunk's first cost position folds it
-      if (p0 >= x0) {
-        flat_mark(a, j, 0);
-        flat_complete(a, d, 0u, 0u, fs);
-        __syncthreads();
-        flat_mark(a, j, 7);
-      }
-      continue;
-    }
-    if (plan_whole(n, range)) {
-      // a chunk of at most a quarter of a CTA's range is not split: the
-      // range holding its first cost position counts it whole, so it needs
-      // no accumulator or ring; a small one is left to the groups
-      if (p0 >= x0) {
-        if (n <= a.plan.group_max) {
-          if (threadIdx.x == 0) fs.wl[nwl] = (uint16_t)j;
-          ++nwl;
-        } else {
-          flat_piece(a, d, 0, n, table, fs);
-        }
-      }
-      continue;
-    }
-    // byte b sits at cost q0 + b, after the chunk's tail cost
-    const unsigned long long q0 = p0 + flat_tail(n, j, a.count);
-    if (x1 <= q0) continue;
-    const unsigned long long c0 = x0 > q0 ? split_point(d.in, x0 - q0) : 0ull;
-    const unsigned long long c1 = split_point(d.in, x1 - q0);
-    const unsigned long long e0 = c1 < (unsigned long long)n ? c1 : (unsigned long long)n;
-    if (c0 < e0) flat_piece(a, d, (uint32_t)c0, (uint32_t)e0, table, fs);
-  }
-  return nwl;
 }
 
 // ------------------------------------------------ whole small chunks --
@@ -752,9 +735,9 @@ __device__ __forceinline__ void flat_groups(const A& a, uint32_t nwl, int first,
 // before the other and the SM then runs a single CTA at half its loads in
 // flight; one CTA per SM has no such pair.  Bound by the HBM read on large
 // chunks, by a chain of round trips to L2 on one small one: on the GPU,
-// pushes in a row, 64 x 16 MiB 166.6 -> 160 us (6.7 TB/s; overlapping
-// 162 -> 157 us), 128 x 1 MiB 39.2 -> 31 us, one chunk of 9 KB in AUTO mode
-// 17.4 -> 5.4 us, of 1 MiB 15.6 -> 9.1 us.
+// pushes in a row, 64 x 16 MiB 166.6 -> 158.7 us (6.8 TB/s; overlapping
+// 162 -> 155.7 us), 128 x 1 MiB 39.2 -> 28.1 us, one chunk of 9 KB in AUTO
+// mode 17.4 -> 5.3 us, of 1 MiB 15.6 -> 7.6 us.
 template <class A>
 __global__ void __launch_bounds__(kThreads, 1) batch_flat_kernel(const __grid_constant__ A a) {
   extern __shared__ __align__(16) uint32_t tables[];
@@ -762,24 +745,26 @@ __global__ void __launch_bounds__(kThreads, 1) batch_flat_kernel(const __grid_co
   const int t = threadIdx.x;
 
   pdl_launch_dependents();
-  if (t < HIST_BINS) fs.eh[t] = fs.samp[t] = 0;
   if (t == 0) {
     fs.released = a.early ? 0 : 1;
-    fs.ring_ok = 0;
     fs.epis = 0;
   }
   // what the range needs of the parameters is read before the wait
-  const bool groups = a.plan.groups[blockIdx.x >> 5] >> (blockIdx.x & 31) & 1u;
-  const uint32_t s0 = a.plan.s[blockIdx.x], s1 = a.plan.s[blockIdx.x + 1], j0 = a.plan.j[blockIdx.x];
-  const unsigned long long lo = a.plan.lo[blockIdx.x], hi = a.plan.lo[blockIdx.x + 1];
-  if (groups) {
+  if (a.plan.groups[blockIdx.x >> 5] >> (blockIdx.x & 31) & 1u) {
     // the range holds whole chunks for the groups only
+    const uint32_t s0 = a.plan.s[blockIdx.x], s1 = a.plan.s[blockIdx.x + 1];
     __syncthreads();
     flat_groups(a, s1 - s0, (int)s0, !a.early, tables, fs);
     if (!a.early && blockIdx.x == 0 && t == kThreads - 1) flat_prev_done(a);
   } else {
+    const uint32_t j0 = a.plan.j[blockIdx.x];
+    if (t == 0) {
+      fs.pos = a.plan.pre[blockIdx.x];
+      fs.nwl = 0;
+    }
     zero_table(tables);
-    const uint32_t wend = flat_descs(a, j0, fs);
+    if (t < HIST_BINS) fs.eh[0][t] = fs.eh[1][t] = fs.samp[0][t] = fs.samp[1][t] = 0;
+    flat_window(a, j0, fs);
     if (!a.early) {
       pdl_wait();
       if (blockIdx.x == 0 && t == kThreads - 1) flat_prev_done(a);
@@ -788,10 +773,16 @@ __global__ void __launch_bounds__(kThreads, 1) batch_flat_kernel(const __grid_co
                      "l"(&a.st->h.launches_done)
                      : "memory");
     }
-    uint32_t nwl = 0;
-    if (lo < hi) nwl = flat_range(a, lo, hi, a.plan.range, wend, tables, fs);
+    bool ring = false;
+    uint32_t turn = 0;
+    for (uint32_t j = j0;;) {
+      for (uint32_t k = 0; k < fs.npiece; ++k) flat_piece(a, k, turn++, ring, tables, fs);
+      j += kWarps;
+      if (fs.pos >= a.plan.lo[blockIdx.x + 1] || j >= a.count) break;
+      flat_window(a, j, fs);
+    }
     __syncthreads();
-    if (nwl) flat_groups(a, nwl, -1, false, tables, fs);
+    if (fs.nwl) flat_groups(a, fs.nwl, -1, false, tables, fs);
   }
   __syncthreads();
   if (t == 0) {
