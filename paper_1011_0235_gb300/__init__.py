@@ -220,9 +220,18 @@ class TorchAllocator:
 
 
 
+_U64 = np.dtype(np.uint64)
+
+
 def _u64_array(seq, n: int, name: str):
     """The address of n 8-byte integers for a C array argument, and the
     object that owns them (kept alive for the call)."""
+    if type(seq) is np.ndarray and seq.dtype == _U64 and seq.shape == (n,) and n and seq.flags.c_contiguous:
+        # the usual case, without the checks below
+        try:
+            return ctypes.addressof(ctypes.c_char.from_buffer(seq)), seq
+        except (TypeError, ValueError):  # read-only
+            return seq.ctypes.data, seq
     if isinstance(seq, torch.Tensor):
         if seq.device.type != "cpu":
             raise ValueError(f"{name}: a CPU tensor or a sequence of ints")

@@ -627,21 +627,20 @@ int admit(hist_server* s) {
   a->c.budget = s->cfg.pattern_budget;
   a->c.theta = s->cfg.theta_milli;
   a->c.mode = s->cfg.mode;
-  unsigned long long cost = 0;
   for (uint32_t i = 0; i < count; ++i) {
     const PendingReq& r = f->reqs[i];
     a->req[i].in = r.in;
     a->req[i].out = r.out;
     a->req[i].n = (uint32_t)r.n;
     a->req[i].stream = r.stream;
-    cost += srv_cost(r.n);
   }
-  unsigned long long grid = (cost + kCtaCost - 1) / kCtaCost;
+  PlanCosts<kSrvMaxBatch> pc;
+  auto size = [&](uint32_t i) { return (unsigned long long)a->req[i].n; };
+  plan_costs(&pc, count, size, [&](uint32_t i) { return srv_cost(a->req[i].n); });
+  unsigned long long grid = (pc.pos[count] + kCtaCost - 1) / kCtaCost;
   if (grid > (unsigned long long)s->max_grid) grid = (unsigned long long)s->max_grid;
   if (grid < 1) grid = 1;
-  plan_ranges(
-      &a->plan, count, (uint32_t)grid, kSmallReq, [&](uint32_t i) { return (unsigned long long)a->req[i].n; },
-      [&](uint32_t i) { return srv_cost(a->req[i].n); });
+  plan_ranges(&a->plan, pc, count, (uint32_t)grid, kSmallReq, size);
   // the small variant's parameters are a prefix of the large one's
   static_assert(offsetof(SrvArgs<kSmallCap>, req) == offsetof(SrvArgs<kSrvMaxBatch>, req), "parameter layout");
   static_assert(sizeof(SrvArgs<kSrvMaxBatch>) <= 32764, "kernel parameters are limited to 32764 bytes");

@@ -1058,14 +1058,13 @@ cudaError_t launch_chained(const void* fn, dim3 grid, dim3 block, void** params,
 // CTAs, and no more than kCtaCost bytes, or a chunk, each needs.
 constexpr unsigned long long kCtaCost = 32ull << 10;
 uint32_t flat_plan(RangePlan* p, uint32_t count, const size_t* ns, uint32_t grid) {
-  unsigned long long bytes = 0;
-  for (uint32_t i = 0; i < count; ++i) bytes += ns[i];
-  unsigned long long want = (bytes + kCtaCost - 1) / kCtaCost;
+  PlanCosts<kMaxBatch> c;
+  auto size = [&](uint32_t i) { return (unsigned long long)ns[i]; };
+  plan_costs(&c, count, size, [&](uint32_t i) { return flat_cost(ns[i], i, count); });
+  unsigned long long want = (c.bytes + kCtaCost - 1) / kCtaCost;
   if (want < count) want = count;
   if (want < grid) grid = (uint32_t)want;
-  plan_ranges(
-      p, count, grid, kGroupChunkMax, [&](uint32_t i) { return (unsigned long long)ns[i]; },
-      [&](uint32_t i) { return flat_cost(ns[i], i, count); });
+  plan_ranges(p, c, count, grid, kGroupChunkMax, size);
   return grid;
 }
 
