@@ -547,13 +547,14 @@ int hist_ablation(const uint8_t* d_in, size_t n, const hist_pattern* d_pat, uint
  *           the last poll -- a request's epilogue on the GPU writes its
  *           completion word in pinned host memory once the request's output
  *           is written, so a request completes without waiting for the rest
- *           of its batch; it then updates the stream's state and writes the
- *           request's state word, and poll gives a returned request's stream
- *           back to admission once that word is seen -- and releases the
- *           batch slots whose completion event has fired (with them, their
- *           bytes of the budget); then it admits the next batch if one of
- *           max_inflight batch slots is free: in FIFO order, every queued
- *           request whose stream has no request on the GPU and whose bytes
+ *           of its batch, and its stream goes back to admission when its
+ *           completion has been returned; the epilogue then updates the
+ *           stream's state and writes the request's state word -- and
+ *           releases the batch slots whose requests' words are all written
+ *           (with them, their bytes of the budget); then it admits the next
+ *           batch if one of max_inflight batch slots is free: in FIFO order,
+ *           every queued request whose stream's last request has been
+ *           returned (and the one before has written its state) and whose bytes
  *           fit the HBM budget (bytes of all requests on the GPU <=
  *           hbm_budget), up to max_batch requests.  The batch is one kernel
  *           on the slot's own CUDA stream, so batches overlap on the device:

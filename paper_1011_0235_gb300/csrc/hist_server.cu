@@ -3,28 +3,30 @@
 // Each request is the next chunk of one of `streams` independent streams; a
 // stream's adaptive state (the switch flag, the binning pattern and the
 // layout derived from it, the totals and the last histogram) stays on the
-// device, so a request gets the kernel and pattern chosen from its stream's
-// previous request (Sec. III.B / III.C), exactly as hist_stream_push would;
-// every kernel and pattern counts in the lane-private table.
+// device, as hist_stream_push would leave it (Sec. III.B / III.C).
 //
 // Continuous batching on the host: submitted requests wait in a FIFO queue;
 // whenever a batch slot is free, the queued requests that fit the HBM byte
-// budget and whose stream has no request on the GPU form a batch, launched
+// budget and whose stream's last request has completed form a batch, launched
 // on the slot's own CUDA stream, so batches overlap on the device.  A batch
 // is one kernel with no device-side waits: the host splits the requests among
 // the CTAs by a cost model (bytes plus a fixed cost per request), each CTA
 // counts its pieces and adds them into the requests' accumulators; the CTA
-// that completes a request computes its degeneracy and next pattern and
-// updates the stream's state.  Small requests are counted whole by groups of
-// warps, each of which runs its requests' epilogues itself.  A request counted
-// whole by one CTA skips the accumulator.  Once a request's output is written, its
-// epilogue writes the batch's sequence number into the request's completion
-// word in pinned host memory, so the host sees each request complete without
-// waiting for the rest of its batch; it then updates the stream's state and
-// writes the number into the request's state word, which releases the stream
-// to admission: the stream's next request may run in a batch that fills the
-// SMs while this one drains.  The slot itself (its scratch and its bytes of
-// the budget) is released when the slot's event shows the whole batch done.
+// that completes a request runs its epilogue.  Small requests are counted
+// whole by groups of warps, each of which runs its requests' epilogues itself.
+// A request counted whole by one CTA skips the accumulator.
+//
+// Once a request's output is written, its epilogue writes the batch's sequence
+// number into the request's completion word in pinned host memory, so the
+// host sees each request complete without waiting for the rest of its batch,
+// and the stream's next request may run in a batch that fills the SMs while
+// this one drains.  Every kernel and pattern counts in the lane-private table,
+// so nothing that the epilogue does after that has to be waited for: the
+// totals are added to, and the rest of the stream's state follows from its
+// last two requests' histograms alone, each of which writes a record of its
+// own (SrvRec), then the request's state word.  A batch whose words are all
+// there is done: its slot (its scratch and its bytes of the budget) is
+// released without a driver call.
 #include <cuda_runtime.h>
 #include <stddef.h>
 #include <stdint.h>
@@ -67,36 +69,36 @@ constexpr int kEpiBar = 1 + kGroups;  // named barrier of the threads of a CTA's
 // dynamic shared memory: the groups' tables in a batch with groups, else one
 constexpr size_t kSrvSmem = (size_t)kTableWords * 4;
 constexpr size_t kSrvGroupSmem = kGroups * kSrvSmem;
-// request-table capacities of the two kernel variants (the table travels in
-// the launch's parameters: 24 bytes per request)
-constexpr uint32_t kSmallCap = 32;
+// request-table capacities of the kernel variants (the table travels in the
+// launch's parameters, 24 bytes per request; from the launch call to a word
+// seen on the host, an empty kernel takes 7.6 us with few parameters, 8.7 with
+// 9.6 KB, 10.2 with 28 KB)
+constexpr uint32_t kSmallCap = 32, kMidCap = 256;
 
 __host__ __device__ __forceinline__ unsigned long long srv_cost(unsigned long long n) {
   return n + (n <= kSmallReq ? kSmallReqCost : kReqCost);
 }
 
-// Per-stream state on the device.  The two patterns sit in two slots: the
-// next request's in pat[cur], the last request's in the other; a request's
-// epilogue writes the new pattern over the older one and flips cur, so no
-// pattern is ever copied.  ctl holds the switch (bit 0) and cur (bit 1).
+// Per-stream state on the device: the totals, and the records of the stream's
+// last two requests, request c's (from 0) in rec[c & 1].  The state is the
+// last record's, with the pattern and the kernel choice of the one before.
+// Admission of request c waits for request c - 2's state word, so a record is
+// never written by two requests at a time.
+struct SrvRec {
+  uint32_t hist[HIST_BINS];
+  hist_pattern pat;  // derived from it
+  uint32_t flag;     // the switch after it
+};
 struct SrvStream {
   unsigned long long totals[HIST_BINS];
-  uint32_t last_hist[HIST_BINS];
-  hist_pattern pat[2];
-  unsigned long long chunks;
-  uint32_t ctl;
-  uint32_t last_kernel;  // kernel the last request ran
+  SrvRec rec[2];
 };
-
-__host__ __device__ __forceinline__ uint32_t srv_ctl(uint32_t flag, uint32_t cur) {
-  return (flag & 1u) | ((cur & 1u) << 1);
-}
 
 struct SrvReq {
   const uint8_t* in;
   uint32_t* out;
   uint32_t n;
-  uint32_t stream;
+  uint32_t stream;  // 2 stream + the request's record
 };
 
 // Per batch slot, on the device.  Both return to zero when a request's
@@ -116,8 +118,6 @@ struct SrvCommon {
   uint32_t count;
   uint32_t budget;
   uint32_t theta;
-  uint32_t mode;
-  uint32_t pad;
 };
 
 template <uint32_t CAP>
@@ -126,10 +126,6 @@ struct SrvArgs {
   RangePlan plan;
   SrvReq req[CAP];
 };
-
-__device__ __forceinline__ uint32_t srv_kernel_for(uint32_t mode, uint32_t flag) {
-  return mode == HIST_MODE_AUTO ? flag : (mode == HIST_MODE_PLAIN ? HIST_FLAG_PLAIN : HIST_FLAG_ADAPTIVE);
-}
 
 // A piece of a request, bytes [b0, e0) (e0 = 0: an empty request), as the CTAs
 // keep it in shared memory (the table sits in the kernel's parameters, read
@@ -157,18 +153,14 @@ struct SrvShared {
   uint32_t geh[kGroups][HIST_BINS];
 };
 
-// Request r of stream `sid` (n bytes) is complete, threads t = 0..255 (which
-// share named barrier `id`) hold a bin each in h: write its output and publish
-// the request's completion word, then advance its stream's state.  The state
-// can follow the completion: the stream's next request is admitted only once
-// the state word below has been seen.  The state is read at L2: it was
-// written by another batch's epilogue, possibly while an older batch that
-// read it on this SM is still resident.
-__device__ __noinline__ void srv_epilogue(const SrvCommon& a, uint32_t r, uint32_t sid, uint32_t n, uint32_t* out,
+// Request r (n bytes) is complete, threads t = 0..255 (which share named
+// barrier `id`) hold a bin each in h: write its output and publish the
+// request's completion word, then add to its stream's totals, write its record
+// (`sr`: SrvReq::stream) and publish its state word.
+__device__ __noinline__ void srv_epilogue(const SrvCommon& a, uint32_t r, uint32_t sr, uint32_t n, uint32_t* out,
                                           uint32_t h, EpiShared& es, int t, int id) {
-  SrvStream* st = a.streams + sid;
+  SrvStream* st = a.streams + (sr >> 1);
   const GroupBar<HIST_BINS> bar = {id};
-  const uint32_t ctl = __ldcg(&st->ctl);
   if (out) out[t] = h;
   // the output precedes the completion word: the barrier orders the threads'
   // writes before thread 0's system-scope release store, whose release is
@@ -178,21 +170,13 @@ __device__ __noinline__ void srv_epilogue(const SrvCommon& a, uint32_t r, uint32
   if (t == 0)
     asm volatile("st.release.sys.global.u32 [%0], %1;" ::"l"(a.done + r), "r"(a.seq) : "memory");
   if (h) atomicAdd(&st->totals[t], (unsigned long long)h);
-  st->last_hist[t] = h;
+  SrvRec* rec = st->rec + (sr & 1u);
+  rec->hist[t] = h;
   BinPlace place;
   const hist_degeneracy_result d = block_pattern(h, n, a.budget, a.theta, es, t, bar, place);
-  // the new pattern replaces the older of the two
-  const uint32_t cur = (ctl >> 1) & 1u;
-  store_place(st->pat[cur ^ 1u], t, a.budget, place);
-  if (t == 0) {
-    st->ctl = srv_ctl(d.flag, cur ^ 1u);
-    st->last_kernel = srv_kernel_for(a.mode, ctl & 1u);
-    atomicAdd(&st->chunks, 1ull);  // at L2, like every other read of the state
-  }
-  // the stream's state is written: its state word releases the stream to
-  // the host's admission, so that its next request may run in a batch that
-  // starts while this one is still counting (the same release argument as
-  // for the completion word)
+  store_place(rec->pat, t, a.budget, place);
+  if (t == 0) rec->flag = d.flag;
+  // (the same release argument as for the completion word)
   bar.sync();
   if (t == 0)
     asm volatile("st.release.sys.global.u32 [%0], %1;" ::"l"(a.done + kSrvMaxBatch + r), "r"(a.seq) : "memory");
@@ -314,26 +298,19 @@ __device__ __forceinline__ void srv_window(const SrvArgs<CAP>& args, uint32_t r0
   __syncthreads();
 }
 
-// The groups' requests [i0, i0 + kSrvItems) of the list (first >= 0: first,
-// first + 1, ...; else ss.wl) into ss.items, a warp per request.
-template <uint32_t CAP>
-__device__ __forceinline__ void srv_items(const SrvArgs<CAP>& args, uint32_t nwl, int first, uint32_t i0,
-                                          SrvShared& ss) {
-  for (uint32_t k = threadIdx.x >> 5; k < kSrvItems && i0 + k < nwl; k += kWarps) {
-    const uint32_t r = first >= 0 ? (uint32_t)first + i0 + k : ss.wl[i0 + k];
-    const SrvReq q = args.req[r];
-    if ((threadIdx.x & 31) == 0) {
-      const Split sp = split_bytes(q.in, q.n);
-      GroupItem it;
-      it.body = reinterpret_cast<const uint4*>(q.in + sp.head);
-      it.out = q.out;
-      it.nvec = (uint32_t)sp.nvec;
-      it.n = q.n;
-      it.j = q.stream;
-      it.edges = (uint32_t)sp.head | ((uint32_t)sp.tail << 8);
-      ss.items[k] = it;
-      ss.item_r[k] = r;
-    }
+// Request r of the batch as the groups' k-th item.  A warp calls.
+__device__ __forceinline__ void srv_item(const SrvReq& q, uint32_t r, uint32_t k, SrvShared& ss) {
+  if ((threadIdx.x & 31) == 0) {
+    const Split sp = split_bytes(q.in, q.n);
+    GroupItem it;
+    it.body = reinterpret_cast<const uint4*>(q.in + sp.head);
+    it.out = q.out;
+    it.nvec = (uint32_t)sp.nvec;
+    it.n = q.n;
+    it.j = q.stream;
+    it.edges = (uint32_t)sp.head | ((uint32_t)sp.tail << 8);
+    ss.items[k] = it;
+    ss.item_r[k] = r;
   }
 }
 
@@ -372,8 +349,12 @@ __device__ __forceinline__ void srv_group(const SrvCommon& a, uint32_t count, ui
 // on single requests.  Before -- per-warp tables for the streams the switch
 // called plain, the default pattern's slot lookup for first requests, a cost
 // prefix with 64-bit divisions in every CTA -- and now: a burst of 600
-// requests of 4 KiB .. 64 MiB on 256 streams 1320 -> 767 us, one of 4000 3.48
-// -> 6.0 TB/s; at 50k requests/s p50 18.3 -> 14.2 us, p99 40.7 -> 26.8.
+// requests of 4 KiB .. 64 MiB on 256 streams 1320 -> 740 us, one of 4000 3.48
+// -> 6.1 TB/s; at 50k requests/s p50 18.3 -> 13.5 us, p99 40.7 -> 25.8.  Where
+// streams have many requests waiting, the chain of a stream's requests bounds,
+// 12 us a request: 600 of 1 .. 8 KiB on 16 streams 788 us with the stream held
+// until its state was written and an event per batch, 665 without, 636 with
+// the tables of only the groups that have a request cleared.
 template <uint32_t CAP>
 __global__ void __launch_bounds__(kThreads, 1) server_batch_kernel(const __grid_constant__ SrvArgs<CAP> args) {
   extern __shared__ __align__(16) uint32_t tables[];
@@ -403,38 +384,44 @@ __global__ void __launch_bounds__(kThreads, 1) server_batch_kernel(const __grid_
     first = -1;
   }
   if (nwl == 0) return;
-  __syncthreads();
+  const uint32_t w = (uint32_t)t >> 5;
+  auto number = [&](uint32_t k) { return first >= 0 ? (uint32_t)first + k : (uint32_t)ss.wl[k]; };
+  // (a request's parameters arrive while the groups that have one clear their
+  // tables)
+  const uint32_t r = w < nwl ? number(w) : 0;
+  const SrvReq q = w < nwl ? args.req[r] : SrvReq{nullptr, nullptr, 0, 0};
+  if (!groups) __syncthreads();
   {
     const int g = t / kGroupThreads, gt = t % kGroupThreads;
     uint4* t4 = reinterpret_cast<uint4*>(tables + (size_t)g * kTableWords);
+    if ((uint32_t)g < nwl) {
 #pragma unroll
-    for (int i = 0; i < kTableWords / 4 / kGroupThreads; ++i) t4[gt + i * kGroupThreads] = make_uint4(0, 0, 0, 0);
+      for (int i = 0; i < kTableWords / 4 / kGroupThreads; ++i) t4[gt + i * kGroupThreads] = make_uint4(0, 0, 0, 0);
+    }
     ss.geh[g][gt] = 0;
   }
+  if (w < nwl) srv_item(q, r, w, ss);
   for (uint32_t i0 = 0; i0 < nwl; i0 += kSrvItems) {
     if (i0) __syncthreads();
-    srv_items(args, nwl, first, i0, ss);
+    for (uint32_t k = w; k < kSrvItems && i0 + k < nwl; k += kWarps)
+      if (i0 || k >= kWarps) srv_item(args.req[number(i0 + k)], number(i0 + k), k, ss);
     __syncthreads();
     srv_group(a, nwl - i0 < kSrvItems ? nwl - i0 : kSrvItems, tables, ss);
   }
 }
 
-// Every stream starts with no chunks, the plain kernel and the default
-// pattern (one CTA).
+// Every stream starts with the plain kernel and the default pattern, in both
+// records (one CTA).
 __global__ void __launch_bounds__(HIST_BINS) server_init_kernel(SrvStream* s, uint32_t streams, uint32_t budget) {
   __shared__ EpiShared es;
   const int t = threadIdx.x;
   BinPlace place;
   block_pattern(0u, 0ull, budget, HIST_THETA_MILLI_DEFAULT, es, t, CtaBar(), place);
-  for (uint32_t i = 0; i < streams; ++i) {
-    SrvStream* st = s + i;
-    store_place(st->pat[0], t, budget, place);
-    store_place(st->pat[1], t, budget, place);
-    if (t == 0) {
-      st->ctl = srv_ctl(HIST_FLAG_PLAIN, 0u);
-      st->last_kernel = HIST_FLAG_PLAIN;
+  for (uint32_t i = 0; i < streams; ++i)
+    for (int k = 0; k < 2; ++k) {
+      store_place(s[i].rec[k].pat, t, budget, place);
+      if (t == 0) s[i].rec[k].flag = HIST_FLAG_PLAIN;
     }
-  }
 }
 
 uint64_t now_ns() {
@@ -452,11 +439,17 @@ struct PendingReq {
   uint64_t submit_ns;
 };
 
+// A stream as the host sees it.
+struct HostStream {
+  uint64_t admitted = 0;   // requests put on the GPU
+  uint64_t scan = 0;       // the last admission scan that met the stream
+  bool busy = false;       // the last one's completion has not been returned
+  bool owed[2] = {false, false};  // a request that writes record k has not published its state word
+};
+
 struct BatchSlot {
   bool busy = false;
-  bool waited = false;  // completed by a host wait (its event could not be recorded)
   cudaStream_t cs = nullptr;
-  cudaEvent_t done = nullptr;
   SrvSlot* d_slot = nullptr;
   // completion words of the batch's requests, then their state words
   // (pinned, mapped: 2 kSrvMaxBatch words)
@@ -464,8 +457,9 @@ struct BatchSlot {
   uint32_t* d_done = nullptr;  // the same words as the device sees them
   uint32_t seq = 0;            // the running batch's sequence number
   std::vector<PendingReq> reqs;
+  std::vector<uint8_t> rec;       // the record that the request writes
   std::vector<uint8_t> reported;  // the request's completion has been returned
-  std::vector<uint8_t> released;  // the request's stream has gone back to admission
+  std::vector<uint8_t> released;  // the request's state word has been seen
   uint32_t n_reported = 0;
   uint32_t n_released = 0;
   uint32_t polls = 0;  // polls of the running batch
@@ -478,9 +472,8 @@ struct BatchSlot {
 struct hist_server {
   hist_server_config cfg;
   SrvStream* d_streams = nullptr;
-  std::vector<uint8_t> stream_busy;  // a request of the stream is on the GPU
-  std::vector<uint64_t> scan_mark;   // the stream was passed over in admission scan #mark
-  uint64_t scan = 0;
+  std::vector<HostStream> streams;
+  uint64_t scan = 0;  // number of the last admission scan
   std::list<PendingReq> queue;  // FIFO; admission erases from the middle
   std::vector<std::list<PendingReq>::iterator> pick;  // the admission scan's requests
   BatchSlot slot[kSrvMaxSlots];
@@ -503,34 +496,33 @@ bool server_config_ok(const hist_server_config* c) {
 }
 
 // Return the completions of finished requests -- those whose completion word
-// holds their batch's sequence number, and every request of a batch whose
-// event shows it done -- writing at most `cap` of them to `out` (out null:
-// discard them); give a returned request's stream back to admission once its
-// state word holds the number too, and release the slots of finished
-// batches; returns how many completions were written or discarded.
+// holds their batch's sequence number -- writing at most `cap` of them to
+// `out` (out null: discard them), which gives their streams back to admission,
+// and release the slots of the batches whose words are all there; returns how
+// many completions were written or discarded.
 uint32_t retire(hist_server* s, hist_completion* out, uint32_t cap, int* err) {
   uint32_t n = 0;
   for (uint32_t k = 0; k < s->cfg.max_inflight; ++k) {
     BatchSlot& f = s->slot[k];
     if (!f.busy) continue;
     const uint32_t count = (uint32_t)f.reqs.size();
-    // the event is asked (a driver call) once every request's stream has
-    // been released, and every 32nd poll before that, so that a failed batch
-    // is still seen; the words themselves are plain reads of host memory
-    cudaError_t q = cudaErrorNotReady;
-    if (f.waited) q = cudaSuccess;
-    else if (f.n_released == count || (++f.polls & 31u) == 0) q = cudaEventQuery(f.done);
-    if (q != cudaSuccess && q != cudaErrorNotReady) {
-      *err = cuda_fail(q);
-      return n;
+    // the words are plain reads of host memory; the driver is asked every
+    // 32nd poll, so that a failed batch is still seen
+    bool all = false;
+    if ((++f.polls & 31u) == 0) {
+      const cudaError_t q = cudaStreamQuery(f.cs);
+      if (q != cudaSuccess && q != cudaErrorNotReady) {
+        *err = cuda_fail(q);
+        return n;
+      }
+      all = q == cudaSuccess;
     }
-    const bool all = q == cudaSuccess;
-    for (uint32_t i = 0; i < count && f.n_released < count; ++i) {
+    for (uint32_t i = 0; i < count; ++i) {
       const PendingReq& r = f.reqs[i];
-      if (!f.reported[i]) {
-        // the acquire pairs with the epilogue's release: the request's
-        // output is written before its completion word is
-        if ((out && n >= cap) || (!all && __atomic_load_n(f.h_done + i, __ATOMIC_ACQUIRE) != f.seq)) continue;
+      HostStream& h = s->streams[r.stream];
+      // (the acquires pair with the epilogue's releases: what it writes
+      // before a word is written when the word is seen)
+      if (!f.reported[i] && !(out && n >= cap) && (all || __atomic_load_n(f.h_done + i, __ATOMIC_ACQUIRE) == f.seq)) {
         if (out) {
           hist_completion& c = out[n];
           c.tag = r.tag;
@@ -542,23 +534,21 @@ uint32_t retire(hist_server* s, hist_completion* out, uint32_t cap, int* err) {
           c.done_ns = now_ns();
         }
         ++n;
+        h.busy = false;
         f.reported[i] = 1;
         f.n_reported += 1;
         s->stats.completed += 1;
         s->stats.bytes += r.n;
       }
-      // the stream's state is written before its state word is; a stream
-      // goes back only after its request's completion has been returned, so
-      // a stream's completions are returned in its order
-      if (f.released[i] ||
-          (!all && __atomic_load_n(f.h_done + kSrvMaxBatch + i, __ATOMIC_ACQUIRE) != f.seq))
-        continue;
-      s->stream_busy[r.stream] = 0;
-      f.released[i] = 1;
-      f.n_released += 1;
+      if (!f.released[i] && (all || __atomic_load_n(f.h_done + kSrvMaxBatch + i, __ATOMIC_ACQUIRE) == f.seq)) {
+        h.owed[f.rec[i]] = false;
+        f.released[i] = 1;
+        f.n_released += 1;
+      }
     }
-    if (!all || f.n_released < count) continue;
-    // the whole batch is done: its bytes go back to admission
+    if (f.n_reported < count || f.n_released < count) continue;
+    // the whole batch is done (the next one in this slot follows it on the
+    // slot's CUDA stream): its bytes go back to admission
     s->inflight_bytes -= f.bytes;
     f.reqs.clear();
     f.busy = false;
@@ -568,7 +558,8 @@ uint32_t retire(hist_server* s, hist_completion* out, uint32_t cap, int* err) {
 
 // Launch one batch if a slot is free and the queue holds admissible requests.
 // FIFO order; only each stream's first queued request is a candidate, and
-// only if the stream has no request on the GPU; the scan stops at the first
+// only if the completion of the stream's last request has been returned and
+// its record is free; the scan stops at the first
 // candidate that does not fit the byte budget, so no request waits forever
 // behind smaller later ones; it ends once every stream has been met.  A
 // batch is launched whatever its size: one formed while the batches on the
@@ -590,10 +581,11 @@ int admit(hist_server* s) {
   for (auto it = s->queue.begin();
        it != s->queue.end() && s->pick.size() < s->cfg.max_batch && met < s->cfg.streams; ++it) {
     const PendingReq& r = *it;
-    if (s->scan_mark[r.stream] == mark) continue;  // not the stream's first: keep its order
-    s->scan_mark[r.stream] = mark;
+    HostStream& h = s->streams[r.stream];
+    if (h.scan == mark) continue;  // not the stream's first: keep its order
+    h.scan = mark;
     ++met;
-    if (s->stream_busy[r.stream]) continue;
+    if (h.busy || h.owed[h.admitted & 1u]) continue;
     if (s->inflight_bytes + bytes + r.n > s->cfg.hbm_budget) {
       s->stats.deferred += 1;
       break;
@@ -605,7 +597,6 @@ int admit(hist_server* s) {
   f->reqs.clear();
   f->bytes = bytes;
   for (const auto& it : s->pick) {
-    s->stream_busy[it->stream] = 1;
     f->reqs.push_back(*it);
     s->queue.erase(it);
   }
@@ -615,6 +606,7 @@ int admit(hist_server* s) {
   f->seq = s->seq;
   f->reported.assign(count, 0);
   f->released.assign(count, 0);
+  f->rec.resize(count);
   f->n_reported = 0;
   f->n_released = 0;
   f->polls = 0;
@@ -626,13 +618,15 @@ int admit(hist_server* s) {
   a->c.count = count;
   a->c.budget = s->cfg.pattern_budget;
   a->c.theta = s->cfg.theta_milli;
-  a->c.mode = s->cfg.mode;
   for (uint32_t i = 0; i < count; ++i) {
     const PendingReq& r = f->reqs[i];
+    HostStream& h = s->streams[r.stream];
+    f->rec[i] = (uint8_t)(h.admitted++ & 1u);
+    h.busy = h.owed[f->rec[i]] = true;
     a->req[i].in = r.in;
     a->req[i].out = r.out;
     a->req[i].n = (uint32_t)r.n;
-    a->req[i].stream = r.stream;
+    a->req[i].stream = 2 * r.stream + f->rec[i];
   }
   PlanCosts<kSrvMaxBatch> pc;
   auto size = [&](uint32_t i) { return (unsigned long long)a->req[i].n; };
@@ -641,32 +635,29 @@ int admit(hist_server* s) {
   if (grid > (unsigned long long)s->max_grid) grid = (unsigned long long)s->max_grid;
   if (grid < 1) grid = 1;
   plan_ranges(&a->plan, pc, count, (uint32_t)grid, kSmallReq, size);
-  // the small variant's parameters are a prefix of the large one's
-  static_assert(offsetof(SrvArgs<kSmallCap>, req) == offsetof(SrvArgs<kSrvMaxBatch>, req), "parameter layout");
+  // the smaller variants' parameters are a prefix of the large one's
+  static_assert(offsetof(SrvArgs<kSmallCap>, req) == offsetof(SrvArgs<kSrvMaxBatch>, req) &&
+                    offsetof(SrvArgs<kMidCap>, req) == offsetof(SrvArgs<kSrvMaxBatch>, req),
+                "parameter layout");
   static_assert(sizeof(SrvArgs<kSrvMaxBatch>) <= 32764, "kernel parameters are limited to 32764 bytes");
   void* params[] = {a};
   const void* fn = count <= kSmallCap ? (const void*)server_batch_kernel<kSmallCap>
+                   : count <= kMidCap ? (const void*)server_batch_kernel<kMidCap>
                                       : (const void*)server_batch_kernel<kSrvMaxBatch>;
   cudaError_t e = cudaLaunchKernel(fn, dim3((unsigned)grid), dim3(kThreads), params,
                                    a->plan.group_max ? kSrvGroupSmem : kSrvSmem, f->cs);
   if (e != cudaSuccess) {
     // nothing was enqueued: the requests go back to the head of the queue
-    for (const PendingReq& r : f->reqs) s->stream_busy[r.stream] = 0;
+    for (uint32_t i = 0; i < count; ++i) {
+      HostStream& h = s->streams[f->reqs[i].stream];
+      h.admitted -= 1;
+      h.busy = h.owed[f->rec[i]] = false;
+    }
     s->queue.insert(s->queue.begin(), f->reqs.begin(), f->reqs.end());
     f->reqs.clear();
     return cuda_fail(e);
   }
   f->busy = true;
-  e = cudaEventRecord(f->done, f->cs);
-  f->waited = e != cudaSuccess;
-  if (f->waited) {
-    // no completion event: wait for the batch here so that it still retires
-    cudaStreamSynchronize(f->cs);
-    f->admit_ns = now_ns();
-    s->inflight_bytes += f->bytes;
-    s->stats.batches += 1;
-    return cuda_fail(e);
-  }
   f->admit_ns = now_ns();
   s->inflight_bytes += f->bytes;
   s->stats.batches += 1;
@@ -702,13 +693,13 @@ int hist_server_create(const hist_server_config* cfg, hist_server** out) {
   hist_server* s = new (std::nothrow) hist_server();
   if (!s) return HIST_ENOMEM;
   s->cfg = *cfg;
-  s->stream_busy.assign(cfg->streams, 0);
-  s->scan_mark.assign(cfg->streams, 0);
+  s->streams.resize(cfg->streams);
   s->sms = sm_count();
   memset(&s->stats, 0, sizeof(s->stats));
-  static int attr_small[kMaxDevices], attr_large[kMaxDevices];
+  static int attr_small[kMaxDevices], attr_mid[kMaxDevices], attr_large[kMaxDevices];
   int rc = s->sms > 0 ? HIST_OK : HIST_ECUDA;
   if (rc == HIST_OK) rc = ensure_smem_attr_bytes((const void*)server_batch_kernel<kSmallCap>, attr_small, kSrvGroupSmem);
+  if (rc == HIST_OK) rc = ensure_smem_attr_bytes((const void*)server_batch_kernel<kMidCap>, attr_mid, kSrvGroupSmem);
   if (rc == HIST_OK) rc = ensure_smem_attr_bytes((const void*)server_batch_kernel<kSrvMaxBatch>, attr_large, kSrvGroupSmem);
   if (rc == HIST_OK) {
     int per_sm = 0;
@@ -731,7 +722,6 @@ int hist_server_create(const hist_server_config* cfg, hist_server** out) {
       f.h_done = s->h_done + (size_t)k * 2 * kSrvMaxBatch;
       e = cudaHostGetDevicePointer((void**)&f.d_done, f.h_done, 0);
       if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&f.cs, cudaStreamNonBlocking);
-      if (e == cudaSuccess) e = cudaEventCreateWithFlags(&f.done, cudaEventDisableTiming);
       if (e == cudaSuccess) e = cudaMalloc((void**)&f.d_slot, sizeof(SrvSlot));
       if (e == cudaSuccess) e = cudaMemset(f.d_slot, 0, sizeof(SrvSlot));
     }
@@ -763,7 +753,6 @@ int hist_server_destroy(hist_server* s) {
   for (uint32_t k = 0; k < kSrvMaxSlots; ++k) {
     BatchSlot& f = s->slot[k];
     if (f.d_slot) cudaFree(f.d_slot);
-    if (f.done) cudaEventDestroy(f.done);
     if (f.cs) cudaStreamDestroy(f.cs);
   }
   if (s->d_streams) cudaFree(s->d_streams);
@@ -815,13 +804,18 @@ int hist_server_stream_state(hist_server* s, uint32_t stream, hist_stream_state*
   if (e != cudaSuccess) return cuda_fail(e);
   memset(h, 0, sizeof(*h));
   memcpy(h->totals, tmp.totals, sizeof(h->totals));
-  memcpy(h->last_hist, tmp.last_hist, sizeof(h->last_hist));
-  const uint32_t cur = (tmp.ctl >> 1) & 1u;
-  h->pattern = tmp.pat[cur];
-  h->last_pattern = tmp.pat[cur ^ 1u];
-  h->chunks = tmp.chunks;
-  h->flag = tmp.ctl & 1u;
-  h->last_kernel = tmp.last_kernel;
+  const uint64_t c = s->streams[stream].admitted;
+  const SrvRec& last = tmp.rec[(c & 1u) ^ 1u];
+  const SrvRec& before = tmp.rec[c & 1u];
+  memcpy(h->last_hist, last.hist, sizeof(h->last_hist));
+  h->pattern = last.pat;
+  h->last_pattern = before.pat;
+  h->chunks = c;
+  h->flag = last.flag;
+  // the last request ran the kernel chosen from the one before
+  h->last_kernel = c == 0 || s->cfg.mode == HIST_MODE_PLAIN ? HIST_FLAG_PLAIN
+                   : s->cfg.mode == HIST_MODE_AUTO          ? before.flag
+                                                            : HIST_FLAG_ADAPTIVE;
   return HIST_OK;
 }
 
@@ -870,7 +864,7 @@ int hist_server_replay(hist_server* s, const hist_request* reqs, uint32_t count,
     }
     done += n;
   }
-  // every request has completed; the last batches retire once their events fire
+  // every request has completed; the last batches retire with their state words
   while (!server_idle(s)) {
     if (timeout_ms && now_ns() - t0 > (uint64_t)timeout_ms * 1000000ull) return HIST_ETIMEDOUT;
     int err = HIST_OK;

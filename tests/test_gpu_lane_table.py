@@ -1,5 +1,7 @@
 """The lane-private counting paths at the sizes where their splits change,
 against the oracle, bit-exact."""
+import time
+
 import numpy as np
 import pytest
 import torch
@@ -286,3 +288,61 @@ def test_server_requests_around_the_groups_limit(mode, budget):
             assert s.flag == refs[i].flag and s.last_kernel == rec.kernel and s.chunks == rnd + 1
             assert np.array_equal(np.array(s.totals, np.uint64), refs[i].totals)
     srv.close()
+
+
+@pytest.mark.parametrize("streams,max_batch,max_inflight", [(1, 256, 4), (3, 1, 8), (3, 7, 4), (5, 1024, 8), (40, 64, 2)])
+def test_server_long_queues_of_few_streams(streams, max_batch, max_inflight):
+    """More queued requests than streams: a stream's next request is launched
+    while the last one may still be writing its record.  Some requests write
+    where an earlier one of their stream wrote, or read what it wrote: the
+    outputs, the completions' order and the states are those of the stream's
+    order."""
+    rng = np.random.default_rng(streams * 1000 + max_batch)
+    x = rng.integers(0, 256, 2_000_000, dtype=np.uint8)
+    x[rng.random(x.size) < 0.46] = 9  # near the switch's threshold
+    xd = dev(x)
+    for mode in (hl.MODE_AUTO, hl.MODE_ADAPTIVE, hl.MODE_PLAIN):
+        srv = hl.Server(streams=streams, mode=mode, max_batch=max_batch, max_inflight=max_inflight)
+        refs = [oracle.StreamOracle(oracle.BUDGET_MAX, mode=mode) for _ in range(streams)]
+        count = 400
+        outs = torch.full((count, 256), -1, dtype=torch.int32, device="cuda")
+        host = np.full((count, 256), 0xffffffff, np.uint32)
+        rows = [[] for _ in range(streams)]  # each stream's output rows
+        last = [None] * streams
+        torch.cuda.synchronize()
+        for i in range(count):
+            s = int(rng.integers(0, streams))
+            row, n, off = i, int(rng.choice([0, 5, 1000, 30_000, 200_000, 500_000])), int(rng.integers(0, 1_000_000))
+            ptr, data = xd.data_ptr() + off, x[off:off + n]
+            k = int(rng.integers(0, 12))
+            if k == 0 and rows[s]:  # over an earlier output
+                row = rows[s][-1]
+            elif k == 1 and rows[s]:  # from an earlier output, from inside it to its end
+                at = rows[s][-int(rng.integers(1, min(4, len(rows[s])) + 1))]
+                ptr, n = outs[at].data_ptr() + 100, 924
+                data = np.ascontiguousarray(host[at]).view(np.uint8)[100:].copy()
+            last[s] = refs[s].push(data)
+            host[row] = last[s].hist
+            rows[s].append(row)
+            srv.submit_ptr(s, ptr, n, outs[row].data_ptr(), i)
+        order = [[] for _ in range(streams)]
+        got = 0
+        t0 = time.monotonic()
+        while got < count:
+            assert time.monotonic() - t0 < 20
+            for c in srv.poll():
+                order[c.stream].append(c.tag)
+                got += 1
+        srv.drain(20000)
+        assert all(o == sorted(o) for o in order)
+        assert np.array_equal(u32(outs).reshape(count, 256), host)
+        for s in range(streams):
+            if last[s] is None:
+                continue
+            st = srv.stream_state(s)
+            assert bytes(st.pattern) == refs[s].pattern.to_bytes()
+            assert bytes(st.last_pattern) == last[s].pattern.to_bytes()
+            assert np.array_equal(np.array(st.last_hist, np.uint32), last[s].hist)
+            assert np.array_equal(np.array(st.totals, np.uint64), refs[s].totals)
+            assert st.flag == refs[s].flag and st.last_kernel == last[s].kernel and st.chunks == refs[s].chunks
+        srv.close()
