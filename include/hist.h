@@ -413,9 +413,10 @@ int hist_batch_classify(const uint8_t* const* d_ptrs, const size_t* d_sizes, uin
                         uint8_t* d_regime, hist_cuda_stream s);
 
 /* hist_batch with a per-regime table: hist_batch_classify into d_regime
- * (count bytes on the device, the caller's; the regimes stay there), then
+ * (count bytes on the device, the caller's; the regimes stay there) and
  * hist_batch's launches, in which each image is counted with its regime's
- * setting.  No other device memory.
+ * setting (a table of layout 5 throughout, the default, counts first and
+ * classifies behind it).  No other device memory.
  * table null = hist_batch_table_init.  HIST_EINVAL for a bad table. */
 int hist_batch_regimes(const uint8_t* const* d_ptrs, const size_t* d_sizes, uint32_t count, uint32_t* d_out,
                        uint8_t* d_regime, const hist_batch_table* table, hist_cuda_stream s);

@@ -542,32 +542,55 @@ __global__ void __launch_bounds__(kThreads, 1) batch_lane_kernel(const __grid_co
 }
 
 // The regime of image blockIdx.x (rule in hist.h): 256 threads; thread t
-// takes run t of the sample (16 consecutive pixels from floor(t n / 256)),
-// or pixels t, t + 256, ... of an image of at most 4096 pixels, loading all
-// 16 bytes before counting them in shared memory; then the largest bin and
-// the sum of squares (below 2^25: m <= 4096).
+// takes run t of the sample (16 consecutive pixels from floor(t n / 256)), or
+// pixels 16 t .. 16 t + 15 of an image of at most 4096 pixels, as the five
+// words that hold them (byte by byte where one of the words is not all the
+// image's), counts them in shared memory; then the largest bin and the sum of
+// squares (below 2^25: m <= 4096).  With `after` the launch follows the
+// batch's counting launches and fills the SMs as their CTAs end: they started
+// after the work before the call was complete, and this one ends after them.
+// Bound by latency (the arrays, the pixels, three barriers) and the shared
+// atomics' conflicts.  With a byte load per pixel, before the counting
+// launches, and now: the regimes call on 2227 images of 17 .. 375 a side 38.0
+// -> 33.0 us (28.8 without regimes), on 300 of 64 .. 2000 45.0 -> 41.1 (41.1);
+// words, but before the counting launches, 35.0 and 43.2.
 __global__ void __launch_bounds__(HIST_BINS) regime_kernel(const uint8_t* const* ptrs, const size_t* sizes,
-                                                           uint32_t theta, uint8_t* regime) {
+                                                           uint32_t theta, uint8_t* regime, bool after) {
   __shared__ uint32_t h[HIST_BINS];
   __shared__ uint32_t wmax[HIST_BINS / 32], wsq[HIST_BINS / 32];
   const int t = threadIdx.x;
   const uint32_t i = blockIdx.x;
+  if (!after) pdl_wait();
+  pdl_launch_dependents();
   const unsigned long long n = sizes[i];
   const uint8_t* x = ptrs[i];
   h[t] = 0;
-  uint32_t v[16];
   const bool runs = n > HIST_REGIME_SAMPLE;
-  const unsigned long long start = runs ? ((unsigned long long)t * n) >> 8 : (unsigned long long)t;
-  const unsigned long long step = runs ? 1ull : (unsigned long long)HIST_BINS;
+  const unsigned long long start = runs ? ((unsigned long long)t * n) >> 8 : 16ull * (unsigned long long)t;
+  const int len = start >= n ? 0 : n - start < 16 ? (int)(n - start) : 16;
+  const uint8_t* p = x + start;
+  const uint32_t off = (uint32_t)((uintptr_t)p & 3u);
+  const bool whole = len == 16 && start >= off && start - off + 20 <= n;
+  uint32_t v[5];
+  if (whole) {
+    const uint32_t* q = reinterpret_cast<const uint32_t*>(p - off);
 #pragma unroll
-  for (int u = 0; u < 16; ++u) {
-    const unsigned long long at = start + (unsigned long long)u * step;
-    v[u] = at < n ? (uint32_t)__ldg(x + at) : 0xffffffffu;
+    for (int u = 0; u < 5; ++u) v[u] = __ldg(q + u);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) v[u] = __funnelshift_r(v[u], v[u + 1], 8 * off);
+  } else {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      v[u] = 0;
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (4 * u + k < len) v[u] |= (uint32_t)__ldg(p + 4 * u + k) << (8 * k);
+    }
   }
   __syncthreads();
 #pragma unroll
   for (int u = 0; u < 16; ++u)
-    if (v[u] != 0xffffffffu) atomicAdd(&h[v[u]], 1u);
+    if (u < len) atomicAdd(&h[(v[u >> 2] >> (8 * (u & 3))) & 0xffu], 1u);
   __syncthreads();
   const uint32_t c = h[t];
   const uint32_t mx = __reduce_max_sync(0xffffffffu, c);
@@ -590,14 +613,25 @@ __global__ void __launch_bounds__(HIST_BINS) regime_kernel(const uint8_t* const*
     else if (64ull * S >= m * m) r = (uint8_t)HIST_REGIME_PEAKED;
     regime[i] = r;
   }
+  if (after) pdl_wait();
 }
 
+// `after`: the launches before on the stream are this batch's counting ones,
+// which read no regime (else they are any work, which it waits for).
 int launch_regimes(const uint8_t* const* d_ptrs, const size_t* d_sizes, uint32_t count, uint32_t theta,
-                   uint8_t* d_regime, cudaStream_t s) {
+                   uint8_t* d_regime, bool after, cudaStream_t s) {
   for (uint32_t first = 0; first < count; first += 65535u) {
-    const uint32_t c = count - first < 65535u ? count - first : 65535u;
-    regime_kernel<<<c, HIST_BINS, 0, s>>>(d_ptrs + first, d_sizes + first, theta, d_regime + first);
-    const cudaError_t e = cudaGetLastError();
+    cudaLaunchConfig_t lc = {};
+    cudaLaunchAttribute at[1];
+    lc.gridDim = dim3(count - first < 65535u ? count - first : 65535u);
+    lc.blockDim = dim3(HIST_BINS);
+    lc.stream = s;
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    lc.attrs = at;
+    lc.numAttrs = 1;
+    const cudaError_t e =
+        cudaLaunchKernelEx(&lc, regime_kernel, d_ptrs + first, d_sizes + first, theta, d_regime + first, after);
     if (e != cudaSuccess) return cuda_fail(e);
   }
   return HIST_OK;
@@ -736,13 +770,18 @@ hist_batch_tuning shape_of(const hist_batch_table& t) {
   return tu;
 }
 
-// The regimes call: memset, classification, counting.
+// The regimes call.  The lane-private launches count every image alike, so
+// they come first and the classification fills their tail.
 int batch_regimes(const uint8_t* const* d_ptrs, const size_t* d_sizes, uint32_t count, uint32_t* d_out,
                   uint8_t* d_regime, const hist_batch_table& tb, cudaStream_t s) {
   if (count == 0) return HIST_OK;
-  int rc = launch_regimes(d_ptrs, d_sizes, count, tb.theta_milli, d_regime, s);
-  if (rc) return rc;
-  return launch_batch_images(shape_of(tb), layouts_of(tb), d_regime, d_ptrs, d_sizes, count, d_out, s);
+  const RegimeLayouts lay = layouts_of(tb);
+  const bool after = lane_layouts(lay);
+  int rc = HIST_OK;
+  if (!after) rc = launch_regimes(d_ptrs, d_sizes, count, tb.theta_milli, d_regime, false, s);
+  if (rc == HIST_OK) rc = launch_batch_images(shape_of(tb), lay, d_regime, d_ptrs, d_sizes, count, d_out, s);
+  if (rc == HIST_OK && after) rc = launch_regimes(d_ptrs, d_sizes, count, tb.theta_milli, d_regime, true, s);
+  return rc;
 }
 
 // Capture `enqueue` (which enqueues on the stream it is given) into an
@@ -831,7 +870,7 @@ void hist_batch_table_init(hist_batch_table* t) {
 int hist_batch_classify(const uint8_t* const* d_ptrs, const size_t* d_sizes, uint32_t count, uint32_t theta_milli,
                         uint8_t* d_regime, hist_cuda_stream s) {
   if (theta_milli > 1000 || (count && (!d_ptrs || !d_sizes || !d_regime))) return HIST_EINVAL;
-  return launch_regimes(d_ptrs, d_sizes, count, theta_milli, d_regime, (cudaStream_t)s);
+  return launch_regimes(d_ptrs, d_sizes, count, theta_milli, d_regime, false, (cudaStream_t)s);
 }
 
 int hist_batch_regimes(const uint8_t* const* d_ptrs, const size_t* d_sizes, uint32_t count, uint32_t* d_out,
@@ -978,7 +1017,7 @@ extern "C" int hist_batch_autotune_regimes(const uint8_t* const* d_ptrs, const s
   std::vector<uint8_t> reg(count);
   std::vector<const uint8_t*> ptrs(count);
   std::vector<size_t> sizes(count);
-  int rc = launch_regimes(d_ptrs, d_sizes, count, tb.theta_milli, d_regime, s);
+  int rc = launch_regimes(d_ptrs, d_sizes, count, tb.theta_milli, d_regime, false, s);
   if (rc == HIST_OK) {
     e = cudaMemcpyAsync(reg.data(), d_regime, count, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(ptrs.data(), d_ptrs, count * sizeof(void*), cudaMemcpyDeviceToHost, s);

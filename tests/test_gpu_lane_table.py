@@ -259,6 +259,44 @@ def test_batch_lane_launches(name, sizes, out_shift):
     _batch(sizes, 17, 40, out_shift)
 
 
+@pytest.mark.parametrize("sizes", [
+    [0, 1, 15, 16, 17, 19, 20, 255, 4079, 4080, 4095, 4096, 4097, 4100, 4111, 4112, 5000] * 4,
+    [3000 + 401 * k for k in range(300)] + [2_000_003, 4096 * 256 + 1],
+])
+def test_regimes_behind_a_copy(sizes):
+    """Classification behind the counting launches, right after a copy wrote
+    the images and before another reads the regimes, images at every
+    alignment: the oracle's regimes and histograms, three times over."""
+    rng = np.random.default_rng(len(sizes))
+    offs = np.concatenate(([0], np.cumsum([n + 1 + k % 16 for k, n in enumerate(sizes)])))[:-1] + 3
+    host = np.zeros((3, int(offs[-1]) + sizes[-1] + 64), np.uint8)
+    for r in range(3):
+        for k, (o, n) in enumerate(zip(offs, sizes)):
+            x = rng.integers(0, 256, n) if (k + r) % 3 == 0 else np.clip(rng.normal(128, 8 if k % 2 else 25, n), 0, 255)
+            if (k + r) % 3 == 1:
+                x[rng.random(n) < rng.choice([0.4, 0.45, 0.95])] = 77
+            host[r, o:o + n] = x
+    src, x = dev(host), torch.zeros(host.shape[1], dtype=torch.uint8, device="cuda")
+    ptrs = torch.tensor([x.data_ptr() + int(o) for o in offs], dtype=torch.int64).cuda()
+    sz = torch.tensor(sizes, dtype=torch.int64).cuda()
+    out = torch.empty((3, len(sizes), 256), dtype=torch.int32, device="cuda")
+    reg = torch.empty(len(sizes), dtype=torch.uint8, device="cuda")
+    regs = torch.empty((3, len(sizes)), dtype=torch.uint8, device="cuda")
+    torch.cuda.synchronize()
+    s = torch.cuda.current_stream().cuda_stream
+    for r in range(3):
+        x.copy_(src[r])
+        assert hl.lib().hist_batch_regimes(ptrs.data_ptr(), sz.data_ptr(), len(sizes), out[r].data_ptr(), reg.data_ptr(),
+                                           None, s) == 0
+        regs[r].copy_(reg)
+    got, greg = u32(out).reshape(3, len(sizes), 256), regs.cpu().numpy()
+    for r in range(3):
+        for k, (o, n) in enumerate(zip(offs, sizes)):
+            im = host[r, o:o + n]
+            assert np.array_equal(got[r, k], oracle.hist_u32(im)), (r, k, n)
+            assert greg[r, k] == oracle.batch_regime(im), (r, k, n)
+
+
 @pytest.mark.parametrize("mode,budget", [(hl.MODE_AUTO, 8192), (hl.MODE_PLAIN, 960), (hl.MODE_ADAPTIVE, 2048)])
 def test_server_requests_around_the_groups_limit(mode, budget):
     """Requests around the sizes at which a batch's paths change (empty, inside
