@@ -257,14 +257,17 @@ int hist_stream_totals(hist_stream* st, uint64_t* d_totals, hist_cuda_stream s);
  * resumed with hist_stream_set_state restarts its window at that point. */
 int hist_stream_window(hist_stream* st, uint64_t* d_window, hist_cuda_stream s);
 
-/* Host-fed chunks (Sec. III.B: double-buffered transfers to the GPU overlapped
- * with the kernels).  attach_staging allocates `depth` (2..4) device staging
- * buffers of max_chunk bytes, an internal copy stream and events; call it
- * once, outside stream capture.  push_host copies h_chunk (n <= max_chunk; pin
- * it with cudaHostAlloc for the copy to overlap) into the next staging buffer
- * on the copy stream once the kernel that last read that buffer has finished,
- * makes `s` wait for the copy and pushes the staged chunk.  The caller may
- * reuse h_chunk once `s` has passed this call.  HIST_ESTATE without staging. */
+/* Host-fed chunks (Sec. III.B: transfers to the GPU overlapped with the
+ * kernels).  attach_staging allocates `depth` (2..4) device staging buffers of
+ * max_chunk bytes, an internal copy stream and events; call it once, outside
+ * stream capture.  push_host pushes the n <= max_chunk bytes at h_chunk, which
+ * are complete when it is called.  Pinned memory (cudaHostAlloc,
+ * cudaHostRegister) is read by the counting kernel over the host link, a
+ * chunk's first reads beside the previous chunk's last; other memory is copied
+ * into the next staging buffer on the copy stream once the kernel that last
+ * read that buffer has finished, `s` waits for the copy and the staged chunk
+ * is pushed.  The caller may reuse h_chunk once `s` has passed this call.
+ * HIST_ESTATE without staging. */
 int hist_stream_attach_staging(hist_stream* st, size_t max_chunk, uint32_t depth);
 int hist_stream_push_host(hist_stream* st, const uint8_t* h_chunk, size_t n, uint32_t* d_chunk_out,
                           hist_cuda_stream s);

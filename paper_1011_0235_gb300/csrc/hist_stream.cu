@@ -7,6 +7,7 @@
 // count it (every kernel counts in the lane-private table, which refines
 // every pattern), and the chunks' epilogues record the exact switches and
 // patterns (see the comments above the kernels).
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <stddef.h>
 #include <mutex>
@@ -86,11 +87,14 @@ struct PushHead {
   uint32_t theta;
   uint32_t mode;
   uint32_t window;                  // chunks in the moving window
-  uint32_t early;                   // chunks may be read before the work before the launch completes
+  uint32_t early;                   // chunks may be read before the work before the launch completes (kHostChunk:
+                                    // over the host link, one chunk)
   unsigned long long first_chunk;   // number of this batch's first chunk among the stream's chunks
   unsigned long long launch;        // number of this launch among the stream's launches (from 1)
   unsigned long long prev;          // number of the launch before it (0: none)
 };
+
+constexpr uint32_t kHostChunk = 2;
 
 // The counting launch's parameters: the header and the chunk table.  Two
 // capacities, so that a launch of a few chunks does not carry (and the driver
@@ -389,6 +393,23 @@ __device__ __noinline__ void flat_ring_ready(const A& a, FlatShared<A::kCap>& fs
   }
 }
 
+// A launch that reads over the host link lets the next one start only when
+// CTA 0 has half of its piece, and at most 64 KiB, left: the next chunk's
+// first reads come before this one's last, and however many chunks are queued
+// two or three launches of kHostGrid CTAs hold SMs while they wait for the
+// link (else all of them would: eight one-shots of 64 MiB on another stream
+// beside 16 x 16 MiB take 1145 us, so 264; 402 when the chunks were copied).
+template <class A>
+__device__ __forceinline__ bool host_late(const A& a) {
+  return a.early == kHostChunk && blockIdx.x == 0;
+}
+__device__ __forceinline__ uint32_t host_mid(const uint8_t* in, uint32_t b, uint32_t e) {
+  uint32_t left = (e - b) / 2;
+  if (left > 65536u) left = 65536u;
+  const uint32_t m = e - left, over = (uint32_t)(((uintptr_t)in + m) & (kLineBytes - 1));
+  return m - b > over && left ? m - over : e;
+}
+
 // Count piece k of the window's (the CTA's number `turn`; `ring`: whether the
 // ring check is behind) into the table, which is clear before and after, and
 // publish it: into the chunk's accumulator, or, when it is the whole chunk,
@@ -411,7 +432,17 @@ __device__ __forceinline__ void flat_piece(const A& a, uint32_t k, uint32_t turn
       const uint32_t at = sample_at(p.d.in, p.d.n, t);
       if (at != 0xffffffffu && at >= p.b0 && at < p.e0) vec = p.d.in + at;
     }
-    piece_count(p.d.in + p.b0, p.e0 - p.b0, table, fs.eh[turn & 1], vec, fs.samp[turn & 1]);
+    const bool late = host_late(a);
+    uint32_t b = p.b0, e = late ? host_mid(p.d.in, b, p.e0) : p.e0;
+    for (;;) {
+      piece_count(p.d.in + b, e - b, table, fs.eh[turn & 1], vec, fs.samp[turn & 1]);
+      if (!late) break;
+      pdl_launch_dependents();
+      if (e == p.e0) break;
+      b = e;
+      e = p.e0;
+      vec = nullptr;
+    }
     if (k + 1 < fs.npiece) {
       const FlatPiece& q = fs.piece[k + 1];
       const uint32_t at = (uint32_t)t * kLineBytes;
@@ -744,13 +775,14 @@ __global__ void __launch_bounds__(kThreads, 1) batch_flat_kernel(const __grid_co
   __shared__ FlatShared<A::kCap> fs;
   const int t = threadIdx.x;
 
-  pdl_launch_dependents();
+  // what the range needs of the parameters is read before the wait
+  const bool groups = a.plan.groups[blockIdx.x >> 5] >> (blockIdx.x & 31) & 1u;
+  if (groups || !host_late(a)) pdl_launch_dependents();
   if (t == 0) {
     fs.released = a.early ? 0 : 1;
     fs.epis = 0;
   }
-  // what the range needs of the parameters is read before the wait
-  if (a.plan.groups[blockIdx.x >> 5] >> (blockIdx.x & 31) & 1u) {
+  if (groups) {
     // the range holds whole chunks for the groups only
     const uint32_t s0 = a.plan.s[blockIdx.x], s1 = a.plan.s[blockIdx.x + 1];
     __syncthreads();
@@ -1068,12 +1100,20 @@ uint32_t flat_plan(RangePlan* p, uint32_t count, const size_t* ns, uint32_t grid
   return grid;
 }
 
+// The grid of a launch that reads over the host link: 1 MiB of loads in
+// flight.  16 x 16 MiB take 1272 us with 8 CTAs as with 152, 64 x 1 MiB 394
+// with 8, 388 with 16, 402 with 24 to 152; the other SMs are left to other
+// streams.
+constexpr uint32_t kHostGrid = 16;
+
 // The launches of one batch: the counting launch, and with a window of more
 // than one chunk the window's switches.  Each may start while the one before
-// ends and waits for it before it reads what that one writes.
+// ends and waits for it before it reads what that one writes.  `host`: the
+// chunks are in host memory that the kernels can read, and were complete when
+// they were pushed.
 template <class A>
 int launch_batch(hist_stream* st, uint32_t count, const uint8_t* const* ins, const size_t* ns, uint32_t* const* outs,
-                 cudaStream_t s) {
+                 bool host, cudaStream_t s) {
   // the stream's parameter buffer: the header and the plan are cleared, the
   // chunk entries written (the launch copies the parameters)
   static_assert(sizeof(A) <= sizeof(LargeArgs), "one buffer for both parameter blocks");
@@ -1093,14 +1133,16 @@ int launch_batch(hist_stream* st, uint32_t count, const uint8_t* const* ins, con
   a->trace = st->trace;
   a->trace_cap = st->trace_cap;
   a->trace_first = st->trace_next;
-  a->early = (st->cfg.flags & HIST_OVERLAP_PUSHES) ? 1u : 0u;
+  a->early = host ? kHostChunk : (st->cfg.flags & HIST_OVERLAP_PUSHES) ? 1u : 0u;
   for (uint32_t i = 0; i < count; ++i) {
     a->c[i].in = ins[i];
     a->c[i].n = (uint32_t)ns[i];
     a->c[i].out = outs ? outs[i] : nullptr;
   }
   const bool windowed = st->cfg.window > 1;
-  const uint32_t grid = flat_plan(&a->plan, count, ns, (uint32_t)st->grid);
+  uint32_t most = (uint32_t)st->grid;
+  if (host && most > kHostGrid) most = kHostGrid;
+  const uint32_t grid = flat_plan(&a->plan, count, ns, most);
   void* params[] = {a};
   cudaError_t e =
       launch_chained((const void*)batch_flat_kernel<A>, dim3(grid), dim3(kThreads), params,
@@ -1120,14 +1162,50 @@ int launch_batch(hist_stream* st, uint32_t count, const uint8_t* const* ins, con
 }
 
 int push_chunks(hist_stream* st, uint32_t count, const uint8_t* const* ins, const size_t* ns, uint32_t* const* outs,
-                cudaStream_t s) {
+                cudaStream_t s, bool host = false) {
   for (uint32_t i = 0; i < count; i += kMaxBatch) {
     const uint32_t c = count - i < kMaxBatch ? count - i : kMaxBatch;
-    int rc = c <= kSmallBatch ? launch_batch<SmallArgs>(st, c, ins + i, ns + i, outs ? outs + i : nullptr, s)
-                              : launch_batch<LargeArgs>(st, c, ins + i, ns + i, outs ? outs + i : nullptr, s);
+    int rc = c <= kSmallBatch ? launch_batch<SmallArgs>(st, c, ins + i, ns + i, outs ? outs + i : nullptr, host, s)
+                              : launch_batch<LargeArgs>(st, c, ins + i, ns + i, outs ? outs + i : nullptr, host, s);
     if (rc) return rc;
   }
   return HIST_OK;
+}
+
+// The address at which kernels launched on `s` read the n bytes of host memory
+// at p, or null: the bytes must lie in one range of memory that CUDA has
+// pinned, and `s` must not be capturing (a push from the host is no part of a
+// graph: the staged path's error says so).  About 0.1 us.
+const uint8_t* host_readable(const uint8_t* p, size_t n, cudaStream_t s) {
+  typedef CUresult (*Ask)(unsigned int, CUpointer_attribute*, void**, CUdeviceptr);
+  static const Ask ask = []() -> Ask {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    const cudaError_t e =
+        cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000, cudaEnableDefault, &found);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e == cudaSuccess && found == cudaDriverEntryPointSuccess ? (Ask)f : nullptr;
+  }();
+  if (!ask) return nullptr;
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusActive;
+  if (cudaStreamIsCapturing(s, &capture) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  if (capture != cudaStreamCaptureStatusNone) return nullptr;
+  unsigned int type = 0, managed = 1;
+  CUdeviceptr d = 0, start = 0;
+  size_t size = 0;
+  CUpointer_attribute at[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED,
+                              CU_POINTER_ATTRIBUTE_DEVICE_POINTER, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                              CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+  void* data[] = {&type, &managed, &d, &start, &size};
+  if (ask(5, at, data, (CUdeviceptr)(uintptr_t)p) != CUDA_SUCCESS) return nullptr;
+  const uint64_t at0 = (uint64_t)(uintptr_t)p - (uint64_t)start;
+  if (type != CU_MEMORYTYPE_HOST || managed || !d || (uint64_t)(uintptr_t)p < (uint64_t)start || at0 > size ||
+      n > size - at0)
+    return nullptr;
+  return reinterpret_cast<const uint8_t*>((uintptr_t)d);
 }
 
 bool config_ok(const hist_config* c) {
@@ -1305,6 +1383,14 @@ int hist_stream_push_host(hist_stream* st, const uint8_t* h_chunk, size_t n, uin
   if (!st || (!h_chunk && n)) return HIST_EINVAL;
   if (!st->depth) return HIST_ESTATE;
   if (n > st->max_chunk) return HIST_EINVAL;
+  // Pinned memory is counted in place, a chunk's reads beside the launch
+  // before it, as with HIST_OVERLAP_PUSHES (the caller's bytes were complete
+  // before too: the copies waited for no work of his).  Copied into staging,
+  // with the events between copy and count, and now: 64 x 64 KiB 729 -> 263
+  // us, 64 x 1 MiB 860 -> 421, 16 x 4 MiB 404 -> 350, 16 x 16 MiB 1335 -> 1298
+  // (1272 at the link's rate).
+  if (const uint8_t* d = n ? host_readable(h_chunk, n, (cudaStream_t)s) : nullptr)
+    return push_chunks(st, 1, &d, &n, d_chunk_out ? &d_chunk_out : nullptr, (cudaStream_t)s, true);
   const uint32_t b = (uint32_t)(st->host_pushes % st->depth);
   cudaStream_t cs = st->copy_stream;
   // the buffer's previous chunk kernel must be done before it is overwritten

@@ -259,6 +259,55 @@ def test_batch_lane_launches(name, sizes, out_shift):
     _batch(sizes, 17, 40, out_shift)
 
 
+@pytest.mark.parametrize("depth,window,overlap", [(2, 1, False), (4, 5, False), (3, 1, True)])
+def test_host_chunks_pinned_registered_and_pageable(depth, window, overlap):
+    """Chunks read in place (pinned, registered: at every alignment, to the
+    range's last byte) and staged ones (pageable) in turn with device chunks,
+    sizes around the limits of the launch's grid, several in flight; the
+    buffers are rewritten when the stream has passed their pushes."""
+    rng = np.random.default_rng(depth)
+    big = 3 << 20
+    pinned = torch.empty(20 << 20, dtype=torch.uint8, pin_memory=True).numpy()
+    page = np.zeros((20 << 20) + 4096, np.uint8)
+    first = -page.ctypes.data % 4096
+    reg, plain = page[first:first + (20 << 20)], np.zeros(20 << 20, np.uint8)
+    assert int(torch.cuda.cudart().cudaHostRegister(reg.ctypes.data, reg.size, 0)) == 0
+    st = hl.Stream(window=window, overlap=overlap)
+    st.attach_staging(big, depth)
+    ref = oracle.StreamOracle(oracle.BUDGET_MAX)
+    sizes = [1, 100, 4097, 32768, 65536 + 1, 16 * 32768 - 1, 16 * 32768 + 129, 1 << 20, 2_000_003, big, 0]
+    outs = torch.full((66, 256), -1, dtype=torch.int32, device="cuda")
+    hists, rec, keep = [], None, []
+    for i in range(66):
+        if i % 22 == 0:  # the buffers from their ends down
+            torch.cuda.current_stream().synchronize()
+            end = {id(b): b.size for b in (pinned, reg, plain)}
+            for b in (pinned, reg, plain):
+                b[:] = 0
+        n, where = sizes[i % len(sizes)], (pinned, reg, pinned, plain, None)[int(rng.integers(0, 5))]
+        data = rng.integers(0, 256, n, dtype=np.uint8)
+        data[rng.random(n) < rng.choice([0.0, 0.45, 0.9])] = 31
+        if where is None:
+            keep.append(dev(data) if n else torch.empty(0, dtype=torch.uint8, device="cuda"))
+            st.push(keep[-1], outs[i])
+        else:
+            at = end[id(where)] - n
+            end[id(where)] = at - int(rng.integers(0, 300))
+            where[at:at + n] = data
+            st.push_host(where.ctypes.data + at, n, outs[i].data_ptr())
+        rec = ref.push(data)
+        hists.append(rec.hist)
+    win = st.window().cpu().numpy().view(np.uint64)
+    torch.cuda.synchronize()
+    s = st.state()
+    assert np.array_equal(u32(outs).reshape(66, 256), np.stack(hists))
+    assert np.array_equal(win, np.sum(np.stack(hists[-window:]).astype(np.uint64), axis=0))
+    assert np.array_equal(np.array(s.totals, np.uint64), ref.totals) and s.status == 0 and s.chunks == 66
+    assert bytes(s.pattern) == ref.pattern.to_bytes() and s.flag == ref.flag and s.last_kernel == rec.kernel
+    st.close()
+    assert int(torch.cuda.cudart().cudaHostUnregister(reg.ctypes.data)) == 0
+
+
 @pytest.mark.parametrize("sizes", [
     [0, 1, 15, 16, 17, 19, 20, 255, 4079, 4080, 4095, 4096, 4097, 4100, 4111, 4112, 5000] * 4,
     [3000 + 401 * k for k in range(300)] + [2_000_003, 4096 * 256 + 1],
