@@ -180,7 +180,11 @@ __global__ void __launch_bounds__(kThreads, MINB) batch_images_kernel(BatchImgAr
 // images.  The second launch counts those, piece by piece, the whole CTA on
 // each, which has the start of the next piece fetched into L2 while it
 // reduces the table; its CTAs start on the SMs that the first's leave and
-// wait for it before they write.  Two launches because the groups' tables
+// wait for it before they write.  With at most kBatchFew images the first
+// launch is a light one (batch_few_kernel: a warp per image counts the tiny
+// ones and clears the others' outputs) and the second counts all the rest:
+// the groups' tables and ranges cost more than they bring for few images, and
+// the second launch's CTAs find free SMs at once.  Two launches because the groups' tables
 // (128 KiB) would take the L1 cache from the large images' loads (64 stream
 // chunks of 16 MiB: 161 us with 80 KiB of shared memory, 176 with 146), and
 // because one kernel with both loops spills registers.
@@ -219,6 +223,13 @@ __device__ __forceinline__ unsigned long long lane_cost(unsigned long long n) {
   return n + (SMALL ? kLaneSmallCost : kImageCost);
 }
 
+// Batches of at most so many images are of few images (batch_few_kernel).
+// Both ways, us: 1 image of 8 .. 22 a side 2.7 (with the group launch 4.7),
+// 26 of 36 .. 249 5.8 (8.1), 100 of 180 .. 948 12.2 (18.1), 300 of 20 .. 1686
+// 24.3 (30.3), 1000 of 16 .. 256 14.0 (16.3), 1000 of 180 .. 948 58.6 (60.2);
+// but 1500 of 36 .. 249 20.1 (19.7), 2048 of 16 .. 256 20.6 (19.1).
+constexpr uint32_t kBatchFew = 1024;
+
 struct LanePiece {
   const uint8_t* base;
   uint32_t len;
@@ -237,6 +248,7 @@ struct LaneArgs {
   uint32_t* out;
   unsigned long long inv;  // floor((2^64 - 1) / grid)
   uint32_t count;
+  bool few;  // every image that is not tiny is the second launch's
 };
 
 template <bool SMALL>
@@ -386,6 +398,30 @@ __device__ __forceinline__ void lane_pieces(const LaneArgs& a, uint32_t* table, 
   }
 }
 
+// Count an image of head bytes, nvec vectors and tail bytes with one warp, U
+// vectors in flight per lane, into its 256 words h.
+template <int U>
+__device__ __forceinline__ void tiny_image(const uint4* body, uint32_t head, uint32_t nvec, uint32_t tail,
+                                           uint32_t* h) {
+  const uint32_t lane = threadIdx.x & 31;
+  uint32_t edge = 0x100u;
+  if (lane < head) edge = (reinterpret_cast<const uint8_t*>(body) - head)[lane];
+  else if (lane - head < tail) edge = reinterpret_cast<const uint8_t*>(body + nvec)[lane - head];
+  LaneRange r = lane_range(body, 0, nvec, (int)lane);
+  uint4 v[U];
+  lane_load<U, 32>(v, r);
+  if (edge < 0x100u) atomicAdd(&h[edge], 1u);
+  while (r.left) {
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if ((uint32_t)(u * 32) < r.left) vec_count(v[u], h);
+    r.q += U * 32;
+    r.left = r.left > U * 32 ? r.left - U * 32 : 0u;
+    lane_load<U, 32>(v, r);
+  }
+  __syncwarp();
+}
+
 // Count the window's tiny images, a warp each, in the warp's 256 words of the
 // first table (clear before and after).
 __device__ __forceinline__ void lane_tiny(const LaneArgs& a, uint32_t* tables, const LaneShared<true>& ls) {
@@ -393,23 +429,7 @@ __device__ __forceinline__ void lane_tiny(const LaneArgs& a, uint32_t* tables, c
   uint32_t* h = tables + w * HIST_BINS;
   for (uint32_t i = w; i < ls.tiny; i += kWarps) {
     const LaneItem& it = ls.item[i];
-    const uint8_t* in = reinterpret_cast<const uint8_t*>(it.body) - it.head;
-    uint32_t edge = 0x100u;
-    if (lane < it.head) edge = in[lane];
-    else if (lane - it.head < it.tail) edge = reinterpret_cast<const uint8_t*>(it.body + it.nvec)[lane - it.head];
-    LaneRange r = lane_range(it.body, 0, it.nvec, (int)lane);
-    uint4 v[kTinyLoads];
-    lane_load<kTinyLoads, 32>(v, r);
-    if (edge < 0x100u) atomicAdd(&h[edge], 1u);
-    while (r.left) {
-#pragma unroll
-      for (int u = 0; u < kTinyLoads; ++u)
-        if ((uint32_t)(u * 32) < r.left) vec_count(v[u], h);
-      r.q += kTinyLoads * 32;
-      r.left = r.left > kTinyLoads * 32 ? r.left - kTinyLoads * 32 : 0u;
-      lane_load<kTinyLoads, 32>(v, r);
-    }
-    __syncwarp();
+    tiny_image<kTinyLoads>(it.body, it.head, it.nvec, it.tail, h);
     uint32_t* out = a.out + (size_t)it.image * HIST_BINS;
 #pragma unroll
     for (int k = 0; k < HIST_BINS / 32; ++k) {
@@ -461,6 +481,32 @@ __device__ __forceinline__ void lane_items(const LaneArgs& a, uint32_t* tables, 
   }
 }
 
+// The first launch of a batch of few images: a warp each, which counts a tiny
+// one, all its vectors in flight, and clears the output of any other.  Bound
+// by the chain of three reads (sizes, pointers, pixels).
+constexpr int kFewWarps = 8;
+__global__ void __launch_bounds__(kFewWarps * 32) batch_few_kernel(const __grid_constant__ LaneArgs a) {
+  __shared__ uint32_t tables[kFewWarps][HIST_BINS];
+  const uint32_t w = threadIdx.x >> 5, lane = threadIdx.x & 31, i = blockIdx.x * kFewWarps + w;
+  uint32_t* h = tables[w];
+#pragma unroll
+  for (int k = 0; k < HIST_BINS / 32; ++k) h[lane + 32 * k] = 0;
+  __syncwarp();
+  pdl_wait();
+  pdl_launch_dependents();
+  if (i >= a.count) return;
+  const unsigned long long n = a.sizes[i];
+  if (n != 0 && n <= kLaneTiny) {
+    const uint8_t* p = a.ptrs[i];
+    const Split sp = split_bytes_at(p, (size_t)n, 16);
+    tiny_image<kLaneTiny / (32 * 16)>(reinterpret_cast<const uint4*>(p + sp.head), (uint32_t)sp.head,
+                                      (uint32_t)sp.nvec, (uint32_t)sp.tail, h);
+  }
+  uint32_t* out = a.out + (size_t)i * HIST_BINS;
+#pragma unroll
+  for (int k = 0; k < HIST_BINS / 32; ++k) out[lane + 32 * k] = h[lane + 32 * k];
+}
+
 template <bool SMALL>
 __global__ void __launch_bounds__(kThreads, 1) batch_lane_kernel(const __grid_constant__ LaneArgs a) {
   extern __shared__ __align__(16) uint32_t tables[];
@@ -489,7 +535,7 @@ __global__ void __launch_bounds__(kThreads, 1) batch_lane_kernel(const __grid_co
   const uint32_t zi = blockIdx.x * kWarps + ((uint32_t)t >> 5);
   const unsigned long long zsize = SMALL && zi < a.count ? (unsigned long long)a.sizes[zi] : 0ull;
   block_scan(local, ls.wsum, total);
-  const unsigned long long share = grid_share(total, a.inv);
+  const unsigned long long share = a.few ? 0 : grid_share(total, a.inv);
   if (SMALL && zi < a.count && !(zsize && lane_small(zsize, share))) {
     // an output that is not this launch's to write
 #pragma unroll
@@ -690,8 +736,17 @@ int launch_batch_lane(const uint8_t* const* d_ptrs, const size_t* d_sizes, uint3
     at[0].val.programmaticStreamSerializationAllowed = 1;
     lc.attrs = at;
     lc.numAttrs = 1;
-    lc.dynamicSmemBytes = lane_smem<true>();
-    cudaError_t e = cudaLaunchKernelEx(&lc, batch_lane_kernel<true>, a);
+    a.few = a.count <= kBatchFew;
+    cudaError_t e;
+    if (a.few) {
+      cudaLaunchConfig_t cc = lc;
+      cc.gridDim = dim3((a.count + kFewWarps - 1) / kFewWarps);
+      cc.blockDim = dim3(kFewWarps * 32);
+      e = cudaLaunchKernelEx(&cc, batch_few_kernel, a);
+    } else {
+      lc.dynamicSmemBytes = lane_smem<true>();
+      e = cudaLaunchKernelEx(&lc, batch_lane_kernel<true>, a);
+    }
     if (e != cudaSuccess) return cuda_fail(e);
     lc.dynamicSmemBytes = lane_smem<false>();
     e = cudaLaunchKernelEx(&lc, batch_lane_kernel<false>, a);

@@ -243,12 +243,16 @@ def _batch(sizes, seed, spread, out_shift=0):
 @pytest.mark.parametrize("name,sizes,out_shift", [
     # on both sides of the warps', the groups' and the whole-image limits
     ("edges", [0, 1, 15, 16, 127, 128, 143, 4095, 4096, 4097, 131_071, 131_072, 131_073, 500_000] * 40, 1),
+    ("edges of more", [0, 1, 15, 16, 127, 128, 143, 4095, 4096, 4097, 131_071, 131_072, 131_073, 250_000] * 80, 1),
+    # the most images of a few, and one more
+    ("most", [1 + (i * 977) % 9000 for i in range(1024)], 0),
+    ("not few", [1 + (i * 977) % 9000 for i in range(1025)], 0),
     # a few images, all cut between CTAs
     ("few", [300_000, 131_072, 70_001, 5000, 4096, 3], 0),
     # one range holds hundreds of tiny images (many windows of 64) between
     # pieces of large ones
     ("long", [20_000_000] + [9] * 700 + [5000] * 300 + [30_000_001] + [0] * 100 + [4097] * 200, 3),
-    # more images than one launch takes, tiny and not
+    # more images than one launch takes, tiny and not (and the rest few)
     ("many", [100 + 37 * (i % 300) for i in range(4096 + 70)], 2),
     ("empty", [0, 0, 0], 0),
     ("one", [1], 0),
