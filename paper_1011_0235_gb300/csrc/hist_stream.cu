@@ -826,22 +826,19 @@ __global__ void __launch_bounds__(kThreads, 1) batch_flat_kernel(const __grid_co
 // A window of W > 1 chunks.  The window histogram after chunk g is the sum
 // of the histograms of chunks g-W+1 .. g (chunks before number 0 count as
 // empty; a resumed stream restarts at 0).  The histograms of the last
-// kChunkRing chunks stay in rings, so each chunk's window is summed on its
-// own: one CTA per chunk of the batch, thread b + 256 q taking bin b of
-// every fourth run of eight chunks, so that a window of 32 is one round of
-// loads.  Bound by L2 latency: a push of 128 x 1 MiB at W = 32 with its
-// totals, window and change queries takes 40.8 us, 56.0 with 256 threads (four
-// rounds) and the queries each waiting for the launch before it to end.
+// kChunkRing chunks stay in rings, so every window is summed on its own:
+// thread b + 256 q takes bin b of every fourth run of eight chunks, so that a
+// window of 32 is one round of loads.
 constexpr int kWindowThreads = 4 * HIST_BINS;
 constexpr uint32_t kWindowRun = 8;                              // chunks per thread and round
 constexpr uint32_t kWindowRound = kWindowRun * kWindowThreads / HIST_BINS;  // chunks per round
 
 // Largest bin and total of a 256-bin window held one bin per thread (256
-// threads on barrier 1 call; two barriers); returned to every thread.
+// threads on barrier `id` call; two barriers); returned to every thread.
 template <class T>
-__device__ __forceinline__ void window_max_sum(T v, T* smax, T* ssum, T& mx, T& sm) {
-  const GroupBar<HIST_BINS> bar = {1};
-  const int b = threadIdx.x, w = b >> 5;
+__device__ __forceinline__ void window_max_sum(T v, T* smax, T* ssum, int id, T& mx, T& sm) {
+  const GroupBar<HIST_BINS> bar = {id};
+  const int b = threadIdx.x & (HIST_BINS - 1), w = b >> 5;
   T m = v, s = v;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -864,13 +861,58 @@ __device__ __forceinline__ void window_max_sum(T v, T* smax, T* ssum, T& mx, T& 
   bar.sync();
 }
 
-// The window switches of a launch's chunks, one CTA per chunk, chained after
-// the counting launch.  The CTA of the last chunk writes the window after it
-// and the stream's switch; the one of the chunk before it the kernel the last
-// chunk ran.  In AUTO mode each CTA but the last also takes the same window's
-// switch from the samples, in FP32 and in the chunks' order (FP64 is slow on
-// this part and the samples are estimates), and counts a chunk whose two
-// switches differ.
+// The end of the window after the launch's chunk c, a bin per thread in x and
+// its samples' sum in f (256 threads on barrier `id`): the switch and what
+// depends on it.
+__device__ __forceinline__ void window_end(const PushHead& a, uint32_t c, unsigned long long x, float f,
+                                           unsigned long long* smax, unsigned long long* ssum, float* fmax,
+                                           float* fsum, int id) {
+  StreamDev* st = a.st;
+  const int b = threadIdx.x & (HIST_BINS - 1);
+  unsigned long long mx, sm;
+  window_max_sum(x, smax, ssum, id, mx, sm);
+  const uint32_t flag = reaches_theta(mx, sm, a.theta) ? HIST_FLAG_ADAPTIVE : HIST_FLAG_PLAIN;
+  if (a.mode == HIST_MODE_AUTO && c + 1 < a.count) {
+    float fm, fs;
+    window_max_sum(f, fmax, fsum, id, fm, fs);
+    const uint32_t pred = (fs > 0.0f && fm * 1000.0f >= fs * (float)a.theta) ? HIST_FLAG_ADAPTIVE : HIST_FLAG_PLAIN;
+    if (b == 0 && pred != flag) atomicAdd(&st->h.recounted, 1u);
+  }
+  const uint32_t fixed = a.mode == HIST_MODE_ADAPTIVE ? HIST_FLAG_ADAPTIVE : HIST_FLAG_PLAIN;
+  if (c + 1 == a.count) {
+    st->wmw[b] = x;
+    if (b == 0) {
+      if (a.count == 1) st->h.last_kernel = a.mode == HIST_MODE_AUTO ? __ldcg(&st->h.flag) : fixed;
+      st->h.flag = flag;
+    }
+  } else if (c + 2 == a.count && b == 0) {
+    st->h.last_kernel = a.mode == HIST_MODE_AUTO ? flag : fixed;
+  }
+}
+
+// The window switches of a launch's chunks, chained after the counting launch.
+// The last chunk's window and the stream's switch after it are kept, and the
+// switch of the chunk before it, which is the kernel the last chunk ran.  In
+// AUTO mode every window but the last also takes its switch from the samples,
+// in FP32 and in the chunks' order (FP64 is slow on this part and the samples
+// are estimates), and a chunk whose two switches differ is counted; in the
+// other modes only the last two windows are asked for.
+//
+// Two kernels.  window_runs_kernel: M windows of consecutive chunks a CTA,
+// which share their rows' loads, the next round's in flight while one is
+// summed (64 registers, one CTA per SM).  window_flat_kernel: a window a CTA
+// in 32 registers, two CTAs per SM.  Bound by L2 latency with few windows, by
+// the rows read (count x W KiB, twice in AUTO mode) with many.  A push with
+// its window, us, with window_flat_kernel for every chunk and now:
+//   128 x 1 MiB W 32         33.7   31.8   (28.9 without a window)
+//   81 x 570 KB W 161        29.6   24.8   (15.9)
+//   152 x 5 KB W 256         25.4   18.5   (6.4)
+//   500 x 5 KB W 100, 256    27.9, 44.6   22.6, 31.4   (9.1)
+//   1000 x 5 KB W 100, 256   42.9, 71.7   34.6, 46.1   (11.4)
+//   639 x 5 KB W 203, plain  35.6   16.0   (10.0)
+// One wave of CTAs is a window each (M = 1; with M = 2 128 x 1 MiB take 34.9);
+// up to two waves, and short windows, stay with window_flat_kernel (300 x 5 KB
+// W 32 11.1, with M = 2 12.9; 1000 x 5 KB W 32 24.2, with M = 8 27.9).
 __global__ void __launch_bounds__(kWindowThreads) window_flat_kernel(const PushHead a) {
   __shared__ unsigned long long part[kWindowThreads / HIST_BINS - 1][HIST_BINS];
   __shared__ uint32_t samp[kWindowRound][HIST_BINS];
@@ -881,10 +923,10 @@ __global__ void __launch_bounds__(kWindowThreads) window_flat_kernel(const PushH
   const int b = threadIdx.x & (HIST_BINS - 1), q = threadIdx.x / HIST_BINS;
   pdl_launch_dependents();
   pdl_wait();
-  const unsigned long long W = a.window, g = a.first_chunk + blockIdx.x;
+  const unsigned long long W = a.window, c = blockIdx.x, g = a.first_chunk + c;
   const unsigned long long first = g >= W - 1 ? g - (W - 1) : 0ull;
   const uint32_t len = (uint32_t)(g - first + 1);
-  const bool sampled = a.mode == HIST_MODE_AUTO && blockIdx.x + 1 < a.count;
+  const bool sampled = a.mode == HIST_MODE_AUTO && c + 1 < a.count;
   // each window chunk's scale, one thread per chunk
   if (sampled && threadIdx.x < len) {
     const uint32_t slot = (uint32_t)((first + threadIdx.x) % kChunkRing);
@@ -921,24 +963,114 @@ __global__ void __launch_bounds__(kWindowThreads) window_flat_kernel(const PushH
   if (q > 0) return;
 #pragma unroll
   for (int i = 0; i < kWindowThreads / HIST_BINS - 1; ++i) v += part[i][b];
-  unsigned long long mx, sm;
-  window_max_sum(v, smax, ssum, mx, sm);
-  const uint32_t flag = reaches_theta(mx, sm, a.theta) ? HIST_FLAG_ADAPTIVE : HIST_FLAG_PLAIN;
-  if (sampled) {
-    float fm, fs;
-    window_max_sum(f, fmax, fsum, fm, fs);
-    const uint32_t pred = (fs > 0.0f && fm * 1000.0f >= fs * (float)a.theta) ? HIST_FLAG_ADAPTIVE : HIST_FLAG_PLAIN;
-    if (b == 0 && pred != flag) atomicAdd(&st->h.recounted, 1u);
-  }
-  const uint32_t fixed = a.mode == HIST_MODE_ADAPTIVE ? HIST_FLAG_ADAPTIVE : HIST_FLAG_PLAIN;
-  if (blockIdx.x + 1 == a.count) {
-    st->wmw[b] = v;
-    if (b == 0) {
-      if (a.count == 1) st->h.last_kernel = a.mode == HIST_MODE_AUTO ? __ldcg(&st->h.flag) : fixed;
-      st->h.flag = flag;
+  window_end(a, (uint32_t)c, v, f, smax, ssum, fmax, fsum, 1);
+}
+
+// Windows skip + M blockIdx.x .. + M - 1 of the launch's.  Rows that all of
+// them hold are added once for all, the others window by window.
+template <int M>
+__global__ void __launch_bounds__(kWindowThreads) window_runs_kernel(const PushHead a, uint32_t skip) {
+  constexpr int Q = kWindowThreads / HIST_BINS, E = M < Q ? 1 : M / Q, P = M < Q ? M : Q;
+  // (Q groups of threads; group q < P ends windows q, q + Q, .. of E)
+  __shared__ union {
+    float samp[kWindowRound][HIST_BINS];
+    unsigned long long part[Q][P][HIST_BINS];
+  } u;
+  __shared__ unsigned long long smax[Q][HIST_BINS / 32], ssum[Q][HIST_BINS / 32];
+  __shared__ float fmax[Q][HIST_BINS / 32], fsum[Q][HIST_BINS / 32];
+  __shared__ __align__(16) float scale[(HIST_WINDOW_MAX + M - 2) / kWindowRound * kWindowRound + kWindowRound];
+  StreamDev* st = a.st;
+  const int b = threadIdx.x & (HIST_BINS - 1), q = threadIdx.x / HIST_BINS;
+  pdl_launch_dependents();
+  pdl_wait();
+  const uint32_t c0 = skip + blockIdx.x * M, nw = a.count - c0 < M ? a.count - c0 : M;
+  // row 0 is the first window's first chunk, row r in slot base + r of the
+  // rings; window w's rows are [from(w), to(w))
+  const unsigned long long g0 = a.first_chunk + c0;
+  const uint32_t back = g0 < a.window - 1 ? (uint32_t)g0 : a.window - 1;
+  const uint32_t base = (uint32_t)((g0 - back) % kChunkRing), rows = back + nw;
+  auto from = [&](uint32_t w) { return back + w + 1 > a.window ? back + w + 1 - a.window : 0u; };
+  auto to = [&](uint32_t w) { return back + w + 1; };
+  const bool sampled = a.mode == HIST_MODE_AUTO && c0 + 1 < a.count;
+  // each row's scale, one thread per row
+  if (sampled && threadIdx.x < sizeof(scale) / sizeof(scale[0])) {
+    float x = 0.0f;
+    if (threadIdx.x < rows) {
+      const uint32_t slot = (base + threadIdx.x) % kChunkRing;
+      const uint32_t sn = __ldcg(&st->wsn[slot]);
+      x = sn ? (float)__ldcg(&st->wn[slot]) / (float)sn : 0.0f;
     }
-  } else if (blockIdx.x + 2 == a.count && b == 0) {
-    st->h.last_kernel = a.mode == HIST_MODE_AUTO ? flag : fixed;
+    scale[threadIdx.x] = x;
+  }
+  unsigned long long all = 0, v[M] = {};  // rows of every window, and of window w beside them
+  float f[E] = {};
+  uint32_t h[kWindowRun], s[kWindowRun];
+  auto load = [&](uint32_t k0) {
+#pragma unroll
+    for (uint32_t i = 0; i < kWindowRun; ++i) {
+      const uint32_t k = k0 + q * kWindowRun + i;
+      const uint32_t slot = (base + k) % kChunkRing;
+      h[i] = k < rows ? __ldcg(&st->whist[slot][b]) : 0u;
+      s[i] = sampled && k < rows ? __ldcg(&st->wsamp[slot][b]) : 0u;
+    }
+  };
+  load(0);
+  for (uint32_t k0 = 0; k0 < rows; k0 += kWindowRound) {
+    // (rows past the last are zeros: they change no sum of one window)
+    const bool common = M == 1 || (k0 >= from(M - 1) && k0 + kWindowRound <= to(0));
+#pragma unroll
+    for (uint32_t i = 0; i < kWindowRun; ++i) {
+      if (common) {
+        all += h[i];
+      } else {
+        const uint32_t k = k0 + q * kWindowRun + i;
+#pragma unroll
+        for (int w = 0; w < M; ++w)
+          if (k >= from(w) && k < to(w)) v[w] += h[i];
+      }
+      if (sampled) u.samp[q * kWindowRun + i][b] = (float)s[i];
+    }
+    if (k0 + kWindowRound < rows) load(k0 + kWindowRound);
+    if (sampled) {
+      __syncthreads();
+      if (q < P) {
+        if (common) {
+#pragma unroll 2
+          for (uint32_t i = 0; i < kWindowRound; i += 4) {
+            const float4 sc = *reinterpret_cast<const float4*>(&scale[k0 + i]);
+            const float x[4] = {sc.x, sc.y, sc.z, sc.w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const float y = u.samp[i + j][b];
+#pragma unroll
+              for (int e = 0; e < E; ++e) f[e] = fmaf(y, x[j], f[e]);
+            }
+          }
+        } else {
+#pragma unroll 4
+          for (uint32_t i = 0; i < kWindowRound; ++i) {
+            const float y = u.samp[i][b], x = scale[k0 + i];
+#pragma unroll
+            for (int e = 0; e < E; ++e)
+              if (k0 + i >= from(e * Q + q) && k0 + i < to(e * Q + q)) f[e] = fmaf(y, x, f[e]);
+          }
+        }
+      }
+      __syncthreads();
+    }
+  }
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    if (e) __syncthreads();
+#pragma unroll
+    for (int w = 0; w < P; ++w) u.part[q][w][b] = v[e * Q + w] + all;
+    __syncthreads();
+    if (q < P && (uint32_t)(e * Q + q) < nw) {
+      unsigned long long x = 0;
+#pragma unroll
+      for (int i = 0; i < Q; ++i) x += u.part[i][q][b];
+      window_end(a, c0 + e * Q + q, x, f[e], smax[q], ssum[q], fmax[q], fsum[q], 1 + q);
+    }
   }
 }
 
@@ -1148,9 +1280,20 @@ int launch_batch(hist_stream* st, uint32_t count, const uint8_t* const* ins, con
       launch_chained((const void*)batch_flat_kernel<A>, dim3(grid), dim3(kThreads), params,
                      a->plan.group_max ? kFlatGroupSmem : kFlatSmem, s);
   PushHead head = *a;
-  void* hparams[] = {&head};
-  if (e == cudaSuccess && windowed)
-    e = launch_chained((const void*)window_flat_kernel, dim3(count), dim3(kWindowThreads), hparams, 0, s);
+  if (e == cudaSuccess && windowed) {
+    // (window_flat_kernel's comment: which kernel, with M = m)
+    uint32_t skip = st->cfg.mode != HIST_MODE_AUTO && count > 2 ? count - 2 : 0;
+    const uint32_t windows = count - skip;
+    void* hparams[] = {&head, &skip};
+    const uint32_t sms = (uint32_t)st->sms;
+    const uint32_t m = windows <= sms ? 1u : windows <= 4 * sms ? 4u : 8u;
+    const bool runs = m == 1 || (m == 4 ? windows > 2 * sms && st->cfg.window >= 100 : windows * st->cfg.window >= 100000);
+    const void* fn = !runs    ? (const void*)window_flat_kernel
+                     : m == 1 ? (const void*)window_runs_kernel<1>
+                     : m == 4 ? (const void*)window_runs_kernel<4>
+                              : (const void*)window_runs_kernel<8>;
+    e = launch_chained(fn, dim3(runs ? (windows + m - 1) / m : windows), dim3(kWindowThreads), hparams, 0, s);
+  }
   if (own) free(a);
   if (e != cudaSuccess) return cuda_fail(e);
   st->flat_launches += 1;

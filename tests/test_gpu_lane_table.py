@@ -178,6 +178,74 @@ def test_recounted_is_the_samples_misjudgements(sizes, cuts, overlap):
     st.close()
 
 
+def _sample_hist(x, addr):
+    """A chunk's sample (_sample_flag) as a histogram, and its pixels' weight."""
+    head = min((16 - addr % 16) % 16, x.size)
+    nvec = (x.size - head) // 16
+    if nvec < 256:
+        return oracle.hist_u32(x), np.float32(1.0 if x.size else 0.0)
+    v = (np.arange(256, dtype=np.int64) * nvec) // 256
+    y = x[(head + 16 * v)[:, None] + np.arange(16)[None, :]].reshape(-1)
+    return oracle.hist_u32(y), np.float32(x.size) / np.float32(4096)
+
+
+# pushes of as many chunks as one window a CTA takes, one more, and so on for
+# four and eight windows a CTA, windows shorter and longer than the pushes
+@pytest.mark.parametrize("mode,window,pushes", [
+    (hl.MODE_AUTO, 256, [1, 2, 152, 153, 305]),
+    (hl.MODE_AUTO, 100, [304, 305, 608]),
+    (hl.MODE_AUTO, 165, [609, 7, 152]),
+    (hl.MODE_AUTO, 5, [152, 153, 305, 609]),
+    (hl.MODE_ADAPTIVE, 7, [1, 2, 3, 400, 1]),
+    (hl.MODE_PLAIN, 256, [3, 200, 2, 1]),
+])
+def test_windows_of_long_pushes(mode, window, pushes):
+    """The window, the switches and, in AUTO mode, the windows whose switch
+    their samples misjudge (a host model in FP32 and the chunks' order;
+    windows within 1e-5 of the threshold count either way)."""
+    rng = np.random.default_rng(window)
+    count = sum(pushes)
+    sizes = [int(n) for n in rng.choice([0, 700, 4111, 4200, 5000, 7001], count)]
+    offs = np.cumsum([0] + [n + int(rng.integers(0, 20)) for n in sizes])[:-1]
+    host = rng.integers(0, 256, int(offs[-1]) + sizes[-1] + 16).astype(np.uint8)
+    for o, n in zip(offs, sizes):
+        x = host[o:o + n]
+        x[rng.random(n) < 0.4475 + 0.01 * rng.standard_normal()] = 9
+    bd = dev(host)
+    outs = torch.full((count, 256), -1, dtype=torch.int32, device="cuda")
+    st = hl.Stream(mode=mode, window=window)
+    ref = oracle.StreamOracle(8192, mode=mode, window=window)
+    low = high = done = 0
+    sampled = []
+    for push in pushes:
+        lo, hi = done, done + push
+        st.push_many(np.uint64(bd.data_ptr()) + offs[lo:hi].astype(np.uint64), np.array(sizes[lo:hi], dtype=np.uint64),
+                     np.array([outs[j].data_ptr() for j in range(lo, hi)], dtype=np.uint64))
+        for j in range(lo, hi):
+            x = host[offs[j]:offs[j] + sizes[j]]
+            rec = ref.push(x)
+            sampled.append(_sample_hist(x, bd.data_ptr() + int(offs[j])))
+            if mode != hl.MODE_AUTO or j + 1 == hi:
+                continue
+            f = np.zeros(256, np.float32)
+            for s, w in sampled[-window:]:
+                f = (s.astype(np.float64) * np.float64(w) + f).astype(np.float32)
+            fm, fs = float(f.max()) * 1000.0, float(f.astype(np.float64).sum()) * 450.0
+            near = abs(fm - fs) <= 1e-5 * fs
+            wrong = int(fs > 0 and fm >= fs) != ref.flag
+            low += wrong and not near
+            high += wrong or near
+        done = hi
+        s = st.state()
+        assert s.flag == ref.flag and s.last_kernel == rec.kernel and s.status == 0
+        assert low <= s.recounted <= high, push
+        assert np.array_equal(st.window().cpu().numpy().view(np.uint64), ref.mw)
+    assert np.array_equal(u32(outs).reshape(count, 256), np.stack([oracle.hist_u32(host[o:o + n]) for o, n in zip(offs, sizes)]))
+    if mode == hl.MODE_AUTO and window < 10:
+        assert low > 0
+    st.close()
+
+
 def test_a_captured_push_replayed():
     """Pushes of one and of two chunks captured into a graph and replayed over
     new pixels: totals, the last two patterns and the switch follow the
