@@ -159,7 +159,8 @@ def measured_peaks():
 # The sources a kernel is compiled from (its translation unit and headers).
 KERNEL_SOURCES = {
     "batch_flat_kernel": ["paper_1011_0235_gb300/csrc/hist_stream.cu", "paper_1011_0235_gb300/csrc/hist_device.cuh",
-                          "paper_1011_0235_gb300/csrc/hist_internal.h", "include/hist.h"],
+                          "paper_1011_0235_gb300/csrc/hist_internal.h", "paper_1011_0235_gb300/csrc/hist_plan.h",
+                          "include/hist.h"],
 }
 
 
@@ -274,8 +275,9 @@ def host_fed_extras(torch, hl, hx, chunks, steps):
     """Sec. III.B's host-fed stream on this machine (Table 3's question: how
     much of the transfer the kernels hide): GB/s of the adaptive stream fed
     from pinned host memory, sequentially (each chunk copied, then counted,
-    on one CUDA stream) and pipelined through 2, 3 and 4 staging buffers
-    (copies on their own stream, overlapped with the kernels)."""
+    on one CUDA stream) and pipelined (hist_stream_push_host with 2, 3 and 4
+    staging buffers attached, which pinned chunks do not use: the counting
+    kernels read them over the host link)."""
     res = {}
     d = torch.empty(CHUNK, dtype=torch.uint8, device="cuda")
     st = hl.Stream(budget=8192, mode=hl.MODE_ADAPTIVE)
@@ -570,9 +572,8 @@ def serving_extras(torch, np, hl, synth, hbm, rates=SERVE_RATES):
     cap = run(reqs, at_zero=True)
     cap["frac_of_hbm"] = round(cap["served_gbs"] / hbm, 4)
     # the counting kernels' own rate on this mix: each stream's 64 MiB region
-    # counted once by the kernel AUTO gives its law (the adaptive kernel's
-    # full table for the degenerate streams, the per-warp kernel for the
-    # rest), the requests' bytes weighted by it
+    # counted once by the kernel AUTO gives its law (one-shot calls on 64 MiB,
+    # launch included), the requests' bytes weighted by it
     o = hl.empty_hist()
 
     def t_of(f):
@@ -597,9 +598,7 @@ def serving_extras(torch, np, hl, synth, hbm, rates=SERVE_RATES):
     nbytes = float(sum(r.n for r in reqs))
     cap["auto_kernels_alone_gbs"] = round(nbytes / sum(r.n / rate[r.stream] for r in reqs) / 1e9, 1)
     out["capacity"] = cap
-    # the same burst with every stream in ADAPTIVE mode (the full table for
-    # every law): what the serving loop delivers when the switch's choice of
-    # the per-warp kernel does not bound it
+    # the same burst with every stream in ADAPTIVE mode
     cad = run(reqs, at_zero=True, mode=hl.MODE_ADAPTIVE)
     cad["frac_of_hbm"] = round(cad["served_gbs"] / hbm, 4)
     out["capacity_adaptive"] = cad
@@ -646,8 +645,8 @@ def summary_of(ex, value, hbm):
     if ad and pl:
         sm["degenerate_gbs"] = {"adaptive": ad, "plain": pl, "auto": au, "auto_window32": g("degenerate_auto_window32_gbs"),
                                 "adaptive_over_plain": round(ad / pl, 2),
-                                "note": "3x would need %.0f GB/s, above the HBM copy peak: same-bin increments of "
-                                        "the per-warp kernel are not serialised on this GPU" % (3 * pl)}
+                                "note": "3x would need %.0f GB/s, above the HBM copy peak: both kernels count in the "
+                                        "lane-private table" % (3 * pl)}
     sm["table2_plain_gbs"] = dict(zip(g("table2", "inputs") or [], g("table2", "plain_gbs") or []))
     sm["batch_graph_gbs"] = g("batch_graph_gbs")
     sm["batch_regimes_graph_gbs"] = g("batch_regimes", "graph_gbs")
@@ -746,7 +745,7 @@ def run_part(args):
         ptrs = [xdg.data_ptr() + c * CHUNK for c in range(64)]
         out = {}
         # a window of one chunk, then a window of 32 chunks (its window
-        # kernels, one CTA per chunk), both with the chunks declared complete
+        # kernel), both with the chunks declared complete
         for name, window in (("auto", 1), ("auto_window32", 32)):
             st = hl.Stream(budget=8192, mode=hl.MODE_AUTO, window=window, overlap=True)
             el = time_steps(torch, lambda: st.push_many(ptrs, [CHUNK] * 64), 1, 2)
@@ -777,8 +776,8 @@ def run_part(args):
         # the 4096-image batch tuned per regime, then one graph launch
         out = batch_extras(torch, hl, synth, 6800.0, steps=1, autotune=True)
     elif args.profile_part == "budget960":
-        # the headline's N(128, 8) stream with the paper's 960-slot table:
-        # predict_kernel, then the counting launch; 3 pushes of 64 chunks
+        # the headline's N(128, 8) stream with the paper's 960-slot pattern:
+        # 3 pushes of 64 chunks
         x = gen_workload_device(torch, synth, 64, synth.SEED_BASE + 2, lambda c: synth.normal(128, 8))
         st = hl.Stream(budget=960, mode=hl.MODE_ADAPTIVE)
         ptrs = [x.data_ptr() + c * CHUNK for c in range(64)]
@@ -922,8 +921,8 @@ def run_native(args):
         extras["oneshot_plain_gbs"] = round(nbytes * 10 / e4 / 1e9, 2)
         st_pl.close()
         # the same stream below the full table (the paper's 960 slots and
-        # between): layouts predicted from samples; beside it, one
-        # hist_adaptive call over the same bytes with the rule's pattern
+        # between); beside it, one hist_adaptive call over the same bytes with
+        # the rule's pattern
         sb = {"budgets": [960, 2048, 4096]}
         hx1 = hl.hist_plain(x, hl.empty_hist())
         for name, mode in (("adaptive", hl.MODE_ADAPTIVE), ("auto", hl.MODE_AUTO)):
@@ -1006,8 +1005,8 @@ def run_native(args):
         e2e = {"value": round(world * nbytes * ksteps / el_e / 1e9, 2), "unit": UNIT,
                "h2d_bytes_per_step": nbytes, "d2h_bytes_per_step": 256 * 8, "steps": ksteps,
                "windows_gbs": [round(world * nbytes * ksteps / w / 1e9, 2) for w in wins],
-               "path": "hist_stream_push_host: pinned host -> 3 staging buffers, copies overlapped with kernels; "
-                       "median of three windows of `steps` steps",
+               "path": "hist_stream_push_host: pinned host memory read by the counting kernels over the host link, a "
+                       "chunk's reads beside the launch before; median of three windows of `steps` steps",
                "h2d_copy_gbs": round(nbytes * 3 / el_c / 1e9, 2)}
         st_e.close()
         if world == 1:

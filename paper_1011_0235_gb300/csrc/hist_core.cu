@@ -241,8 +241,6 @@ int sm_count() {
   return sms;
 }
 
-int ensure_smem_attr(const void* fn, int* done) { return ensure_smem_attr_bytes(fn, done, kSmemBytes); }
-
 int ensure_smem_attr_bytes(const void* fn, int* done, size_t bytes) {
   // Kernels using more than 48 KiB of dynamic shared memory need the opt-in,
   // once per (kernel, device); `done` is the caller's per-kernel array of

@@ -14,8 +14,7 @@ constexpr int kMaxDevices = 64;
 int cuda_fail(cudaError_t e);
 // SMs of the current device.
 int sm_count();
-// Opt a kernel into the library's dynamic shared-memory size on this device.
-int ensure_smem_attr(const void* fn, int* done);
+// Opt a kernel into `bytes` of dynamic shared memory on this device.
 int ensure_smem_attr_bytes(const void* fn, int* done, size_t bytes);
 // Allow a kernel clusters of more than 8 CTAs on this device (once per kernel
 // and device; `done` as above).
