@@ -1,7 +1,7 @@
 """GB300 (sm_103a) exact 256-bin histograms of 8-bit pixel streams.
 
 Python binding of the C ABI in ``include/hist.h`` ("Fast Histograms using
-Adaptive CUDA Streams": per-warp and adaptive sub-binned kernels, the binning
+Adaptive CUDA Streams": plain and adaptive sub-binned kernels, the binning
 pattern, the degeneracy switch and the chunked stream, all on the device).
 
 Tensors are ``torch`` CUDA tensors; the work is enqueued on the current torch
@@ -94,7 +94,7 @@ def as_u64(h: torch.Tensor):
 # ---------------------------------------------------------------- one-shot --
 
 def hist_plain(x: torch.Tensor, out: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
-    """Per-warp kernel (NVHist).  Returns a 256-entry int32 tensor holding u32 counts."""
+    """Plain kernel (NVHist's place).  Returns a 256-entry int32 tensor holding u32 counts."""
     x = _dev_u8(x)
     out = empty_hist(x.device) if out is None else _dev_buf(out, 4 * BINS, "out", 4)
     _abi.check("hist_plain", lib().hist_plain(x.data_ptr(), x.numel(), out.data_ptr(), _stream_ptr(stream)))
@@ -334,7 +334,8 @@ class Stream:
         _abi.check("hist_stream_attach_staging", lib().hist_stream_attach_staging(self._h, max_chunk, depth))
 
     def push_host(self, ptr: int, n: int, out_ptr: Optional[int] = None, stream=None) -> None:
-        """Push a chunk held in host memory at `ptr` (pinned for overlap)."""
+        """Push a chunk held in host memory at `ptr` (pinned memory is read in
+        place by the counting kernel, other memory copied first)."""
         _abi.check("hist_stream_push_host", lib().hist_stream_push_host(self._h, ptr, n, out_ptr, _stream_ptr(stream)))
 
     def flush(self, stream=None) -> None:
