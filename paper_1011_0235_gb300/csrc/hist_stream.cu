@@ -823,6 +823,35 @@ __global__ void __launch_bounds__(kThreads, 1) batch_flat_kernel(const __grid_co
   }
 }
 
+// A push of one short chunk: one CTA, without a plan, a chunk table or
+// accumulators.  Bound by the chain of the wait, one or two rounds of loads,
+// the reduction, the epilogue's pattern and the launch itself; batch_flat_kernel
+// reads its ranges and its chunk's entry from 6.6 KB of parameters first (two
+// constant misses) and clears the groups' tables.  A chunk of 9001 bytes in AUTO
+// mode, pushes in a row: 5.1 -> 3.5 us (declared complete 3.8 -> 2.2).
+__global__ void __launch_bounds__(kThreads, 1) push_one_kernel(const PushHead a, const FlatDesc d) {
+  __shared__ __align__(16) uint32_t table[kTableWords];
+  __shared__ uint32_t res[HIST_BINS], eh[HIST_BINS];
+  __shared__ EpiShared es;
+  const int t = threadIdx.x;
+  pdl_launch_dependents();
+  zero_table(table);
+  if (t < HIST_BINS) eh[t] = 0;
+  if (!a.early) pdl_wait();
+  __syncthreads();
+  if (d.n) piece_count(d.in, d.n, table, eh, nullptr, nullptr);
+  __syncthreads();
+  lane_reduce<kThreads, false>(table, res, t);
+  __syncthreads();
+  if (t >= HIST_BINS) return;
+  if (a.early) pdl_wait();
+  if (t == 0) flat_prev_done(a);
+  flat_epilogue(a, d, res[t] + eh[t], 0u, es, t, kEpiBar);
+  const GroupBar<HIST_BINS> bar = {kEpiBar};
+  bar.sync();
+  if (t == 0) flat_finish(a, 1);
+}
+
 // A window of W > 1 chunks.  The window histogram after chunk g is the sum
 // of the histograms of chunks g-W+1 .. g (chunks before number 0 count as
 // empty; a resumed stream restarts at 0).  The histograms of the last
@@ -1238,6 +1267,47 @@ uint32_t flat_plan(RangePlan* p, uint32_t count, const size_t* ns, uint32_t grid
 // streams.
 constexpr uint32_t kHostGrid = 16;
 
+// What every kernel of the next push of `count` chunks is given, and the
+// stream's counters after it.
+void push_head(const hist_stream* st, uint32_t count, bool host, PushHead* a) {
+  a->st = st->d;
+  a->count = count;
+  a->first_chunk = st->flat_chunks;
+  a->window = st->cfg.window;
+  a->launch = st->flat_launches + 1;
+  a->prev = st->prev_launch;
+  a->budget = st->cfg.budget;
+  a->theta = st->cfg.theta_milli;
+  a->mode = st->cfg.mode;
+  a->early = host ? kHostChunk : (st->cfg.flags & HIST_OVERLAP_PUSHES) ? 1u : 0u;
+}
+void pushed(hist_stream* st, uint32_t count) {
+  st->flat_launches += 1;
+  st->prev_launch = st->flat_launches;
+  st->flat_chunks += count;
+  st->chunks_launched += count;
+}
+
+// A push of one chunk of at most kOneMax bytes (window of one chunk, no trace)
+// is one CTA's (push_one_kernel); pushes in a row, with batch_flat_kernel and so:
+// 16 bytes 4.6 and 3.2 us, 16 KiB 5.4 and 3.6, 64 KiB 6.3 and 4.8, 128 KiB 8.0
+// and 6.5.
+constexpr size_t kOneMax = 128u << 10;
+int launch_one(hist_stream* st, const uint8_t* in, size_t n, uint32_t* out, bool host, cudaStream_t s) {
+  PushHead a;
+  push_head(st, 1, host, &a);
+  FlatDesc d;
+  d.in = in;
+  d.out = out;
+  d.n = (uint32_t)n;
+  d.j = 0;
+  void* params[] = {&a, &d};
+  const cudaError_t e = launch_chained((const void*)push_one_kernel, dim3(1), dim3(kThreads), params, 0, s);
+  if (e != cudaSuccess) return cuda_fail(e);
+  pushed(st, 1);
+  return HIST_OK;
+}
+
 // The launches of one batch: the counting launch, and with a window of more
 // than one chunk the window's switches.  Each may start while the one before
 // ends and waits for it before it reads what that one writes.  `host`: the
@@ -1253,19 +1323,10 @@ int launch_batch(hist_stream* st, uint32_t count, const uint8_t* const* ins, con
   A* a = own ? (A*)calloc(1, sizeof(A)) : (A*)st->args;
   if (!a) return HIST_ENOMEM;
   if (!own) memset((void*)a, 0, (size_t)((char*)a->c - (char*)a));
-  a->st = st->d;
-  a->count = count;
-  a->first_chunk = st->flat_chunks;
-  a->window = st->cfg.window;
-  a->launch = st->flat_launches + 1;
-  a->prev = st->prev_launch;
-  a->budget = st->cfg.budget;
-  a->theta = st->cfg.theta_milli;
-  a->mode = st->cfg.mode;
+  push_head(st, count, host, a);
   a->trace = st->trace;
   a->trace_cap = st->trace_cap;
   a->trace_first = st->trace_next;
-  a->early = host ? kHostChunk : (st->cfg.flags & HIST_OVERLAP_PUSHES) ? 1u : 0u;
   for (uint32_t i = 0; i < count; ++i) {
     a->c[i].in = ins[i];
     a->c[i].n = (uint32_t)ns[i];
@@ -1296,16 +1357,15 @@ int launch_batch(hist_stream* st, uint32_t count, const uint8_t* const* ins, con
   }
   if (own) free(a);
   if (e != cudaSuccess) return cuda_fail(e);
-  st->flat_launches += 1;
-  st->prev_launch = st->flat_launches;
-  st->flat_chunks += count;
-  st->chunks_launched += count;
+  pushed(st, count);
   if (st->trace) st->trace_next += count;
   return HIST_OK;
 }
 
 int push_chunks(hist_stream* st, uint32_t count, const uint8_t* const* ins, const size_t* ns, uint32_t* const* outs,
                 cudaStream_t s, bool host = false) {
+  if (count == 1 && ns[0] <= kOneMax && st->cfg.window == 1 && !st->trace)
+    return launch_one(st, ins[0], ns[0], outs ? outs[0] : nullptr, host, s);
   for (uint32_t i = 0; i < count; i += kMaxBatch) {
     const uint32_t c = count - i < kMaxBatch ? count - i : kMaxBatch;
     int rc = c <= kSmallBatch ? launch_batch<SmallArgs>(st, c, ins + i, ns + i, outs ? outs + i : nullptr, host, s)
@@ -1529,8 +1589,8 @@ int hist_stream_push_host(hist_stream* st, const uint8_t* h_chunk, size_t n, uin
   // Pinned memory is counted in place, a chunk's reads beside the launch
   // before it, as with HIST_OVERLAP_PUSHES (the caller's bytes were complete
   // before too: the copies waited for no work of his).  Copied into staging,
-  // with the events between copy and count, and now: 64 x 64 KiB 729 -> 263
-  // us, 64 x 1 MiB 860 -> 421, 16 x 4 MiB 404 -> 350, 16 x 16 MiB 1335 -> 1298
+  // with the events between copy and count, and now: 64 x 64 KiB 729 -> 199
+  // us, 64 x 1 MiB 860 -> 410, 16 x 4 MiB 404 -> 342, 16 x 16 MiB 1335 -> 1296
   // (1272 at the link's rate).
   if (const uint8_t* d = n ? host_readable(h_chunk, n, (cudaStream_t)s) : nullptr)
     return push_chunks(st, 1, &d, &n, d_chunk_out ? &d_chunk_out : nullptr, (cudaStream_t)s, true);

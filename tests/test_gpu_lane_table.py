@@ -178,6 +178,41 @@ def test_recounted_is_the_samples_misjudgements(sizes, cuts, overlap):
     st.close()
 
 
+@pytest.mark.parametrize("mode,overlap,window", [(hl.MODE_AUTO, False, 1), (hl.MODE_PLAIN, True, 1),
+                                                 (hl.MODE_ADAPTIVE, False, 1), (hl.MODE_AUTO, True, 2)])
+def test_single_pushes_around_the_one_cta_limit(mode, overlap, window):
+    """Pushes of one chunk on both sides of the largest that one CTA counts
+    alone, at every alignment, without an output now and then, between pushes
+    of several chunks: outputs and the state after each push are the oracle's."""
+    rng = np.random.default_rng(11 + mode)
+    sizes = [0, 1, 15, 143, 4097, 16_384, 65_536, 65_537, 131_071, 131_072, 131_073, 200_000]
+    x = rng.integers(0, 256, 500_000, dtype=np.uint8)
+    x[rng.random(x.size) < 0.46] = 9
+    xd = dev(x)
+    st = hl.Stream(mode=mode, overlap=overlap, window=window)
+    ref = oracle.StreamOracle(oracle.BUDGET_MAX, mode=mode, window=window)
+    outs = torch.full((3 * len(sizes), 256), -1, dtype=torch.int32, device="cuda")
+    torch.cuda.synchronize()
+    for i in range(3 * len(sizes)):
+        n, off = sizes[(5 * i) % len(sizes)], int(rng.integers(0, 299_000))
+        st.push_ptr(xd.data_ptr() + off, n, None if i % 5 == 4 else outs[i].data_ptr())
+        rec = ref.push(x[off:off + n])
+        if i % 7 == 6:
+            st.push_many([xd.data_ptr() + 3, xd.data_ptr() + 40_000], [30_001, 140_000])
+            ref.push(x[3:30_004])
+            rec = ref.push(x[40_000:180_000])
+        if i % 3 == 2:
+            s = st.state()
+            assert bytes(s.pattern) == ref.pattern.to_bytes() and bytes(s.last_pattern) == rec.pattern.to_bytes(), i
+            assert s.flag == ref.flag and s.last_kernel == rec.kernel and s.chunks == ref.chunks and s.status == 0
+            assert np.array_equal(np.array(s.last_hist, np.uint32), rec.hist)
+            assert np.array_equal(np.array(s.totals, np.uint64), ref.totals)
+        got = None if i % 5 == 4 else u32(outs[i])
+        if i % 7 != 6 and got is not None:
+            assert np.array_equal(got, rec.hist), (i, n)
+    st.close()
+
+
 def _sample_hist(x, addr):
     """A chunk's sample (_sample_flag) as a histogram, and its pixels' weight."""
     head = min((16 - addr % 16) % 16, x.size)
