@@ -767,8 +767,8 @@ __device__ __forceinline__ void flat_groups(const A& a, uint32_t nwl, int first,
 // flight; one CTA per SM has no such pair.  Bound by the HBM read on large
 // chunks, by a chain of round trips to L2 on one small one: on the GPU,
 // pushes in a row, 64 x 16 MiB 166.6 -> 158.7 us (6.8 TB/s; overlapping
-// 162 -> 155.7 us), 128 x 1 MiB 39.2 -> 28.1 us, one chunk of 9 KB in AUTO
-// mode 17.4 -> 5.3 us, of 1 MiB 15.6 -> 7.6 us.
+// 162 -> 155.7 us), 128 x 1 MiB 39.2 -> 28.1 us, one chunk of 1 MiB
+// 15.6 -> 7.6 us.
 template <class A>
 __global__ void __launch_bounds__(kThreads, 1) batch_flat_kernel(const __grid_constant__ A a) {
   extern __shared__ __align__(16) uint32_t tables[];
