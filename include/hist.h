@@ -140,6 +140,12 @@ int degeneracy_u64(const uint64_t* d_hist, uint32_t theta_milli, hist_degeneracy
  * only if n == 0. */
 int hist_plain(const uint8_t* d_in, size_t n, uint32_t* d_out, hist_cuda_stream s);
 
+/* Test hook: hist_plain as it runs where no cluster of more than `widest` CTAs
+ * (1..16) can be placed -- on a part of a GPU -- so that inputs of more than
+ * 16 KiB for each of them take the kernels of longer inputs.  The counts are
+ * the same.  HIST_EINVAL for a width out of range. */
+int hist_plain_test_cluster(const uint8_t* d_in, size_t n, uint32_t widest, uint32_t* d_out, hist_cuda_stream s);
+
 /* Adaptive kernel (AHist, Sec. III.A) for the device-resident pattern d_pat.
  * Same contract as hist_plain.  The counts are those of the pattern's slots
  * summed per bin, which every valid pattern gives; they are held in the

@@ -215,6 +215,7 @@ SIGNATURES = [
     ("degeneracy", _I, [_P, _U32, _P, _P]),
     ("degeneracy_u64", _I, [_P, _U32, _P, _P]),
     ("hist_plain", _I, [_P, _Z, _P, _P]),
+    ("hist_plain_test_cluster", _I, [_P, _Z, _U32, _P, _P]),
     ("hist_adaptive", _I, [_P, _Z, _P, _P, _P]),
     ("hist_config_init", None, [ctypes.POINTER(HistConfig)]),
     ("hist_stream_create", _I, [ctypes.POINTER(HistConfig), ctypes.POINTER(_P)]),

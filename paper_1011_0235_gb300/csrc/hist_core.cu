@@ -4,6 +4,8 @@
 #include <stdint.h>
 #include <string.h>
 
+#include <atomic>
+
 #include "hist.h"
 #include "hist_device.cuh"
 #include "hist_internal.h"
@@ -41,8 +43,8 @@ __device__ __forceinline__ uint32_t cluster_ld(uint32_t a, uint32_t rank) {
   return v;
 }
 
-// A short input: one cluster of 1, 2, 4, 8 or 16 CTAs counts it, each CTA an
-// equal part, and the CTAs sum each other's tables through distributed
+// A short input: one cluster of 1, 2, 4, 8 or 16 CTAs (as far as the device
+// places them: widest_cluster) counts it, each CTA an equal part, and the CTAs sum each other's tables through distributed
 // shared memory: no cleared output, no global atomics, one launch.  Bound by
 // latency (launch, one round of loads, two barriers of the cluster): 1 MiB of
 // uniform pixels 10.3 -> 4.8 us a call in a row (a clearing memset and 16
@@ -255,17 +257,6 @@ int ensure_smem_attr_bytes(const void* fn, int* done, size_t bytes) {
   return HIST_OK;
 }
 
-int ensure_wide_cluster(const void* fn, int* done) {
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return cuda_fail(e);
-  if (dev >= 0 && dev < kMaxDevices && done[dev]) return HIST_OK;
-  e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  if (e != cudaSuccess) return cuda_fail(e);
-  if (dev >= 0 && dev < kMaxDevices) done[dev] = 1;
-  return HIST_OK;
-}
-
 // Bytes of one load per thread of a CTA: a cluster has a CTA for each, up to
 // 16.
 constexpr size_t kClusterStep = (size_t)kThreads * 16;
@@ -277,49 +268,85 @@ constexpr size_t kClusterStep = (size_t)kThreads * 16;
 constexpr size_t kClusterMax = 16 * 4 * kClusterStep;
 constexpr size_t kOneshotSmem = (size_t)kTableWords * 4;
 
-int oneshot(const uint8_t* d_in, size_t n, uint32_t* d_out, cudaStream_t s) {
+// A one-shot launch that may start while the work before it on `s` ends, of
+// `grid` CTAs, or of one cluster of that many (`at`: room for its attributes).
+static cudaLaunchConfig_t oneshot_launch(unsigned grid, bool cluster, cudaLaunchAttribute (&at)[2], cudaStream_t s) {
+  cudaLaunchConfig_t lc = {};
+  lc.gridDim = dim3(grid);
+  lc.blockDim = dim3(kThreads);
+  lc.dynamicSmemBytes = kOneshotSmem;
+  lc.stream = s;
+  lc.attrs = at;
+  lc.numAttrs = cluster ? 2 : 1;
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = grid;
+  at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+  return lc;
+}
+
+// The widest cluster of oneshot_cluster_kernel (a power of two up to 16) that
+// the current device places, asked once per device: a CTA fills an SM, and
+// a part of a GPU may have no 16 SMs in one place.
+static uint32_t widest_cluster() {
+  static std::atomic<uint32_t> known[kMaxDevices];
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess) cudaGetLastError();
+  const bool keep = dev >= 0 && dev < kMaxDevices;
+  if (keep)
+    if (const uint32_t w = known[dev].load(std::memory_order_relaxed)) return w;
+  bool asked = true;
+  uint32_t c = 16;
+  for (; c > 1; c >>= 1) {
+    cudaLaunchAttribute at[2];
+    const cudaLaunchConfig_t lc = oneshot_launch(c, true, at, nullptr);
+    int placed = 0;
+    cudaError_t e = cudaSuccess;
+    if (c > 8)  // (more than the portable size)
+      e = cudaFuncSetAttribute((const void*)oneshot_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&placed, oneshot_cluster_kernel, &lc);
+    if (e == cudaSuccess && placed > 0) break;
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      asked = asked && e == cudaErrorInvalidClusterSize;
+    }
+  }
+  if (keep && asked) known[dev].store(c, std::memory_order_relaxed);
+  return c;
+}
+
+int oneshot(const uint8_t* d_in, size_t n, uint32_t* d_out, cudaStream_t s, uint32_t widest) {
   if (!d_out || (!d_in && n) || n >= ((size_t)1 << 32)) return HIST_EINVAL;
   cudaError_t e;
   if (n == 0) {
     e = cudaMemsetAsync(d_out, 0, HIST_BINS * sizeof(uint32_t), s);
     return e == cudaSuccess ? HIST_OK : cuda_fail(e);
   }
-  cudaLaunchConfig_t lc = {};
-  cudaLaunchAttribute at[2];
-  lc.stream = s;
-  lc.attrs = at;
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  lc.numAttrs = 1;
   const uint32_t nvec = (uint32_t)split_bytes(d_in, n).nvec;
+  cudaLaunchAttribute at[2];
   if (n <= kClusterMax) {
     unsigned c = 1;
     while (c < 16 && c * kClusterStep < n) c <<= 1;
-    static int wide_done[kMaxDevices];
-    if (c > 8) {
-      const int rc = ensure_wide_cluster((const void*)oneshot_cluster_kernel, wide_done);
-      if (rc) return rc;
+    // a cluster that cannot be placed leaves the input to the grid below
+    if (c == 1 || c <= (widest ? widest : widest_cluster())) {
+      const cudaLaunchConfig_t lc = oneshot_launch(c, c > 1, at, s);
+      e = cudaLaunchKernelEx(&lc, oneshot_cluster_kernel, d_in, (uint32_t)n, d_out, make_parts(nvec, c));
+      if (e == cudaSuccess) return HIST_OK;
+      // (the answer is the device's; a context may hold fewer of its SMs)
+      const bool placed = e != cudaErrorInvalidClusterSize && e != cudaErrorLaunchOutOfResources &&
+                          e != cudaErrorInvalidConfiguration;
+      if (c == 1 || placed) return cuda_fail(e);
+      cudaGetLastError();
     }
-    lc.gridDim = dim3(c);
-    lc.blockDim = dim3(kThreads);
-    lc.dynamicSmemBytes = kOneshotSmem;
-    if (c > 1) {
-      at[1].id = cudaLaunchAttributeClusterDimension;
-      at[1].val.clusterDim.x = c;
-      at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
-      lc.numAttrs = 2;
-    }
-    e = cudaLaunchKernelEx(&lc, oneshot_cluster_kernel, d_in, (uint32_t)n, d_out, make_parts(nvec, c));
-    return e == cudaSuccess ? HIST_OK : cuda_fail(e);
   }
-  lc.gridDim = dim3(1);
+  const uint32_t grid = (uint32_t)sm_count();
+  cudaLaunchConfig_t lc = oneshot_launch(1, false, at, s);
   lc.blockDim = dim3(HIST_BINS);
+  lc.dynamicSmemBytes = 0;
   e = cudaLaunchKernelEx(&lc, oneshot_clear_kernel, d_out);
   if (e != cudaSuccess) return cuda_fail(e);
-  const uint32_t grid = (uint32_t)sm_count();
-  lc.gridDim = dim3(grid);
-  lc.blockDim = dim3(kThreads);
-  lc.dynamicSmemBytes = kOneshotSmem;
+  lc = oneshot_launch(grid, false, at, s);
   e = cudaLaunchKernelEx(&lc, oneshot_kernel, d_in, (uint32_t)n, d_out, make_parts(nvec, grid));
   return e == cudaSuccess ? HIST_OK : cuda_fail(e);
 }
@@ -369,13 +396,18 @@ int hist_pattern_check(const hist_pattern* p) {
 }
 
 int hist_plain(const uint8_t* d_in, size_t n, uint32_t* d_out, hist_cuda_stream s) {
-  return oneshot(d_in, n, d_out, (cudaStream_t)s);
+  return oneshot(d_in, n, d_out, (cudaStream_t)s, 0);
+}
+
+int hist_plain_test_cluster(const uint8_t* d_in, size_t n, uint32_t widest, uint32_t* d_out, hist_cuda_stream s) {
+  if (widest < 1 || widest > 16) return HIST_EINVAL;
+  return oneshot(d_in, n, d_out, (cudaStream_t)s, widest);
 }
 
 int hist_adaptive(const uint8_t* d_in, size_t n, const hist_pattern* d_pat, uint32_t* d_out,
                   hist_cuda_stream s) {
   if (!d_pat) return HIST_EINVAL;
-  return oneshot(d_in, n, d_out, (cudaStream_t)s);
+  return oneshot(d_in, n, d_out, (cudaStream_t)s, 0);
 }
 
 int binning_pattern(const uint32_t* d_prev_hist, uint32_t budget, hist_pattern* d_pat, hist_cuda_stream s) {

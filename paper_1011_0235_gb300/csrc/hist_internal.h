@@ -16,10 +16,8 @@ int cuda_fail(cudaError_t e);
 int sm_count();
 // Opt a kernel into `bytes` of dynamic shared memory on this device.
 int ensure_smem_attr_bytes(const void* fn, int* done, size_t bytes);
-// Allow a kernel clusters of more than 8 CTAs on this device (once per kernel
-// and device; `done` as above).
-int ensure_wide_cluster(const void* fn, int* done);
-// The one-shot histogram (hist_plain / hist_adaptive).
-int oneshot(const uint8_t* d_in, size_t n, uint32_t* d_out, cudaStream_t s);
+// The one-shot histogram (hist_plain / hist_adaptive) with clusters of at most
+// `widest` CTAs (0: as many as the device places).
+int oneshot(const uint8_t* d_in, size_t n, uint32_t* d_out, cudaStream_t s, uint32_t widest);
 
 }  // namespace histlib

@@ -1,5 +1,8 @@
 """The lane-private counting paths at the sizes where their splits change,
 against the oracle, bit-exact."""
+import os
+import subprocess
+import sys
 import time
 
 import numpy as np
@@ -41,6 +44,53 @@ def test_oneshot_cluster_and_grid_splits(n):
         assert np.array_equal(u32(hl.hist_plain(xd[off:off + n], out)), ref), off
         out.fill_(9)
         assert np.array_equal(u32(hl.hist_adaptive(xd[off:off + n], pat, out)), ref), off
+
+
+@pytest.mark.parametrize("widest", [1, 2, 8, 15, 16])
+@pytest.mark.parametrize("n", [0, 1, 143, STEP, STEP + 1, 2 * STEP + 77, 8 * STEP, 8 * STEP + 1, 16 * STEP, 64 * STEP - 3,
+                               64 * STEP, 64 * STEP + 1])
+def test_oneshot_where_wide_clusters_cannot_be_placed(n, widest):
+    """Short one-shot calls on a part of a GPU that places clusters of at most
+    `widest` CTAs: the inputs of a wider one are counted by a plain grid, on
+    both sides of every limit, at an aligned and an odd address."""
+    x = synth.host(n + 77, synth.mixture([0.3, 0.7], [10, 200], [2, 40]), SEED + 93, n)
+    xd = dev(x)
+    s = torch.cuda.current_stream().cuda_stream
+    for off in (0, 77):
+        out = torch.full((256,), -7, dtype=torch.int32, device="cuda")
+        assert hl.lib().hist_plain_test_cluster(xd.data_ptr() + off, n, widest, out.data_ptr(), s) == 0
+        assert np.array_equal(u32(out), oracle.hist_u32(x[off:off + n])), off
+
+
+def test_oneshot_cluster_hook_rejects_bad_widths():
+    out, s = hl.empty_hist(), torch.cuda.current_stream().cuda_stream
+    for widest in (0, 17, 1 << 31):
+        assert hl.lib().hist_plain_test_cluster(out.data_ptr(), 100, widest, out.data_ptr(), s) == hl._abi.EINVAL
+
+
+def test_first_call_of_a_process_is_captured():
+    """The device's widest cluster is asked for by the first call, which may
+    be a captured one."""
+    prog = """
+import numpy as np, torch
+import paper_1011_0235_gb300 as hl
+x = torch.full((300_001,), 9, dtype=torch.uint8, device="cuda")
+out, s = hl.empty_hist(), torch.cuda.Stream()
+torch.cuda.synchronize()
+g = torch.cuda.CUDAGraph()
+with torch.cuda.graph(g, stream=s):
+    hl.hist_plain(x, out)
+for _ in range(2):
+    out.zero_()
+    torch.cuda.synchronize()
+    g.replay()
+    torch.cuda.synchronize()
+    h = hl.as_u32(out)
+    assert h[9] == 300_001 and h.sum() == 300_001
+"""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", prog], cwd=root, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
 
 
 @pytest.mark.parametrize("n", [5000, 300_001, 5_000_011])
