@@ -88,13 +88,14 @@ struct PushHead {
   uint32_t mode;
   uint32_t window;                  // chunks in the moving window
   uint32_t early;                   // chunks may be read before the work before the launch completes (kHostChunk:
-                                    // over the host link, one chunk)
+                                    // over the host link, one chunk; kReplayed: a captured launch)
   unsigned long long first_chunk;   // number of this batch's first chunk among the stream's chunks
   unsigned long long launch;        // number of this launch among the stream's launches (from 1)
   unsigned long long prev;          // number of the launch before it (0: none)
 };
 
 constexpr uint32_t kHostChunk = 2;
+constexpr uint32_t kReplayed = 3;
 
 // The counting launch's parameters: the header and the chunk table.  Two
 // capacities, so that a launch of a few chunks does not carry (and the driver
@@ -365,24 +366,38 @@ __device__ __forceinline__ void flat_finish(const A& a, uint32_t epis) {
 // chunk complete when it was pushed (a.early, HIST_OVERLAP_PUSHES), a CTA
 // then waits for the work before the launch on the CUDA stream to complete
 // before it reads a chunk byte: that work may be the kernel that wrote the
-// chunk, and only the wait makes its writes visible.  A CTA also waits for
-// the previous launch to complete before its first epilogue, which reads
-// and writes the stream state, and before it first adds into a chunk ring
-// slot, the last user of the slot -- a launch at least kChunkRing / kMaxBatch
-// - 1 launches back -- must be complete (flat_ring_ready, a bounded wait for
-// the number that each launch writes once it knows the launch before it to be
-// complete).
+// chunk, and only the wait makes its writes visible.  A CTA waits for it in
+// any case before its first epilogue, which reads and writes the stream
+// state, and before it first adds into a chunk ring slot, whose last user -- a
+// launch at least kChunkRing / kMaxBatch - 1 launches back -- must be complete
+// (flat_ring_ready: by launches_done, the number that each launch writes once
+// it knows the launch before it to be complete, or by the wait).
 __device__ __forceinline__ void flat_prev_done(const PushHead& a) {
   asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(&a.st->h.launches_done), "l"(a.prev) : "memory");
 }
 
-// Thread 0.  (A launch that waited at its start has its slots: for it this
-// only checks the number, as it stood then.)
+// Thread 0, before its CTA first adds into a ring slot.  A launch that waited at
+// its start has its slots.  For an early one launches_done says that it has
+// them, or, where that number is too old -- a replayed graph sets it back to
+// what it was when its pushes were captured, and captured pushes advance the
+// launches' numbers without running -- the wait for the launch before does; a
+// captured launch always waits, since the replay before leaves the number ahead
+// of it.  Only hist_stream_test_hold_ring holds the slots for longer (a
+// bounded wait).  (1 GiB overlapping: 152.3 us a push, 153.5 if every early
+// launch waits.)
 template <class A>
 __device__ __noinline__ void flat_ring_ready(const A& a, FlatShared<A::kCap>& fs) {
   constexpr unsigned long long back = kChunkRing / kMaxBatch - 1;
   asm volatile("cp.async.wait_all;" ::: "memory");
   if (!a.early && fs.ring_seen[0] + back >= a.launch) return;
+  if (a.early) {
+    if (a.early != kReplayed && ld_acquire(&a.st->h.launches_done) + back >= a.launch) return;
+    pdl_wait();
+    if (!fs.released) {
+      fs.released = 1;
+      flat_prev_done(a);
+    }
+  }
   uint32_t it = 0;
   while (a.launch > back && ld_acquire(&a.st->h.launches_done) < a.launch - back) {
     if (++it >= kPollLimit) {
@@ -1267,9 +1282,19 @@ uint32_t flat_plan(RangePlan* p, uint32_t count, const size_t* ns, uint32_t grid
 // streams.
 constexpr uint32_t kHostGrid = 16;
 
+// Whether launches on `s` are captured (or may be: the question failed).
+bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusActive;
+  if (cudaStreamIsCapturing(s, &capture) != cudaSuccess) {
+    cudaGetLastError();
+    return true;
+  }
+  return capture != cudaStreamCaptureStatusNone;
+}
+
 // What every kernel of the next push of `count` chunks is given, and the
 // stream's counters after it.
-void push_head(const hist_stream* st, uint32_t count, bool host, PushHead* a) {
+void push_head(const hist_stream* st, uint32_t count, bool host, cudaStream_t s, PushHead* a) {
   a->st = st->d;
   a->count = count;
   a->first_chunk = st->flat_chunks;
@@ -1279,7 +1304,8 @@ void push_head(const hist_stream* st, uint32_t count, bool host, PushHead* a) {
   a->budget = st->cfg.budget;
   a->theta = st->cfg.theta_milli;
   a->mode = st->cfg.mode;
-  a->early = host ? kHostChunk : (st->cfg.flags & HIST_OVERLAP_PUSHES) ? 1u : 0u;
+  a->early = host ? kHostChunk : 0u;
+  if (!host && (st->cfg.flags & HIST_OVERLAP_PUSHES)) a->early = capturing(s) ? kReplayed : 1u;
 }
 void pushed(hist_stream* st, uint32_t count) {
   st->flat_launches += 1;
@@ -1295,7 +1321,7 @@ void pushed(hist_stream* st, uint32_t count) {
 constexpr size_t kOneMax = 128u << 10;
 int launch_one(hist_stream* st, const uint8_t* in, size_t n, uint32_t* out, bool host, cudaStream_t s) {
   PushHead a;
-  push_head(st, 1, host, &a);
+  push_head(st, 1, host, s, &a);
   FlatDesc d;
   d.in = in;
   d.out = out;
@@ -1323,7 +1349,7 @@ int launch_batch(hist_stream* st, uint32_t count, const uint8_t* const* ins, con
   A* a = own ? (A*)calloc(1, sizeof(A)) : (A*)st->args;
   if (!a) return HIST_ENOMEM;
   if (!own) memset((void*)a, 0, (size_t)((char*)a->c - (char*)a));
-  push_head(st, count, host, a);
+  push_head(st, count, host, s, a);
   a->trace = st->trace;
   a->trace_cap = st->trace_cap;
   a->trace_first = st->trace_next;
@@ -1390,12 +1416,7 @@ const uint8_t* host_readable(const uint8_t* p, size_t n, cudaStream_t s) {
     return e == cudaSuccess && found == cudaDriverEntryPointSuccess ? (Ask)f : nullptr;
   }();
   if (!ask) return nullptr;
-  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusActive;
-  if (cudaStreamIsCapturing(s, &capture) != cudaSuccess) {
-    cudaGetLastError();
-    return nullptr;
-  }
-  if (capture != cudaStreamCaptureStatusNone) return nullptr;
+  if (capturing(s)) return nullptr;
   unsigned int type = 0, managed = 1;
   CUdeviceptr d = 0, start = 0;
   size_t size = 0;
@@ -1703,14 +1724,14 @@ int hist_stream_set_state(hist_stream* st, const hist_stream_state* h, hist_cuda
   tmp.chunks = h->chunks;
   tmp.flag = h->flag;
   tmp.last_kernel = h->last_kernel;
-  // the scratch is zero again
+  // launches go on to be numbered (a graph captured before may write its own
+  // numbers), none before them is running; the scratch is zero again
+  tmp.launches_done = st->prev_launch = st->flat_launches;
   cudaError_t e = cudaMemsetAsync(st->d, 0, sizeof(StreamDev), (cudaStream_t)s);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(&st->d->h, &tmp, sizeof(StreamHead), cudaMemcpyHostToDevice, (cudaStream_t)s);
   if (e == cudaSuccess) e = cudaStreamSynchronize((cudaStream_t)s);
-  st->flat_launches = 0;   // the rings restart with the zeroed scratch
-  st->prev_launch = 0;
-  st->flat_chunks = 0;
+  st->flat_chunks = 0;  // the rings restart with the zeroed scratch
   st->resume_chunk = st->chunks_launched;  // and so does the moving window
   return e == cudaSuccess ? HIST_OK : cuda_fail(e);
 }

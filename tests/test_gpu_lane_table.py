@@ -465,6 +465,125 @@ def test_host_chunks_pinned_registered_and_pageable(depth, window, overlap):
     assert int(torch.cuda.cudart().cudaHostUnregister(reg.ctypes.data)) == 0
 
 
+@pytest.mark.parametrize("overlap", [False, True])
+@pytest.mark.parametrize("mode", [hl.MODE_AUTO, hl.MODE_ADAPTIVE])
+def test_early_pushes_after_captured_and_replayed_ones(mode, overlap):
+    """A captured push advances the stream's launch numbers without a launch,
+    and its replay sets the device's number back: pushes that start early
+    behind both (from pinned memory, and with overlap from the device) are
+    exact and no wait of theirs runs out."""
+    rng = np.random.default_rng(5 + mode)
+    n = 700_001
+    st = hl.Stream(mode=mode, overlap=overlap)
+    st.attach_staging(n, 2)
+    ref, rec, count = oracle.StreamOracle(oracle.BUDGET_MAX, mode=mode), None, 0
+    pinned = torch.empty(n, dtype=torch.uint8, pin_memory=True)
+    chunks = [rng.integers(0, 256, n - 1000 * k, dtype=np.uint8) for k in range(4)]
+    for k, c in enumerate(chunks):
+        c[rng.random(c.size) < (0.0, 0.9, 0.44, 0.5)[k]] = 31
+    on = [dev(c) for c in chunks]
+    pinned.copy_(torch.from_numpy(chunks[0]))
+    out = torch.full((256,), -1, dtype=torch.int32, device="cuda")
+    s = torch.cuda.Stream()
+    torch.cuda.synchronize()
+
+    def live(k):
+        st.push(on[k], out)
+        return chunks[k]
+
+    def host(k):
+        st.push_host(pinned.data_ptr(), n, out.data_ptr())
+        return chunks[0]
+
+    def replay(k):
+        g.replay()
+        return chunks[1]
+
+    with torch.cuda.stream(s):
+        for captured, steps in ((1, [host, live]), (6, [host, live, host]), (1, [live] * 6 + [replay, host]),
+                                (5, [replay, replay, live, live, replay, host, host, live])):
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g, stream=s):
+                for _ in range(captured):
+                    st.push(on[1], out)
+            for i, step in enumerate(steps):
+                t0 = time.monotonic()
+                data = step(i % 4)
+                for _ in range(captured if step is replay else 1):
+                    rec = ref.push(data)
+                    count += 1
+                s.synchronize()
+                assert time.monotonic() - t0 < 0.4, (captured, i)  # (a wait that runs out takes a second)
+                assert np.array_equal(u32(out), rec.hist), (captured, i)
+                state = st.state()
+                assert state.status == 0 and state.chunks == count, (captured, i)
+            # the same steps without a look between them
+            for i, step in enumerate(steps):
+                data = step(i % 4)
+                for _ in range(captured if step is replay else 1):
+                    rec = ref.push(data)
+                    count += 1
+            s.synchronize()
+            state = st.state()
+            assert np.array_equal(u32(out), rec.hist) and state.status == 0 and state.chunks == count
+            assert np.array_equal(np.array(state.totals, np.uint64), ref.totals)
+            assert bytes(state.pattern) == ref.pattern.to_bytes() and state.flag == ref.flag
+            assert state.last_kernel == rec.kernel
+            # and after a resume, with the graph from before it
+            st.set_state(state)
+            for step in (replay, host, live):
+                data = step(1)
+                for _ in range(captured if step is replay else 1):
+                    rec = ref.push(data)
+                    count += 1
+            s.synchronize()
+            state = st.state()
+            assert np.array_equal(u32(out), rec.hist) and state.status == 0 and state.chunks == count
+            assert np.array_equal(np.array(state.totals, np.uint64), ref.totals)
+    st.close()
+
+
+@pytest.mark.parametrize("overlap", [False, True])
+def test_captured_push_longer_than_the_rings(overlap):
+    """Five launches of 1024 chunks on two CTAs, captured and replayed: in each
+    a large chunk is cut between the CTAs, and the fifth launch's uses the ring
+    slot of the first's."""
+    rng = np.random.default_rng(77)
+    big, small, launches = 40 << 20, 100, 5
+    x = rng.integers(0, 256, big + launches, dtype=np.uint8)
+    x[rng.random(x.size) < 0.3] = 200
+    xd = dev(x)
+    ptrs, sizes = [], []
+    for k in range(launches * 1024):
+        launch, j = divmod(k, 1024)
+        ptrs.append(xd.data_ptr() + (launch if j == 512 else 13 * k % 1_000_000))
+        sizes.append(big if j == 512 else small)
+    outs = torch.full((launches, 256), -1, dtype=torch.int32, device="cuda")
+    rows = [outs[k // 1024].data_ptr() if k % 1024 == 512 else None for k in range(len(ptrs))]
+    st = hl.Stream(mode=hl.MODE_ADAPTIVE, grid=2, overlap=overlap)
+    s = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.stream(s):
+        with torch.cuda.graph(g, stream=s):
+            st.push_many(ptrs, sizes, rows)
+        want = np.stack([oracle.hist_u32(x[k:k + big]) for k in range(launches)])
+        total = want.astype(np.uint64).sum(axis=0)
+        for p, n in zip(ptrs, sizes):
+            if n == small:
+                at = p - xd.data_ptr()
+                total += np.bincount(x[at:at + n], minlength=256).astype(np.uint64)
+        for r in range(3):
+            outs.fill_(-1)
+            g.replay()
+            s.synchronize()
+            assert np.array_equal(u32(outs).reshape(launches, 256), want), r
+            state = st.state()
+            assert state.status == 0 and state.chunks == (r + 1) * len(ptrs)
+            assert np.array_equal(np.array(state.totals, np.uint64), (r + 1) * total)
+    st.close()
+
+
 @pytest.mark.parametrize("sizes", [
     [0, 1, 15, 16, 17, 19, 20, 255, 4079, 4080, 4095, 4096, 4097, 4100, 4111, 4112, 5000] * 4,
     [3000 + 401 * k for k in range(300)] + [2_000_003, 4096 * 256 + 1],
