@@ -465,6 +465,42 @@ def test_host_chunks_pinned_registered_and_pageable(depth, window, overlap):
     assert int(torch.cuda.cudart().cudaHostUnregister(reg.ctypes.data)) == 0
 
 
+@pytest.mark.parametrize("mode", [hl.MODE_AUTO, hl.MODE_PLAIN, hl.MODE_ADAPTIVE])
+@pytest.mark.parametrize("window", [1, 2, 5])
+def test_switch_of_host_chunks_over_a_window(window, mode):
+    """The switch and the kernel of chunks pushed from pinned and from pageable
+    memory follow the window's histogram: the window's switch differs from
+    the last chunk's on the way."""
+    rng = np.random.default_rng(window)
+    sizes = [30_000, 70_001, 140_000, 300_007]
+    top = max(sizes)
+    pinned = torch.empty(top, dtype=torch.uint8, pin_memory=True).numpy()
+    plain = np.zeros(top, np.uint8)
+    st = hl.Stream(mode=mode, window=window)
+    st.attach_staging(top, 2)
+    ref = oracle.StreamOracle(oracle.BUDGET_MAX, mode=mode, window=window)
+    single = oracle.StreamOracle(oracle.BUDGET_MAX, mode=mode)
+    out = torch.empty(256, dtype=torch.int32, device="cuda")
+    differ = 0
+    for i in range(24):
+        n = sizes[(i * 7 + i // 4) % 4]
+        data = rng.integers(0, 256, n, dtype=np.uint8)
+        if i // 3 % 2:
+            data[rng.random(n) < 0.8] = 31
+        where = plain if i % 5 == 2 else pinned
+        where[:n] = data
+        st.push_host(where.ctypes.data, n, out.data_ptr())
+        rec = ref.push(data)
+        single.push(data)
+        s = st.state()  # (the stream has passed the push)
+        differ += ref.flag != single.flag
+        assert np.array_equal(u32(out), rec.hist), i
+        assert s.flag == ref.flag and s.last_kernel == rec.kernel and s.status == 0, i
+        assert np.array_equal(st.window().cpu().numpy().view(np.uint64), ref.mw), i
+    assert (differ > 0) == (window > 1)
+    st.close()
+
+
 @pytest.mark.parametrize("overlap", [False, True])
 @pytest.mark.parametrize("mode", [hl.MODE_AUTO, hl.MODE_ADAPTIVE])
 def test_early_pushes_after_captured_and_replayed_ones(mode, overlap):
