@@ -878,7 +878,8 @@ extern "C" {
 void hist_batch_tuning_init(hist_batch_tuning* t) {
   if (!t) return;
   memset(t, 0, sizeof(*t));
-  // the setting the autotuner picks on GB300 for every batch measured
+  // the lane-private layout for every image (its launches have a shape of
+  // their own; this one is the other layouts')
   t->ctas_per_sm = 2;
   t->unroll = 2;
   t->small_bytes = 0;
@@ -975,7 +976,9 @@ int hist_batch_autotune(const uint8_t* const* d_ptrs, const size_t* d_sizes, uin
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
-  // candidates: CTAs per SM, loads in flight, and the sub-bins of small images
+  // candidates: the sub-bins of small images, and CTAs per SM and loads in
+  // flight where they shape the launch (the lane-private launches are the same
+  // for all: timed once, with the default's)
   std::vector<hist_batch_tuning> cands;
   const uint32_t smalls[][2] = {{0, 5}, {1u << 16, 2}, {1u << 16, 3}, {1u << 18, 3}, {1u << 20, 4}};
   for (uint32_t cps = 1; cps <= 2; ++cps)
@@ -984,10 +987,12 @@ int hist_batch_autotune(const uint8_t* const* d_ptrs, const size_t* d_sizes, uin
         if (cps == 2 && un == 4) continue;
         hist_batch_tuning t;
         hist_batch_tuning_init(&t);
+        const bool shape = cps != t.ctas_per_sm || un != t.unroll;
         t.ctas_per_sm = cps;
         t.unroll = un;
         t.small_bytes = sm[0];
         t.small_log2k = sm[1];
+        if (shape && lane_layouts(layouts_of(t))) continue;
         cands.push_back(t);
       }
   float bms = 1e30f;
@@ -1144,13 +1149,16 @@ extern "C" int hist_batch_autotune_regimes(const uint8_t* const* d_ptrs, const s
     cudaFree(dz);
     cudaFree(dout);
   }
-  // the launch shape of the whole batch with the chosen settings
+  // the launch shape of the whole batch with the chosen settings (the
+  // lane-private launches have one: the default's is kept)
   const uint32_t shapes[][2] = {{2, 2}, {1, 2}, {1, 4}};
+  const bool one_shape = lane_layouts(layouts_of(tb));
   float bms = 1e30f;
   hist_batch_table chosen = tb;
   for (const auto& sh : shapes) {
     if (rc) break;
     hist_batch_table t = tb;
+    if (one_shape && (sh[0] != tb.ctas_per_sm || sh[1] != tb.unroll)) continue;
     t.ctas_per_sm = sh[0];
     t.unroll = sh[1];
     const float ms = time_runs([&]() { return batch_regimes(d_ptrs, d_sizes, count, d_out, d_regime, t, s); }, s, e0,

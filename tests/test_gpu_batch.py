@@ -127,6 +127,33 @@ def test_batch_autotune_returns_a_valid_setting():
         assert np.array_equal(got[i], _oracle(images[i])), i
 
 
+def test_autotuners_keep_the_shape_that_a_layout_ignores():
+    """ctas_per_sm and unroll shape no launch of the lane-private layout: where
+    an autotuner picks that layout for every image it returns the default's,
+    not the one that noise favours."""
+    images = workloads.batch_images(count=400, side_lo=16, side_hi=200)
+    buf = _fill(images, workloads.packed_bytes(images))
+    ptrs, sizes = _arrays(buf, images)
+    out = torch.empty((len(images), 256), dtype=torch.int32, device="cuda")
+    reg = torch.empty(len(images), dtype=torch.uint8, device="cuda")
+    lane = 0
+    for _ in range(8):
+        t = _abi.BatchTuning()
+        assert hl.lib().hist_batch_autotune(ptrs.data_ptr(), sizes.data_ptr(), len(images), out.data_ptr(), 1,
+                                            ctypes.byref(t), None) == 0
+        if t.small_bytes == 0:
+            lane += 1
+            assert (t.ctas_per_sm, t.unroll) == (2, 2)
+        b = _abi.BatchTable()
+        hl.lib().hist_batch_table_init(ctypes.byref(b))
+        assert hl.lib().hist_batch_autotune_regimes(ptrs.data_ptr(), sizes.data_ptr(), len(images), out.data_ptr(),
+                                                    reg.data_ptr(), 1, ctypes.byref(b), None) == 0
+        if all(r.layout == 5 and r.small_bytes == 0 for r in b.regime):
+            lane += 1
+            assert (b.ctas_per_sm, b.unroll) == (2, 2)
+    assert lane > 0
+
+
 def _oracle_all(buf, images, threads=None):
     """The oracle's histogram of every image, counted from the workload's own
     bytes (the generator's output in `buf`, copied back in slabs of about
