@@ -39,14 +39,10 @@ enum Path : int { PATH_PLAIN = 0, PATH_SHIFT = 1, PATH_LUT = 2 };
 
 // Static shared state of a CTA (besides the dynamic table + LUT).
 struct CtaShared {
-  hist_pattern pat;          // pattern this CTA counts with
-  uint32_t hist[HIST_BINS];  // a histogram being reduced (epilogues)
-  uint32_t res[HIST_BINS];   // this CTA's partial result
-  unsigned long long red[kWarps];
+  hist_pattern pat;         // pattern this CTA counts with
+  uint32_t res[HIST_BINS];  // this CTA's partial result
   int path;
   int lk;
-  uint32_t flag;
-  uint32_t kernel;
 };
 
 __device__ __forceinline__ uint4 ldg_stream(const uint4* p) {
