@@ -377,29 +377,36 @@ __device__ __forceinline__ void flat_prev_done(const PushHead& a) {
 }
 
 // Thread 0, before its CTA first adds into a ring slot.  A launch that waited at
-// its start has its slots.  For an early one launches_done says that it has
-// them, or, where that number is too old -- a replayed graph sets it back to
-// what it was when its pushes were captured, and captured pushes advance the
-// launches' numbers without running -- the wait for the launch before does; a
-// captured launch always waits, since the replay before leaves the number ahead
-// of it.  Only hist_stream_test_hold_ring holds the slots for longer (a
-// bounded wait).  (1 GiB overlapping: 152.3 us a push, 153.5 if every early
-// launch waits.)
+// its start has its slots.  An early one has them when launches_done says so,
+// which in a queue of small pinned chunks it does some microseconds later; but
+// that number may be too old -- a replayed graph sets it back to what it was
+// when its pushes were captured, and captured pushes advance the launches'
+// numbers without running -- so after kRingPolls polls the launch waits for the
+// one before it instead, as a captured launch does at once (the replay before
+// leaves the number ahead of it).  Only hist_stream_test_hold_ring holds the
+// slots for longer (a bounded wait).  1 GiB overlapping 152.2 us a push, 153.5
+// if every early launch waits; 64 x 1 MiB from pinned memory 413 us, 643 if a
+// launch waits where the number is not there at once.
+constexpr uint32_t kRingPolls = 64;  // about 60 us
 template <class A>
 __device__ __noinline__ void flat_ring_ready(const A& a, FlatShared<A::kCap>& fs) {
   constexpr unsigned long long back = kChunkRing / kMaxBatch - 1;
   asm volatile("cp.async.wait_all;" ::: "memory");
   if (!a.early && fs.ring_seen[0] + back >= a.launch) return;
-  if (a.early) {
-    if (a.early != kReplayed && ld_acquire(&a.st->h.launches_done) + back >= a.launch) return;
+  uint32_t it = a.early == kReplayed ? kRingPolls : 0;
+  if (a.early && it == 0)
+    while (it < kRingPolls && ld_acquire(&a.st->h.launches_done) + back < a.launch) {
+      __nanosleep(256);
+      ++it;
+    }
+  if (it == kRingPolls) {
     pdl_wait();
     if (!fs.released) {
       fs.released = 1;
       flat_prev_done(a);
     }
   }
-  uint32_t it = 0;
-  while (a.launch > back && ld_acquire(&a.st->h.launches_done) < a.launch - back) {
+  while (ld_acquire(&a.st->h.launches_done) + back < a.launch) {
     if (++it >= kPollLimit) {
       atomicOr(&a.st->h.status, kStatusTimeout);
       break;
