@@ -311,9 +311,8 @@ typedef struct hist_stream_state {
   uint32_t status;            /* 0, or device-side error bits: 4 = a bounded wait
                                    ran out */
   uint32_t recounted;         /* AUTO streams: chunks whose kernel a sample of the
-                                   chunk before would have chosen wrongly (counted a
-                                   second time while the kernels had tables of their
-                                   own) */
+                                   chunk before would have chosen wrongly (a
+                                   statistic: no chunk is counted twice) */
   uint32_t reserved[6];
 } hist_stream_state;
 

@@ -1,13 +1,15 @@
 // hist_batch.cu -- many histograms in one launch (Sec. III.B: small slices or
 // packets batched into one call that returns many histograms).
 //
-// One kernel takes up to kBatchMaxImages images.  Each CTA computes the
-// images' size prefix in shared memory, then counts a contiguous range of the
-// concatenated bytes, an equal share of the batch's cost (the bytes plus a
-// fixed cost per image): the part of each image that falls in its range is
-// counted into the CTA's table and added into that image's output at the
-// image boundary.  The kernel needs no scratch memory, so a batch is a memset
-// of the outputs plus one kernel, and captures into a CUDA graph as such.
+// Two ways, for up to kBatchMaxImages images a launch.  With every image in the
+// lane-private layout (the default), two chained launches (batch_few_kernel or
+// batch_lane_kernel<true>, then batch_lane_kernel<false>): small images whole,
+// by warps and groups of warps, the others in pieces.  With other layouts a
+// memset of the outputs and batch_images_kernel, whose CTAs each count a
+// contiguous range of the concatenated bytes, an equal share of the batch's
+// cost (the bytes plus a fixed cost per image), and add what falls in it into
+// the images' outputs at the image boundaries.  Neither needs scratch memory,
+// so a batch captures into a CUDA graph as it is.
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <stdlib.h>

@@ -3,8 +3,8 @@
 //
 // Shared-memory histogram layouts (Sec. III.A).  Every call but the ablation
 // and a batch with layouts of the caller's choice counts in the lane-private
-// table, whatever the kernel or the pattern (the pattern is still derived and
-// kept): each lane owns one bank -- pixel v of lane l is word 32 v + l -- so a
+// table (a batch's images of at most 4 KiB: in 256 words per warp), whatever
+// the kernel or the pattern (the pattern is still derived and kept): each lane owns one bank -- pixel v of lane l is word 32 v + l -- so a
 // warp's 32 increments never meet in a bank whatever the pixel values, and any
 // pattern's counts are its per-bin sums.  64 MiB of uniform pixels: 13 us, 31
 // with a table per warp; at the paper's 960 slots 200 MB of N(128, 8) take 34

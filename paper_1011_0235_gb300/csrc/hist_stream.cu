@@ -418,9 +418,15 @@ __device__ __noinline__ void flat_ring_ready(const A& a, FlatShared<A::kCap>& fs
 // A launch that reads over the host link lets the next one start only when
 // CTA 0 has half of its piece, and at most 64 KiB, left: the next chunk's
 // first reads come before this one's last, and however many chunks are queued
-// two or three launches of kHostGrid CTAs hold SMs while they wait for the
-// link (else all of them would: eight one-shots of 64 MiB on another stream
-// beside 16 x 16 MiB take 1145 us, so 264; 402 when the chunks were copied).
+// two launches of kHostGrid CTAs hold SMs while they wait for the link (if all
+// did, eight one-shots of 64 MiB on another stream beside 16 x 16 MiB would
+// take 1145 us; so 251, alone 117).  With chunks of 512 KiB and 1 MiB, whose
+// epilogues take longer than their bytes over the link, up to five launches
+// (80 CTAs) are resident.  The launches of one CTA (push_one_kernel) let the
+// next one start at once: seven to nine of them are resident at most, whether
+// the link is busy with other copies or not, and the same eight one-shots take
+// 183 us beside 400 chunks of 64 KiB (1.12 ms).  Let in after the loads they
+// would take 143, but the chunks 1.59 ms, those of 128 KiB 2.13 for 1.23.
 template <class A>
 __device__ __forceinline__ bool host_late(const A& a) {
   return a.early == kHostChunk && blockIdx.x == 0;
@@ -788,9 +794,9 @@ __device__ __forceinline__ void flat_groups(const A& a, uint32_t nwl, int first,
 // before the other and the SM then runs a single CTA at half its loads in
 // flight; one CTA per SM has no such pair.  Bound by the HBM read on large
 // chunks, by a chain of round trips to L2 on one small one: on the GPU,
-// pushes in a row, 64 x 16 MiB 166.6 -> 158.7 us (6.8 TB/s; overlapping
-// 162 -> 155.7 us), 128 x 1 MiB 39.2 -> 28.1 us, one chunk of 1 MiB
-// 15.6 -> 7.6 us.
+// pushes in a row, 64 x 16 MiB 166.6 -> 158.4 us (6.8 TB/s; overlapping
+// 162 -> 155.6 us from a graph, 152.2 called one by one), 128 x 1 MiB 39.2 ->
+// 28.0 us (AUTO 28.9), one chunk of 1 MiB 15.6 -> 7.5 us.
 template <class A>
 __global__ void __launch_bounds__(kThreads, 1) batch_flat_kernel(const __grid_constant__ A a) {
   extern __shared__ __align__(16) uint32_t tables[];
@@ -1615,11 +1621,10 @@ int hist_stream_push_host(hist_stream* st, const uint8_t* h_chunk, size_t n, uin
   if (!st->depth) return HIST_ESTATE;
   if (n > st->max_chunk) return HIST_EINVAL;
   // Pinned memory is counted in place, a chunk's reads beside the launch
-  // before it, as with HIST_OVERLAP_PUSHES (the caller's bytes were complete
-  // before too: the copies waited for no work of his).  Copied into staging,
-  // with the events between copy and count, and now: 64 x 64 KiB 729 -> 199
-  // us, 64 x 1 MiB 860 -> 410, 16 x 4 MiB 404 -> 342, 16 x 16 MiB 1335 -> 1296
-  // (1272 at the link's rate).
+  // before it, as with HIST_OVERLAP_PUSHES (the caller's bytes are complete by
+  // contract).  Copied into staging, with the events between copy and count,
+  // and so: 64 x 64 KiB 729 and 195 us, 64 x 1 MiB 860 and 413, 16 x 4 MiB 404
+  // and 344; 16 x 16 MiB take the link's time both ways (1310 and 1271 in a row).
   if (const uint8_t* d = n ? host_readable(h_chunk, n, (cudaStream_t)s) : nullptr)
     return push_chunks(st, 1, &d, &n, d_chunk_out ? &d_chunk_out : nullptr, (cudaStream_t)s, true);
   const uint32_t b = (uint32_t)(st->host_pushes % st->depth);
