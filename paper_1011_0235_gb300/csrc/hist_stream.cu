@@ -393,13 +393,12 @@ __device__ __noinline__ void flat_ring_ready(const A& a, FlatShared<A::kCap>& fs
   constexpr unsigned long long back = kChunkRing / kMaxBatch - 1;
   asm volatile("cp.async.wait_all;" ::: "memory");
   if (!a.early && fs.ring_seen[0] + back >= a.launch) return;
-  uint32_t it = a.early == kReplayed ? kRingPolls : 0;
-  if (a.early && it == 0)
-    while (it < kRingPolls && ld_acquire(&a.st->h.launches_done) + back < a.launch) {
+  uint32_t it = 0;
+  if (a.early) {
+    for (; a.early != kReplayed && it < kRingPolls; ++it) {
+      if (ld_acquire(&a.st->h.launches_done) + back >= a.launch) return;
       __nanosleep(256);
-      ++it;
     }
-  if (it == kRingPolls) {
     pdl_wait();
     if (!fs.released) {
       fs.released = 1;
