@@ -384,8 +384,8 @@ __device__ __forceinline__ void flat_prev_done(const PushHead& a) {
 // numbers without running -- so after kRingPolls polls the launch waits for the
 // one before it instead, as a captured launch does at once (the replay before
 // leaves the number ahead of it).  Only hist_stream_test_hold_ring holds the
-// slots for longer (a bounded wait).  1 GiB overlapping 152.2 us a push, 153.5
-// if every early launch waits; 64 x 1 MiB from pinned memory 413 us, 643 if a
+// slots for longer (a bounded wait).  1 GiB overlapping 152.0 us a push, 153.5
+// if every early launch waits; 64 x 1 MiB from pinned memory 403 us, 643 if a
 // launch waits where the number is not there at once.
 constexpr uint32_t kRingPolls = 64;  // about 60 us
 template <class A>
@@ -794,7 +794,7 @@ __device__ __forceinline__ void flat_groups(const A& a, uint32_t nwl, int first,
 // flight; one CTA per SM has no such pair.  Bound by the HBM read on large
 // chunks, by a chain of round trips to L2 on one small one: on the GPU,
 // pushes in a row, 64 x 16 MiB 166.6 -> 158.4 us (6.8 TB/s; overlapping
-// 162 -> 155.6 us from a graph, 152.2 called one by one), 128 x 1 MiB 39.2 ->
+// 162 -> 155.6 us from a graph, 152.0 called one by one), 128 x 1 MiB 39.2 ->
 // 28.0 us (AUTO 28.9), one chunk of 1 MiB 15.6 -> 7.5 us.
 template <class A>
 __global__ void __launch_bounds__(kThreads, 1) batch_flat_kernel(const __grid_constant__ A a) {
@@ -1622,8 +1622,8 @@ int hist_stream_push_host(hist_stream* st, const uint8_t* h_chunk, size_t n, uin
   // Pinned memory is counted in place, a chunk's reads beside the launch
   // before it, as with HIST_OVERLAP_PUSHES (the caller's bytes are complete by
   // contract).  Copied into staging, with the events between copy and count,
-  // and so: 64 x 64 KiB 729 and 195 us, 64 x 1 MiB 860 and 413, 16 x 4 MiB 404
-  // and 344; 16 x 16 MiB take the link's time both ways (1310 and 1271 in a row).
+  // and so: 64 x 64 KiB 729 and 195 us, 64 x 1 MiB 860 and 403, 16 x 4 MiB 404
+  // and 347; 16 x 16 MiB take the link's time both ways (1310 and 1271 in a row).
   if (const uint8_t* d = n ? host_readable(h_chunk, n, (cudaStream_t)s) : nullptr)
     return push_chunks(st, 1, &d, &n, d_chunk_out ? &d_chunk_out : nullptr, (cudaStream_t)s, true);
   const uint32_t b = (uint32_t)(st->host_pushes % st->depth);
